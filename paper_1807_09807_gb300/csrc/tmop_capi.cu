@@ -148,6 +148,81 @@ void lagrange_bary(int n, const double* z, double s, double* phi, double* dphi) 
   }
 }
 
+// Fixed-point tables of the FP64 contractions (tmop_fixed.cuh) from the 1D
+// tables B[q][i], G[q][i] of a rule and a node set symmetric about 1/2:
+// B[Q-1-q][N-1-i] = B[q][i] and G[Q-1-q][N-1-i] = -G[q][i] up to rounding,
+// of which the mean is taken. The input widths xin and rin keep every value
+// that is split into limbs below 2^60 and every result below 2^62, from the
+// largest row and column sums of |B| and |G|; then the sums M of limb
+// products (at most 3 terms forward, q in the adjoint) stay below 2^63, which
+// is checked too. False if the tables do not fit.
+bool fx_tables(int dim, int n, int q, const double* B, const double* G, FxTab* T) {
+  memset(T, 0, sizeof(*T));
+  const int nh = n / 2, ne = (n + 1) / 2, qh = q / 2, qe = (q + 1) / 2;
+  if (ne > 3 || qe > 4) return false;
+  double gmax = 0.0;
+  for (int t = 0; t < n * q; ++t) gmax = fmax(gmax, fabs(G[t]));
+  if (!(gmax > 0.0) || !isfinite(gmax)) return false;
+  int g = 0;
+  frexp(gmax, &g);   // gmax < 2^g
+  T->gexp = g;
+  auto put = [](double c, int* H, int* L) {
+    const long long v = llround(ldexp(c, 60));
+    const long long lo = ((v + (1LL << 29)) & ((1LL << 30) - 1)) - (1LL << 29);
+    *L = (int)lo;
+    *H = (int)((v - lo) >> 30);
+  };
+  double msum = 0.0;   // largest sum of |entries| that multiply one line's values in the adjoint map
+  for (int a = 0; a < qe; ++a)
+    for (int i = 0; i < ne; ++i) {
+      const int aa = q - 1 - a, ii = n - 1 - i, k = 3 * a + i;
+      const double b0 = 0.5 * (B[a * n + i] + B[aa * n + ii]), b1 = 0.5 * (B[a * n + ii] + B[aa * n + i]);
+      const double g0 = 0.5 * (G[a * n + i] - G[aa * n + ii]), g1 = 0.5 * (G[a * n + ii] - G[aa * n + i]);
+      const bool mid = i >= nh;   // the centre node is its own mirror image
+      put(mid ? b0 : 0.5 * (b0 + b1), &T->BeH[k], &T->BeL[k]);
+      if (!mid && a < qh) put(0.5 * (b0 - b1), &T->BoH[k], &T->BoL[k]);
+      if (a < qh) put(ldexp(mid ? g0 : 0.5 * (g0 + g1), -g), &T->GeH[k], &T->GeL[k]);
+      if (!mid) put(ldexp(0.5 * (g0 - g1), -g), &T->GoH[k], &T->GoL[k]);
+    }
+  for (int i = 0; i < ne; ++i) {
+    double e = 0.0, o = 0.0;
+    for (int a = 0; a < qe; ++a) {
+      e += fabs((double)T->BeH[3 * a + i]) + fabs((double)T->GeH[3 * a + i]);
+      o += fabs((double)T->BoH[3 * a + i]) + fabs((double)T->GoH[3 * a + i]);
+    }
+    msum = fmax(msum, ldexp(fmax(e, o), -30));
+  }
+  double br = 0.0, gr = 0.0, bc = 0.0, gc = 0.0;   // row (points) and column (nodes) sums
+  for (int a = 0; a < q; ++a) {
+    double sb = 0.0, sg = 0.0;
+    for (int i = 0; i < n; ++i) { sb += fabs(B[a * n + i]); sg += fabs(ldexp(G[a * n + i], -g)); }
+    br = fmax(br, sb);
+    gr = fmax(gr, sg);
+  }
+  for (int i = 0; i < n; ++i) {
+    double sb = 0.0, sg = 0.0;
+    for (int a = 0; a < q; ++a) { sb += fabs(B[a * n + i]); sg += fabs(ldexp(G[a * n + i], -g)); }
+    bc = fmax(bc, sb);
+    gc = fmax(gc, sg);
+  }
+  br = fmax(br, 1.0);
+  bc = fmax(bc, 1.0);
+  gr = fmax(gr, 1.0);
+  gc = fmax(gc, 1.0);
+  // largest values that enter a map's last stage as pair sums, and results,
+  // per unit of input: forward one B or G per stage; the adjoint adds two maps
+  // from its second stage on
+  const double fin = dim == 2 ? fmax(br, gr) : br * fmax(br, gr);
+  const double fout = dim == 2 ? br * gr : br * br * gr;
+  const double rmid = dim == 2 ? fmax(bc, gc) : fmax(2.0 * bc * gc, bc * bc);
+  const double rout = dim == 2 ? 2.0 * bc * gc : 3.0 * bc * bc * gc;
+  T->xin = 59 - (int)ceil(log2(fin) + 1e-9);
+  T->rin = 59 - (int)ceil(log2(rmid) + 1e-9);
+  // M: |sum| <= 2^60 sum|c| + terms 2^59 < 2^63
+  return T->xin >= 54 && T->rin >= 54 && ldexp(fout, T->xin) < 0x1p62 && ldexp(rout, T->rin) < 0x1p62 &&
+         fmax(br, gr) + 1.5 < 7.9 && msum + 0.5 * q < 7.9;
+}
+
 static double det_h(int d, const double* M) {
   if (d == 2) return M[0] * M[3] - M[1] * M[2];
   return M[0] * (M[4] * M[8] - M[5] * M[7]) - M[1] * (M[3] * M[8] - M[5] * M[6]) +
@@ -888,6 +963,10 @@ int tmop_setup(const tmop_mesh* mesh, int order, const tmop_quad* quad, int metr
       p.G[a * n + i] = dphi[i];
     }
     p.w1[a] = qw[a];
+  }
+  if (!fx_tables(d, n, nq, p.B, p.G, &p.fx)) {
+    tmop_destroy(c);
+    return TMOP_ERR_ARG;
   }
 
   // targets

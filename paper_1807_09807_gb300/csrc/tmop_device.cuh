@@ -561,637 +561,6 @@ __device__ __forceinline__ void adj2(const R* __restrict__ B, const R* __restric
   __syncwarp();
 }
 
-// 3D forward. P0: X[NC][N][N][N] -> P1: S1[NC][2][N][N][Q] -> P0: S2[NC][3][N][Q][Q]
-// -> P1: A[NC][3][Q][Q][Q]
-template <int N, int Q1, int NC, class R>
-__device__ __forceinline__ void fwd3(const R* __restrict__ B, const R* __restrict__ G, R* P0, R* P1, int lane) {
-  constexpr int NNQ = N * N * Q1, NQQ = N * Q1 * Q1, QQ = Q1 * Q1, QQQ = Q1 * Q1 * Q1;
-  for (int t = lane; t < NC * N * N * Q1; t += 32) {
-    const int q0 = t % Q1, lj = (t / Q1) % (N * N), c = t / (Q1 * N * N);
-    const R* xr = P0 + (c * N * N + lj) * N;
-    R sb = R(0), sg = R(0);
-#pragma unroll
-    for (int i = 0; i < N; ++i) {
-      const R xv = xr[i];
-      sb = fma(xv, B[q0 * N + i], sb);
-      sg = fma(xv, G[q0 * N + i], sg);
-    }
-    P1[(c * 2 + 0) * NNQ + lj * Q1 + q0] = sb;
-    P1[(c * 2 + 1) * NNQ + lj * Q1 + q0] = sg;
-  }
-  __syncwarp();
-  for (int t = lane; t < NC * N * QQ; t += 32) {
-    const int q0 = t % Q1, q1 = (t / Q1) % Q1, l = (t / QQ) % N, c = t / (QQ * N);
-    const R* xb = P1 + (c * 2 + 0) * NNQ + l * N * Q1 + q0;
-    const R* xg = P1 + (c * 2 + 1) * NNQ + l * N * Q1 + q0;
-    R bb = R(0), bg = R(0), gb = R(0);
-#pragma unroll
-    for (int j = 0; j < N; ++j) {
-      const R b = xb[j * Q1], g = xg[j * Q1];
-      bb = fma(b, B[q1 * N + j], bb);
-      bg = fma(b, G[q1 * N + j], bg);
-      gb = fma(g, B[q1 * N + j], gb);
-    }
-    const int o = l * QQ + q1 * Q1 + q0;
-    P0[(c * 3 + 0) * NQQ + o] = bb;
-    P0[(c * 3 + 1) * NQQ + o] = bg;
-    P0[(c * 3 + 2) * NQQ + o] = gb;
-  }
-  __syncwarp();
-  for (int t = lane; t < NC * QQQ; t += 32) {
-    const int q01 = t % QQ, q2 = (t / QQ) % Q1, c = t / QQQ;
-    const R* sbb = P0 + (c * 3 + 0) * NQQ + q01;
-    const R* sbg = P0 + (c * 3 + 1) * NQQ + q01;
-    const R* sgb = P0 + (c * 3 + 2) * NQQ + q01;
-    R a0 = R(0), a1 = R(0), a2 = R(0);
-#pragma unroll
-    for (int l = 0; l < N; ++l) {
-      const R bl = B[q2 * N + l], gl = G[q2 * N + l];
-      a0 = fma(sgb[l * QQ], bl, a0);
-      a1 = fma(sbg[l * QQ], bl, a1);
-      a2 = fma(sbb[l * QQ], gl, a2);
-    }
-    const int o = q2 * QQ + q01;
-    P1[(c * 3 + 0) * QQQ + o] = a0;
-    P1[(c * 3 + 1) * QQQ + o] = a1;
-    P1[(c * 3 + 2) * QQQ + o] = a2;
-  }
-  __syncwarp();
-}
-
-// 3D adjoint. P1: R[NC][3][Q][Q][Q] -> P0: U[NC][3][N][Q][Q] -> P1: V[NC][2][N][N][Q]
-// -> P0: Y[NC][N][N][N]
-template <int N, int Q1, int NC, class R>
-__device__ __forceinline__ void adj3(const R* __restrict__ B, const R* __restrict__ G, R* P0, R* P1, int lane) {
-  constexpr int NNQ = N * N * Q1, NQQ = N * Q1 * Q1, QQ = Q1 * Q1, QQQ = Q1 * Q1 * Q1;
-  for (int t = lane; t < NC * N * QQ; t += 32) {
-    const int q01 = t % QQ, l = (t / QQ) % N, c = t / (QQ * N);
-    const R* r0 = P1 + (c * 3 + 0) * QQQ + q01;
-    const R* r1 = P1 + (c * 3 + 1) * QQQ + q01;
-    const R* r2 = P1 + (c * 3 + 2) * QQQ + q01;
-    R u0 = R(0), u1 = R(0), u2 = R(0);
-#pragma unroll
-    for (int q2 = 0; q2 < Q1; ++q2) {
-      const R bl = B[q2 * N + l], gl = G[q2 * N + l];
-      u0 = fma(r0[q2 * QQ], bl, u0);
-      u1 = fma(r1[q2 * QQ], bl, u1);
-      u2 = fma(r2[q2 * QQ], gl, u2);
-    }
-    const int o = l * QQ + q01;
-    P0[(c * 3 + 0) * NQQ + o] = u0;
-    P0[(c * 3 + 1) * NQQ + o] = u1;
-    P0[(c * 3 + 2) * NQQ + o] = u2;
-  }
-  __syncwarp();
-  for (int t = lane; t < NC * N * N * Q1; t += 32) {
-    const int q0 = t % Q1, j = (t / Q1) % N, l = (t / (Q1 * N)) % N, c = t / (Q1 * N * N);
-    const R* u0 = P0 + (c * 3 + 0) * NQQ + l * QQ + q0;
-    const R* u1 = P0 + (c * 3 + 1) * NQQ + l * QQ + q0;
-    const R* u2 = P0 + (c * 3 + 2) * NQQ + l * QQ + q0;
-    R vg = R(0), vb = R(0);
-#pragma unroll
-    for (int q1 = 0; q1 < Q1; ++q1) {
-      const R bj = B[q1 * N + j], gj = G[q1 * N + j];
-      vg = fma(u0[q1 * Q1], bj, vg);
-      vb = fma(u1[q1 * Q1], gj, fma(u2[q1 * Q1], bj, vb));
-    }
-    const int o = (l * N + j) * Q1 + q0;
-    P1[(c * 2 + 0) * NNQ + o] = vg;  // pairs with G in x
-    P1[(c * 2 + 1) * NNQ + o] = vb;  // pairs with B in x
-  }
-  __syncwarp();
-  for (int t = lane; t < NC * N * N * N; t += 32) {
-    const int i = t % N, lj = (t / N) % (N * N), c = t / (N * N * N);
-    const R* vg = P1 + (c * 2 + 0) * NNQ + lj * Q1;
-    const R* vb = P1 + (c * 2 + 1) * NNQ + lj * Q1;
-    R y = R(0);
-#pragma unroll
-    for (int q0 = 0; q0 < Q1; ++q0) y = fma(vg[q0], G[q0 * N + i], fma(vb[q0], B[q0 * N + i], y));
-    P0[(c * N * N + lj) * N + i] = y;
-  }
-  __syncwarp();
-}
-
-// ---------------------------------------------------------------- folded (even-odd) 3D contractions
-// The Gauss points and the Gauss-Lobatto nodes are symmetric about the
-// element centre, so B[Q-1-q][N-1-i] = B[q][i] and G[Q-1-q][N-1-i] =
-// -G[q][i]. In the mirror basis of each direction -- the butterfly F,
-// (v_i, v_{L-1-i}) -> (v_i + v_{L-1-i}, v_i - v_{L-1-i}) stored in place at
-// (i, L-1-i), the middle entry of an odd length kept -- symmetric vectors
-// live on the "even" positions p < ceil(L/2) and antisymmetric ones on the
-// "odd" positions, and B maps each class to itself while G swaps them. The
-// folded tables Bf = S_Q^-1 F_Q B F_N S_N^-1 and Gf alike (S = F F: 2 on
-// pair positions, 1 in the middle) are therefore block-sparse: an output
-// position needs only the inputs of one parity, half the multiply-adds of
-// the plain 1D contraction. Since F S^-1 F = I and F, S are symmetric, the
-// 3D maps become
-//   forward  A = F_Q^3 (Bf/Gf contractions) F_N^3 x
-//   adjoint  y = F_N^3 (Bf^T/Gf^T contractions) F_Q^3 R
-// with butterfly passes in place around the stage loops. For order-3 hexes
-// (N = 4, Q = 5) a forward or adjoint map takes 5 010 multiply-adds and
-// 3 276 butterfly operations per element where the plain one takes 10 020
-// multiply-adds. Written for an even N (every output then reads N/2 inputs
-// of its parity, and the adjoint stages pair the outputs (l, N-1-l)).
-
-// Entry (p, q) of the mirror butterfly of length L (symmetric).
-__device__ __forceinline__ double mirror_entry(int L, int p, int q) {
-  const int m = L - 1 - p;
-  if (p == m) return q == p ? 1.0 : 0.0;
-  if (q == p) return p < m ? 1.0 : -1.0;
-  return q == m ? 1.0 : 0.0;
-}
-
-// Bf and Gf [Q1][N] from the physical tables B, G [Q1][N] (row-major),
-// computed by threads tid, tid + nth, ... of the block.
-template <int N, int Q1, class R>
-__device__ void folded_tables(const double* B, const double* G, R* Bf, R* Gf, int tid, int nth) {
-  for (int t = tid; t < Q1 * N; t += nth) {
-    const int p = t / N, r = t % N;
-    double b = 0.0, g = 0.0;
-    for (int q = 0; q < Q1; ++q) {
-      const double fq = mirror_entry(Q1, p, q);
-      if (fq == 0.0) continue;
-      for (int i = 0; i < N; ++i) {
-        const double fi = mirror_entry(N, i, r);
-        if (fi == 0.0) continue;
-        b = fma(fq * fi, B[q * N + i], b);
-        g = fma(fq * fi, G[q * N + i], g);
-      }
-    }
-    const double sp = (2 * p == Q1 - 1) ? 1.0 : 0.5, sr = (2 * r == N - 1) ? 1.0 : 0.5;
-    Bf[t] = R(b * sp * sr);
-    Gf[t] = R(g * sp * sr);
-  }
-}
-
-// In-place butterfly along axis AX (0 fastest) of NF consecutive fields,
-// each an [L2][L1][L0] array.
-template <int NF, int L0, int L1, int L2, int AX, class R>
-__device__ __forceinline__ void mirror3(R* buf, int lane) {
-  constexpr int L = AX == 0 ? L0 : (AX == 1 ? L1 : L2);
-  constexpr int H = L / 2, FS = L0 * L1 * L2, LINES = FS / L;
-  constexpr int ST = AX == 0 ? 1 : (AX == 1 ? L0 : L0 * L1);
-#pragma unroll 1
-  for (int t = lane; t < NF * LINES * H; t += 32) {
-    const int i = t % H, line = (t / H) % LINES, f = t / (H * LINES);
-    int base;
-    if constexpr (AX == 0) base = line * L0;
-    else if constexpr (AX == 1) base = (line / L0) * (L0 * L1) + line % L0;
-    else base = line;
-    R* v = buf + f * FS + base;
-    const R a = v[i * ST], b = v[(L - 1 - i) * ST];
-    v[i * ST] = a + b;
-    v[(L - 1 - i) * ST] = a - b;
-  }
-  __syncwarp();
-}
-
-// The butterfly along all three axes.
-template <int NF, int L, class R>
-__device__ __forceinline__ void mirror3_all(R* buf, int lane) {
-  mirror3<NF, L, L, L, 0, R>(buf, lane);
-  mirror3<NF, L, L, L, 1, R>(buf, lane);
-  mirror3<NF, L, L, L, 2, R>(buf, lane);
-}
-
-// Normalised forward: every folded dot of the forward map has N/2 terms of
-// one parity; scaling it by its larger coefficient (the pivot) leaves
-// x[k] + r x[k^1] (N = 4: one multiply-add instead of a multiply and a
-// multiply-add) or the plain copy x[k] (N = 2). For table t (0 = B, 1 = G)
-// and output position p, entry t * Q1 + p of kf is the pivot's input
-// position and of rt the other coefficient over the pivot (0 for a zero
-// pivot, whose outputs the scale then zeroes). The stage outputs are the
-// true ones divided by the pivots along the axes done so far, so the point
-// fields come out divided by Sc[d][q2][q1][q0], the product of the pivots
-// of direction d's tables (G along axis d, B along the others), which the
-// first unfold pass multiplies back (mirror3_scaled).
-template <int N, int Q1, class R>
-__device__ void normalised_tables(const R* Bf, const R* Gf, int* kf, R* rt, R* piv, R* Sc, int tid, int nth) {
-  static_assert(N == 2 || N == 4, "normalised folded dots are written for N / 2 = 1 or 2 terms");
-  constexpr int H = N / 2, QE = (Q1 + 1) / 2, QQQ = Q1 * Q1 * Q1;
-  for (int t = tid; t < 2 * Q1; t += nth) {
-    const int tb = t / Q1, p = t % Q1;
-    const R* T = (tb ? Gf : Bf) + p * N;
-    const int base = ((p >= QE) != (tb == 1)) ? H : 0;   // B keeps the parity, G swaps it
-    int k = base;
-    R b = T[base];
-    if (H == 2 && fabs(T[base + 1]) > fabs(b)) {
-      k = base + 1;
-      b = T[base + 1];
-    }
-    kf[t] = k;
-    rt[t] = (H == 2 && b != R(0)) ? T[k ^ 1] / b : R(0);
-    piv[t] = b;
-  }
-  __syncthreads();
-  for (int t = tid; t < 3 * QQQ; t += nth) {
-    const int q0 = t % Q1, q1 = (t / Q1) % Q1, q2 = (t / (Q1 * Q1)) % Q1, d = t / QQQ;
-    Sc[t] = piv[(d == 0) * Q1 + q0] * piv[(d == 1) * Q1 + q1] * piv[(d == 2) * Q1 + q2];
-  }
-}
-
-// The folded dot of table entry t over inputs x[0], x[stride], ...
-template <int H, class R>
-__device__ __forceinline__ R norm_dot(const R* x, int stride, const int* __restrict__ kf, const R* __restrict__ rt,
-                                      int t) {
-  const int k = kf[t];
-  if constexpr (H == 2) return fma(x[(k ^ 1) * stride], rt[t], x[k * stride]);
-  else return x[k * stride];
-}
-
-// Forward stages of fwd3_eo with normalised dots; P1 holds the folded A
-// divided by Sc on exit.
-template <int N, int Q1, int NC, class R>
-__device__ __forceinline__ void fwd3_eon(const int* __restrict__ kf, const R* __restrict__ rt, R* P0, R* P1,
-                                         int lane) {
-  constexpr int H = N / 2;
-  constexpr int NNQ = N * N * Q1, NQQ = N * Q1 * Q1, QQ = Q1 * Q1, QQQ = Q1 * Q1 * Q1;
-  for (int t = lane; t < NC * N * N * Q1; t += 32) {            // rows (c, l, j) along i -> q0
-    const int q0 = t % Q1, lj = (t / Q1) % (N * N), c = t / (Q1 * N * N);
-    const R* xr = P0 + (c * N * N + lj) * N;
-    P1[(c * 2 + 0) * NNQ + lj * Q1 + q0] = norm_dot<H>(xr, 1, kf, rt, q0);
-    P1[(c * 2 + 1) * NNQ + lj * Q1 + q0] = norm_dot<H>(xr, 1, kf, rt, Q1 + q0);
-  }
-  __syncwarp();
-  for (int t = lane; t < NC * N * QQ; t += 32) {                // (c, l, q1, q0) along j -> q1
-    const int q0 = t % Q1, q1 = (t / Q1) % Q1, l = (t / QQ) % N, c = t / (QQ * N);
-    const R* xb = P1 + (c * 2 + 0) * NNQ + l * N * Q1 + q0;
-    const R* xg = P1 + (c * 2 + 1) * NNQ + l * N * Q1 + q0;
-    const int o = l * QQ + q1 * Q1 + q0;
-    P0[(c * 3 + 0) * NQQ + o] = norm_dot<H>(xb, Q1, kf, rt, q1);
-    P0[(c * 3 + 1) * NQQ + o] = norm_dot<H>(xb, Q1, kf, rt, Q1 + q1);
-    P0[(c * 3 + 2) * NQQ + o] = norm_dot<H>(xg, Q1, kf, rt, q1);
-  }
-  __syncwarp();
-  for (int t = lane; t < NC * QQQ; t += 32) {                   // (c, q2, q1, q0) along l -> q2
-    const int q01 = t % QQ, q2 = (t / QQ) % Q1, c = t / QQQ;
-    const int o = q2 * QQ + q01;
-    P1[(c * 3 + 0) * QQQ + o] = norm_dot<H>(P0 + (c * 3 + 2) * NQQ + q01, QQ, kf, rt, q2);
-    P1[(c * 3 + 1) * QQQ + o] = norm_dot<H>(P0 + (c * 3 + 1) * NQQ + q01, QQ, kf, rt, q2);
-    P1[(c * 3 + 2) * QQQ + o] = norm_dot<H>(P0 + (c * 3 + 0) * NQQ + q01, QQ, kf, rt, Q1 + q2);
-  }
-  __syncwarp();
-}
-
-// The axis-0 butterfly of fwd3_eon's point fields with Sc multiplied back
-// (field f has direction f % 3; the middle entry of an odd length is scaled
-// by the unit of pair 0).
-template <int NF, int L, class R>
-__device__ __forceinline__ void mirror3_scaled(R* buf, const R* __restrict__ Sc, int lane) {
-  constexpr int H = L / 2, FS = L * L * L, LINES = L * L;
-#pragma unroll 1
-  for (int t = lane; t < NF * LINES * H; t += 32) {
-    const int i = t % H, line = (t / H) % LINES, f = t / (H * LINES);
-    R* v = buf + f * FS + line * L;
-    const R* sc = Sc + (f % 3) * FS + line * L;
-    const R bs = v[L - 1 - i] * sc[L - 1 - i];
-    const R a = v[i], sa = sc[i];
-    v[i] = fma(a, sa, bs);
-    v[L - 1 - i] = fma(a, sa, -bs);
-    if (L % 2 == 1 && i == 0) v[H] *= sc[H];
-  }
-  __syncwarp();
-}
-
-// F_Q^3 of fwd3_eon's output, Sc multiplied back on the way: A at the points.
-template <int NF, int L, class R>
-__device__ __forceinline__ void unfold_points(R* buf, const R* __restrict__ Sc, int lane) {
-  mirror3_scaled<NF, L, R>(buf, Sc, lane);
-  mirror3<NF, L, L, L, 1, R>(buf, lane);
-  mirror3<NF, L, L, L, 2, R>(buf, lane);
-}
-
-
-// Forward stages in the folded basis; same buffer layouts as fwd3. P0 holds
-// F_N^3 x on entry; P1 holds the folded A (F_Q^3 of it is A) on exit.
-template <int N, int Q1, int NC, class R>
-__device__ __forceinline__ void fwd3_eo(const R* __restrict__ Bf, const R* __restrict__ Gf, R* P0, R* P1, int lane) {
-  static_assert(N % 2 == 0, "folded contractions need an even node count");
-  constexpr int H = N / 2, QE = (Q1 + 1) / 2;
-  constexpr int NNQ = N * N * Q1, NQQ = N * Q1 * Q1, QQ = Q1 * Q1, QQQ = Q1 * Q1 * Q1;
-  for (int t = lane; t < NC * N * N * Q1; t += 32) {            // rows (c, l, j) along i -> q0
-    const int q0 = t % Q1, lj = (t / Q1) % (N * N), c = t / (Q1 * N * N);
-    const int ob = q0 < QE ? 0 : H, og = H - ob;                 // inputs of the output's parity (B), the other (G)
-    const R* xr = P0 + (c * N * N + lj) * N;
-    const R* tb = Bf + q0 * N;
-    const R* tg = Gf + q0 * N;
-    R sb = R(0), sg = R(0);
-#pragma unroll
-    for (int k = 0; k < H; ++k) {
-      sb = fma(xr[ob + k], tb[ob + k], sb);
-      sg = fma(xr[og + k], tg[og + k], sg);
-    }
-    P1[(c * 2 + 0) * NNQ + lj * Q1 + q0] = sb;
-    P1[(c * 2 + 1) * NNQ + lj * Q1 + q0] = sg;
-  }
-  __syncwarp();
-  for (int t = lane; t < NC * N * QQ; t += 32) {                // (c, l, q1, q0) along j -> q1
-    const int q0 = t % Q1, q1 = (t / Q1) % Q1, l = (t / QQ) % N, c = t / (QQ * N);
-    const int ob = q1 < QE ? 0 : H, og = H - ob;
-    const R* xb = P1 + (c * 2 + 0) * NNQ + l * N * Q1 + q0;
-    const R* xg = P1 + (c * 2 + 1) * NNQ + l * N * Q1 + q0;
-    const R* tb = Bf + q1 * N;
-    const R* tg = Gf + q1 * N;
-    R bb = R(0), bg = R(0), gb = R(0);
-#pragma unroll
-    for (int k = 0; k < H; ++k) {
-      bb = fma(xb[(ob + k) * Q1], tb[ob + k], bb);
-      bg = fma(xb[(og + k) * Q1], tg[og + k], bg);
-      gb = fma(xg[(ob + k) * Q1], tb[ob + k], gb);
-    }
-    const int o = l * QQ + q1 * Q1 + q0;
-    P0[(c * 3 + 0) * NQQ + o] = bb;
-    P0[(c * 3 + 1) * NQQ + o] = bg;
-    P0[(c * 3 + 2) * NQQ + o] = gb;
-  }
-  __syncwarp();
-  for (int t = lane; t < NC * QQQ; t += 32) {                   // (c, q2, q1, q0) along l -> q2
-    const int q01 = t % QQ, q2 = (t / QQ) % Q1, c = t / QQQ;
-    const int ob = q2 < QE ? 0 : H, og = H - ob;
-    const R* sbb = P0 + (c * 3 + 0) * NQQ + q01;
-    const R* sbg = P0 + (c * 3 + 1) * NQQ + q01;
-    const R* sgb = P0 + (c * 3 + 2) * NQQ + q01;
-    const R* tb = Bf + q2 * N;
-    const R* tg = Gf + q2 * N;
-    R a0 = R(0), a1 = R(0), a2 = R(0);
-#pragma unroll
-    for (int k = 0; k < H; ++k) {
-      a0 = fma(sgb[(ob + k) * QQ], tb[ob + k], a0);
-      a1 = fma(sbg[(ob + k) * QQ], tb[ob + k], a1);
-      a2 = fma(sbb[(og + k) * QQ], tg[og + k], a2);
-    }
-    const int o = q2 * QQ + q01;
-    P1[(c * 3 + 0) * QQQ + o] = a0;
-    P1[(c * 3 + 1) * QQQ + o] = a1;
-    P1[(c * 3 + 2) * QQQ + o] = a2;
-  }
-  __syncwarp();
-}
-
-// Normalised adjoint, first stage: the folded dots along q2 read Q1/2 or
-// (Q1+1)/2 inputs of one parity; each is scaled by its largest coefficient
-// (the pivot), taken first, so it costs one multiply-add fewer. For table
-// tb (0 = B, 1 = G) and node position r, row tb * N + r of aperm lists the
-// inputs in that order and of arat their coefficients over the pivot;
-// apiv holds the pivot. The stage-1 outputs of node position l are then
-// u0, u1 over the B pivot and u2 over the G pivot; the second stage takes
-// them through C[w][l][q][j] = (pivot / s(l)) x (Bf for w = 0, 2; Gf for
-// w = 1), s(l) the larger of the two pivots (1 if both are zero, whose
-// outputs C then zeroes), so that its outputs, and the nodal y, carry the
-// one factor s(l): the last unfold pass multiplies it back (ysc).
-template <int N, int Q1, class R>
-__device__ void adjoint_tables(const R* Bf, const R* Gf, int* aperm, R* arat, R* apiv, R* C, R* ysc, int tid,
-                               int nth) {
-  constexpr int H = N / 2, QE = (Q1 + 1) / 2;
-  for (int t = tid; t < 2 * N; t += nth) {
-    const int tb = t / N, r = t % N;
-    const R* T = tb ? Gf : Bf;
-    const bool in_odd = (r >= H) != (tb == 1);   // B keeps the parity, G swaps it
-    const int q0 = in_odd ? QE : 0, M = in_odd ? Q1 - QE : QE;
-    int best = q0;
-    R b = T[q0 * N + r];
-    for (int k = 1; k < M; ++k) {
-      const R c = T[(q0 + k) * N + r];
-      if (fabs(c) > fabs(b)) {
-        best = q0 + k;
-        b = c;
-      }
-    }
-    int* pm = aperm + t * QE;
-    R* rt = arat + t * QE;
-    pm[0] = best;
-    rt[0] = R(1);
-    int m = 1;
-    for (int k = 0; k < M; ++k) {
-      const int q = q0 + k;
-      if (q == best) continue;
-      pm[m] = q;
-      rt[m] = b != R(0) ? T[q * N + r] / b : R(0);
-      ++m;
-    }
-    apiv[t] = b;
-  }
-  __syncthreads();
-  for (int t = tid; t < 3 * N * Q1 * N; t += nth) {
-    const int j = t % N, q = (t / N) % Q1, l = (t / (N * Q1)) % N, w = t / (N * Q1 * N);
-    const R sB = apiv[l], sG = apiv[N + l];
-    const R sl = fabs(sB) >= fabs(sG) ? sB : sG;
-    const R f = sl != R(0) ? (w == 2 ? sG : sB) / sl : R(0);
-    C[t] = f * (w == 1 ? Gf : Bf)[q * N + j];
-  }
-  for (int t = tid; t < N; t += nth) {
-    const R sB = apiv[t], sG = apiv[N + t];
-    const R sl = fabs(sB) >= fabs(sG) ? sB : sG;
-    ysc[t] = sl != R(0) ? sl : R(1);
-  }
-}
-
-// adj3_eo with the normalised first stage and the stage-2 tables C; P0
-// holds the folded y divided by ysc[l] on exit.
-template <int N, int Q1, int NC, class R>
-__device__ __forceinline__ void adj3_eon(const R* __restrict__ Bf, const R* __restrict__ Gf,
-                                         const int* __restrict__ aperm, const R* __restrict__ arat,
-                                         const R* __restrict__ C, R* P0, R* P1, int lane) {
-  static_assert(N % 2 == 0, "folded contractions need an even node count");
-  constexpr int H = N / 2, QE = (Q1 + 1) / 2, QO = Q1 / 2;
-  constexpr int NNQ = N * N * Q1, NQQ = N * Q1 * Q1, QQ = Q1 * Q1, QQQ = Q1 * Q1 * Q1;
-  for (int t = lane; t < NC * H * QQ; t += 32) {                // (c, l pair, q1, q0) along q2 -> l
-    const int q01 = t % QQ, lp = (t / QQ) % H, c = t / (QQ * H);
-    const int le = lp, lo = N - 1 - lp;
-    const R* r0 = P1 + (c * 3 + 0) * QQQ + q01;
-    const R* r1 = P1 + (c * 3 + 1) * QQQ + q01;
-    const R* r2 = P1 + (c * 3 + 2) * QQQ + q01;
-    const int* pBe = aperm + le * QE;        // B column le: the even inputs
-    const int* pBo = aperm + lo * QE;        // B column lo: the odd inputs
-    const int* pGe = aperm + (N + le) * QE;  // G column le: the odd inputs
-    const int* pGo = aperm + (N + lo) * QE;  // G column lo: the even inputs
-    const R* wBe = arat + le * QE;
-    const R* wBo = arat + lo * QE;
-    const R* wGe = arat + (N + le) * QE;
-    const R* wGo = arat + (N + lo) * QE;
-    R u0e = r0[pBe[0] * QQ], u1e = r1[pBe[0] * QQ];
-#pragma unroll
-    for (int k = 1; k < QE; ++k) {
-      const int q = pBe[k] * QQ;
-      u0e = fma(r0[q], wBe[k], u0e);
-      u1e = fma(r1[q], wBe[k], u1e);
-    }
-    R u0o = r0[pBo[0] * QQ], u1o = r1[pBo[0] * QQ];
-#pragma unroll
-    for (int k = 1; k < QO; ++k) {
-      const int q = pBo[k] * QQ;
-      u0o = fma(r0[q], wBo[k], u0o);
-      u1o = fma(r1[q], wBo[k], u1o);
-    }
-    R u2e = r2[pGe[0] * QQ];
-#pragma unroll
-    for (int k = 1; k < QO; ++k) u2e = fma(r2[pGe[k] * QQ], wGe[k], u2e);
-    R u2o = r2[pGo[0] * QQ];
-#pragma unroll
-    for (int k = 1; k < QE; ++k) u2o = fma(r2[pGo[k] * QQ], wGo[k], u2o);
-    R* u = P0 + c * 3 * NQQ + q01;
-    u[0 * NQQ + le * QQ] = u0e; u[0 * NQQ + lo * QQ] = u0o;
-    u[1 * NQQ + le * QQ] = u1e; u[1 * NQQ + lo * QQ] = u1o;
-    u[2 * NQQ + le * QQ] = u2e; u[2 * NQQ + lo * QQ] = u2o;
-  }
-  __syncwarp();
-  for (int t = lane; t < NC * N * H * Q1; t += 32) {            // (c, l, j pair, q0) along q1 -> j
-    const int q0 = t % Q1, jp = (t / Q1) % H, l = (t / (Q1 * H)) % N, c = t / (Q1 * H * N);
-    const int je = jp, jo = N - 1 - jp;
-    const R* u0 = P0 + (c * 3 + 0) * NQQ + l * QQ + q0;
-    const R* u1 = P0 + (c * 3 + 1) * NQQ + l * QQ + q0;
-    const R* u2 = P0 + (c * 3 + 2) * NQQ + l * QQ + q0;
-    const R* C0 = C + (0 * N + l) * Q1 * N;
-    const R* C1 = C + (1 * N + l) * Q1 * N;
-    const R* C2 = C + (2 * N + l) * Q1 * N;
-    R vge = R(0), vgo = R(0), vbe = R(0), vbo = R(0);
-#pragma unroll
-    for (int q = 0; q < QE; ++q) {
-      vge = fma(u0[q * Q1], C0[q * N + je], vge);
-      vbe = fma(u2[q * Q1], C2[q * N + je], vbe);
-      vbo = fma(u1[q * Q1], C1[q * N + jo], vbo);
-    }
-#pragma unroll
-    for (int q = QE; q < Q1; ++q) {
-      vgo = fma(u0[q * Q1], C0[q * N + jo], vgo);
-      vbo = fma(u2[q * Q1], C2[q * N + jo], vbo);
-      vbe = fma(u1[q * Q1], C1[q * N + je], vbe);
-    }
-    R* vg = P1 + (c * 2 + 0) * NNQ + l * N * Q1 + q0;
-    R* vb = P1 + (c * 2 + 1) * NNQ + l * N * Q1 + q0;
-    vg[je * Q1] = vge; vg[jo * Q1] = vgo;
-    vb[je * Q1] = vbe; vb[jo * Q1] = vbo;
-  }
-  __syncwarp();
-  for (int t = lane; t < NC * N * N * H; t += 32) {             // (c, l, j, i pair) along q0 -> i
-    const int ip = t % H, lj = (t / H) % (N * N), c = t / (H * N * N);
-    const int ie = ip, io = N - 1 - ip;
-    const R* vg = P1 + (c * 2 + 0) * NNQ + lj * Q1;
-    const R* vb = P1 + (c * 2 + 1) * NNQ + lj * Q1;
-    R ye = R(0), yo = R(0);
-#pragma unroll
-    for (int q = 0; q < QE; ++q) {
-      ye = fma(vb[q], Bf[q * N + ie], ye);
-      yo = fma(vg[q], Gf[q * N + io], yo);
-    }
-#pragma unroll
-    for (int q = QE; q < Q1; ++q) {
-      yo = fma(vb[q], Bf[q * N + io], yo);
-      ye = fma(vg[q], Gf[q * N + ie], ye);
-    }
-    R* y = P0 + (c * N * N + lj) * N;
-    y[ie] = ye;
-    y[io] = yo;
-  }
-  __syncwarp();
-}
-
-// F_N^3 of adj3_eon's output, ysc multiplied back in the axis-2 pass: y at the nodes.
-template <int NF, int L, class R>
-__device__ __forceinline__ void unfold_nodes(R* buf, const R* __restrict__ ysc, int lane) {
-  static_assert(L % 2 == 0, "even node count");
-  mirror3<NF, L, L, L, 0, R>(buf, lane);
-  mirror3<NF, L, L, L, 1, R>(buf, lane);
-  constexpr int H = L / 2, FS = L * L * L, LINES = L * L, ST = L * L;
-#pragma unroll 1
-  for (int t = lane; t < NF * LINES * H; t += 32) {
-    const int i = t % H, line = (t / H) % LINES, f = t / (H * LINES);
-    R* v = buf + f * FS + line;
-    const R bs = v[(L - 1 - i) * ST] * ysc[L - 1 - i];
-    const R a = v[i * ST], sa = ysc[i];
-    v[i * ST] = fma(a, sa, bs);
-    v[(L - 1 - i) * ST] = fma(a, sa, -bs);
-  }
-  __syncwarp();
-}
-
-// Adjoint stages in the folded basis; same buffer layouts as adj3. P1 holds
-// F_Q^3 R on entry; P0 holds the folded y (F_N^3 of it is y) on exit. Each
-// unit computes a mirror pair of outputs: the even position l, which reads
-// the even inputs through Bf and the odd ones through Gf, and the odd
-// position N-1-l, the other way round.
-template <int N, int Q1, int NC, class R>
-__device__ __forceinline__ void adj3_eo(const R* __restrict__ Bf, const R* __restrict__ Gf, R* P0, R* P1, int lane) {
-  static_assert(N % 2 == 0, "folded contractions need an even node count");
-  constexpr int H = N / 2, QE = (Q1 + 1) / 2;
-  constexpr int NNQ = N * N * Q1, NQQ = N * Q1 * Q1, QQ = Q1 * Q1, QQQ = Q1 * Q1 * Q1;
-  for (int t = lane; t < NC * H * QQ; t += 32) {                // (c, l pair, q1, q0) along q2 -> l
-    const int q01 = t % QQ, lp = (t / QQ) % H, c = t / (QQ * H);
-    const int le = lp, lo = N - 1 - lp;
-    const R* r0 = P1 + (c * 3 + 0) * QQQ + q01;
-    const R* r1 = P1 + (c * 3 + 1) * QQQ + q01;
-    const R* r2 = P1 + (c * 3 + 2) * QQQ + q01;
-    R u0e = R(0), u1e = R(0), u2e = R(0), u0o = R(0), u1o = R(0), u2o = R(0);
-#pragma unroll
-    for (int q = 0; q < QE; ++q) {                              // even inputs
-      const R be = Bf[q * N + le], go = Gf[q * N + lo];
-      u0e = fma(r0[q * QQ], be, u0e);
-      u1e = fma(r1[q * QQ], be, u1e);
-      u2o = fma(r2[q * QQ], go, u2o);
-    }
-#pragma unroll
-    for (int q = QE; q < Q1; ++q) {                             // odd inputs
-      const R bo = Bf[q * N + lo], ge = Gf[q * N + le];
-      u0o = fma(r0[q * QQ], bo, u0o);
-      u1o = fma(r1[q * QQ], bo, u1o);
-      u2e = fma(r2[q * QQ], ge, u2e);
-    }
-    R* u = P0 + c * 3 * NQQ + q01;
-    u[0 * NQQ + le * QQ] = u0e; u[0 * NQQ + lo * QQ] = u0o;
-    u[1 * NQQ + le * QQ] = u1e; u[1 * NQQ + lo * QQ] = u1o;
-    u[2 * NQQ + le * QQ] = u2e; u[2 * NQQ + lo * QQ] = u2o;
-  }
-  __syncwarp();
-  for (int t = lane; t < NC * N * H * Q1; t += 32) {            // (c, l, j pair, q0) along q1 -> j
-    const int q0 = t % Q1, jp = (t / Q1) % H, l = (t / (Q1 * H)) % N, c = t / (Q1 * H * N);
-    const int je = jp, jo = N - 1 - jp;
-    const R* u0 = P0 + (c * 3 + 0) * NQQ + l * QQ + q0;
-    const R* u1 = P0 + (c * 3 + 1) * NQQ + l * QQ + q0;
-    const R* u2 = P0 + (c * 3 + 2) * NQQ + l * QQ + q0;
-    R vge = R(0), vgo = R(0), vbe = R(0), vbo = R(0);
-#pragma unroll
-    for (int q = 0; q < QE; ++q) {
-      const R be = Bf[q * N + je], go = Gf[q * N + jo];
-      vge = fma(u0[q * Q1], be, vge);
-      vbe = fma(u2[q * Q1], be, vbe);
-      vbo = fma(u1[q * Q1], go, vbo);
-    }
-#pragma unroll
-    for (int q = QE; q < Q1; ++q) {
-      const R bo = Bf[q * N + jo], ge = Gf[q * N + je];
-      vgo = fma(u0[q * Q1], bo, vgo);
-      vbo = fma(u2[q * Q1], bo, vbo);
-      vbe = fma(u1[q * Q1], ge, vbe);
-    }
-    R* vg = P1 + (c * 2 + 0) * NNQ + l * N * Q1 + q0;
-    R* vb = P1 + (c * 2 + 1) * NNQ + l * N * Q1 + q0;
-    vg[je * Q1] = vge; vg[jo * Q1] = vgo;
-    vb[je * Q1] = vbe; vb[jo * Q1] = vbo;
-  }
-  __syncwarp();
-  for (int t = lane; t < NC * N * N * H; t += 32) {             // (c, l, j, i pair) along q0 -> i
-    const int ip = t % H, lj = (t / H) % (N * N), c = t / (H * N * N);
-    const int ie = ip, io = N - 1 - ip;
-    const R* vg = P1 + (c * 2 + 0) * NNQ + lj * Q1;
-    const R* vb = P1 + (c * 2 + 1) * NNQ + lj * Q1;
-    R ye = R(0), yo = R(0);
-#pragma unroll
-    for (int q = 0; q < QE; ++q) {
-      ye = fma(vb[q], Bf[q * N + ie], ye);
-      yo = fma(vg[q], Gf[q * N + io], yo);
-    }
-#pragma unroll
-    for (int q = QE; q < Q1; ++q) {
-      yo = fma(vb[q], Bf[q * N + io], yo);
-      ye = fma(vg[q], Gf[q * N + ie], ye);
-    }
-    R* y = P0 + (c * N * N + lj) * N;
-    y[ie] = ye;
-    y[io] = yo;
-  }
-  __syncwarp();
-}
-
 // ---------------------------------------------------------------- register-blocked 3D contractions
 // Same maps as fwd3/adj3 with the same buffer layouts, but each lane owns a
 // whole row of outputs: it loads the row's inputs once into registers and

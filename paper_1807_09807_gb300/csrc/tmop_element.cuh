@@ -12,6 +12,7 @@
 // mu it evaluates anyway.
 #pragma once
 #include "tmop_device.cuh"
+#include "tmop_fixed.cuh"
 #include "tmop_kparams.h"
 
 namespace tmop {
@@ -53,23 +54,29 @@ struct ElemCfg {
   static constexpr int B1 = round16<R>(Buf<D, N, Q1, NC>::B1);
   static constexpr int B2 = SPLIT ? round16<R>(D * D * Shape<D, N, Q1>::QP) : 0;
   static constexpr int PER_WARP = (int)sizeof(R) * (B0 + B1 + B2);
-  // up to 8 warps (elements in flight) per block within ~200 KB of shared
-  // memory; the FP64 3D energy, gradient and stored-Hessian product (16 KB
-  // per warp for order 3) run as 6-warp blocks, two per SM: 12 warps in
-  // flight instead of 8 on the FP64 pipe (gradient -2 %, stored-Hessian
-  // product -8 % on 48^3 order-3 hexes)
-  static constexpr bool TWO = D == 3 && sizeof(R) == 8 && OP != OP_LINEARIZE && !HV &&
-                              12 * PER_WARP <= 200 * 1024;
-  static constexpr int WARPS = TWO ? 6
-                                   : ((200 * 1024 / PER_WARP) >= 8 ? 8
-                                                                   : ((200 * 1024 / PER_WARP) < 1 ? 1 : 200 * 1024 / PER_WARP));
-  // FP64 3D with an even node count: contractions in the mirror basis, whose
-  // normalised forward stages need the pivot tables and their products
-  static constexpr bool EO = D == 3 && sizeof(R) == 8 && N % 2 == 0;
-  static constexpr int EO_FWD = 4 * kMaxQ + 3 * Q1 * Q1 * Q1;                           // pivots, ratios, scales
-  static constexpr int EO_ADJ = 2 * kMaxN * kMaxQ + 2 * kMaxN + 3 * N * Q1 * N + kMaxN;  // ratios, pivots, C, ysc
+  // Warps per element. The FP64 3D kernels with 4 or more points per
+  // direction run two warps on an element, in a block of its own, as many
+  // blocks per SM as shared memory holds: the contractions run on the integer
+  // pipes beside the FP64 pipe, and with one warp per element only 2-3 warps
+  // per scheduler hide their latency (48^3 order-3 hexes, gradient + Hessian
+  // action: 8.30 ms with one warp, 6.87 ms with two, 5.53 ms with one copy of
+  // the forward map's code for x and v, which took the misses of the
+  // instruction cache down).
+  static constexpr bool FX3 = D == 3 && sizeof(R) == 8;
+  static constexpr int G = (FX3 && Q1 >= 4 && OP != OP_ENERGY && OP != OP_LINEARIZE) ? 2 : 1;
+  // Elements in flight per block: up to 8 within ~200 KB of shared memory;
+  // the FP64 3D energy as two blocks of 6 per SM where they fit
+  static constexpr bool TWO = FX3 && OP == OP_ENERGY && 12 * PER_WARP <= 200 * 1024;
+  static constexpr int FIT = 200 * 1024 / PER_WARP;
+  static constexpr int WARPS = G == 2 ? 1 : (TWO ? 6 : (FIT >= 8 ? 8 : (FIT < 1 ? 1 : FIT)));
+  // blocks per SM that bound the registers (0: no bound): 8 (128 registers),
+  // 10 (96) for the gradient, whose pointwise stage needs fewer (32^3 order-2
+  // hexes, mu302: 422 us with 8, 392 us with 10; the stored-Hessian product
+  // 211 us with 8, 223 us with 12)
+  static constexpr int WANT = (OP == OP_GRADIENT || OP == OP_ENERGY_GRAD) ? 10 : 8;
+  static constexpr int MINB = G == 2 ? (FIT >= WANT ? WANT : FIT) : (TWO ? 2 : 0);
   // after the 1D tables: the product weight w_q0 w_q1 (w_q2) of every point
-  static constexpr int WQ_OFF = 2 * kMaxQ * kMaxN + kMaxQ + (EO ? EO_FWD + EO_ADJ : 0);
+  static constexpr int WQ_OFF = 2 * kMaxQ * kMaxN + kMaxQ;
   static constexpr int TABLE = round16<R>(WQ_OFF + Shape<D, N, Q1>::QP);
   static constexpr size_t smem_bytes() { return sizeof(R) * (TABLE + WARPS * (B0 + B1 + B2)); }
 };
@@ -114,39 +121,26 @@ __device__ __forceinline__ bool metric_dP(int id, const R* T, const R* dT, R* S)
 }
 
 template <int D, int N, int Q1, class R, int OP>
-__global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP>::WARPS * 32, ElemCfg<D, N, Q1, R, OP>::TWO ? 2 : 0)
+__global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP>::WARPS * ElemCfg<D, N, Q1, R, OP>::G * 32,
+                                  ElemCfg<D, N, Q1, R, OP>::MINB)
     elem_kernel(const KParams p) {
   using Cfg = ElemCfg<D, N, Q1, R, OP>;
   constexpr int NDOF = Shape<D, N, Q1>::NDOF, QP = Shape<D, N, Q1>::QP, DD = D * D;
-  constexpr int WARPS = Cfg::WARPS;
+  constexpr int WARPS = Cfg::WARPS, G = Cfg::G, GT = 32 * G;   // elements per block, warps and threads per element
   extern __shared__ __align__(16) unsigned char smem_raw[];
   R* sB = reinterpret_cast<R*>(smem_raw);
   R* sG = sB + kMaxQ * kMaxN;
   R* sw = sG + kMaxQ * kMaxN;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int lane = threadIdx.x % GT, warp = threadIdx.x / GT;   // thread of the element's group, group of the block
+  const int bar = 1 + warp;
   R* P0 = sB + Cfg::TABLE + warp * (Cfg::B0 + Cfg::B1 + Cfg::B2);
   R* P1 = P0 + Cfg::B0;
   R* P2 = P1 + Cfg::B1;  // A(x) of the split 3D Hessian action
 
-  // FP64 3D kernels with an even node count contract in the mirror basis
-  // (fwd3_eon / adj3_eon): sB, sG then hold the folded tables, followed by
-  // the normalised maps' pivots, ratios, scale products and stage-2 tables
-  constexpr bool EO = Cfg::EO;
-  R* s_piv = sw + kMaxQ;
-  R* s_rt = s_piv + 2 * kMaxQ;
-  R* s_Sc = s_rt + 2 * kMaxQ;
-  R* s_arat = s_Sc + 3 * Q1 * Q1 * Q1;
-  R* s_apiv = s_arat + 2 * kMaxN * kMaxQ;
-  R* s_C = s_apiv + 2 * kMaxN;
-  R* s_ysc = s_C + 3 * N * Q1 * N;
-  __shared__ int s_kf[2 * kMaxQ];
-  __shared__ int s_aperm[2 * kMaxN * kMaxQ];
-  if constexpr (EO) {
-    folded_tables<N, Q1, R>(p.B, p.G, sB, sG, threadIdx.x, blockDim.x);
-    __syncthreads();
-    normalised_tables<N, Q1, R>(sB, sG, s_kf, s_rt, s_piv, s_Sc, threadIdx.x, blockDim.x);
-    adjoint_tables<N, Q1, R>(sB, sG, s_aperm, s_arat, s_apiv, s_C, s_ysc, threadIdx.x, blockDim.x);
-  } else {
+  // FP64: contractions in fixed point (tmop_fixed.cuh), tables from the
+  // parameter block; FP32: tables in shared memory (2D) or registers (3D)
+  constexpr bool FX = sizeof(R) == 8;
+  if constexpr (!FX) {
     for (int t = threadIdx.x; t < Q1 * N; t += blockDim.x) {
       sB[t] = R(p.B[t]);
       sG[t] = R(p.G[t]);
@@ -161,6 +155,7 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP>::WARPS * 32, ElemCfg<
     if constexpr (D == 3) w *= R(p.w1[t / (Q1 * Q1)]);
     sWq[t] = w;
   }
+  __shared__ unsigned s_mag[WARPS][G * 2 * D];   // per warp and component: largest magnitudes of the group's warps
   R Wi[DD];
 #pragma unroll
   for (int i = 0; i < DD; ++i) Wi[i] = R(p.Winv[i]);
@@ -188,6 +183,7 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP>::WARPS * 32, ElemCfg<
   // its second 3D adjoint runs its stage 2 in the A(x) buffer
   static_assert(!(OP == OP_GRAD_HESS && D == 3) || 2 * D * N * N * Q1 <= Cfg::B2, "B2 too small");
   static_assert(OP != OP_LINEARIZE_C || D == 3, "compact records are 3D");
+  static_assert(!FX || Cfg::NC * FxNodal<D, N>::CS <= Cfg::B0, "B0 too small for the padded nodal fields");
   NodeMap<N> nodes(p.elem_nodes, p.sx, p.sy, D == 3 ? N - 1 : 1);
   const int ecount = p.elist ? p.ecount : p.nelem;
   for (int ei = blockIdx.x * WARPS + warp; ei < ecount; ei += nwarps_total) {
@@ -204,17 +200,20 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP>::WARPS * 32, ElemCfg<
         for (int t = 0; t < NSH; ++t) hpre[t] = __ldg(H0 + (size_t)t * Shape<D, N, Q1>::QP);
       }
     }
-    // ---- gather. In FP32 the coordinates are taken relative to the element's
-    // first node (in FP64) before rounding: A is translation invariant
-    // (sum_i grad phi_i = 0), and this keeps the FP32 relative error of A at
-    // the level of eps32 instead of eps32 |x| / h.
+    // ---- gather. The coordinates are taken relative to the element's first
+    // node (in FP64) before they are rounded (FP32) or given the element's
+    // common exponent (FP64): A is translation invariant (sum_i grad phi_i =
+    // 0), and this keeps the relative error of A at the level of eps instead
+    // of eps |x| / h.
     double xref[D];
-    if constexpr (sizeof(R) == 4 && !PA_APPLY) {
+    unsigned mag[FX ? Cfg::NC : 1] = {};   // FP64: largest magnitude (high word) per gathered component
+    auto nodal = [&](int c, int t) { return FX ? FxNodal<D, N>::at(c, t) : c * NDOF + t; };
+    if constexpr (!PA_APPLY) {
       const int g0 = nodes(0);
 #pragma unroll
       for (int c = 0; c < D; ++c) xref[c] = __ldg(p.x + (size_t)c * p.nnode + g0);
     }
-    for (int t = lane; t < NDOF; t += 32) {
+    for (int t = lane; t < NDOF; t += GT) {
       const int g = nodes(t);
       if constexpr (PA_APPLY) {
         // the partially assembled product needs only the direction v
@@ -222,39 +221,72 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP>::WARPS * 32, ElemCfg<
         for (int c = 0; c < D; ++c) {
           const size_t dof = (size_t)c * p.nnode + g;
           const bool fx = p.fixed && __ldg(p.fixed + dof);
-          P0[c * NDOF + t] = fx ? R(0) : (p.v32 ? R(__ldg(p.v32 + dof)) : from_f64<R>(__ldg(p.v + dof)));
+          const R vv = fx ? R(0) : (p.v32 ? R(__ldg(p.v32 + dof)) : from_f64<R>(__ldg(p.v + dof)));
+          P0[nodal(c, t)] = vv;
+          if constexpr (FX) mag[c] = max(mag[c], fx_mag(vv));
         }
         continue;
       }
 #pragma unroll
       for (int c = 0; c < D; ++c) {
-        const double xv = __ldg(p.x + (size_t)c * p.nnode + g);
-        if constexpr (sizeof(R) == 4) P0[c * NDOF + t] = from_f64<R>(xv - xref[c]);
-        else P0[c * NDOF + t] = R(xv);
+        const double xv = __ldg(p.x + (size_t)c * p.nnode + g) - xref[c];
+        P0[nodal(c, t)] = from_f64<R>(xv);
+        if constexpr (FX) mag[c] = max(mag[c], fx_mag(xv));
       }
       if constexpr (Cfg::HV && !Cfg::SPLIT) {
 #pragma unroll
         for (int c = 0; c < D; ++c) {
           const size_t dof = (size_t)c * p.nnode + g;
           const bool fx = p.fixed && __ldg(p.fixed + dof);
-          P0[(D + c) * NDOF + t] = fx ? R(0) : from_f64<R>(__ldg(p.v + dof));
+          const double vv = fx ? 0.0 : __ldg(p.v + dof);
+          P0[nodal(D + c, t)] = from_f64<R>(vv);
+          if constexpr (FX) mag[D + c] = max(mag[D + c], fx_mag(vv));
         }
       }
     }
-    __syncwarp();
-    // ---- forward contraction: A (and dA) at every point
-    if constexpr (Cfg::SPLIT) {
-      // A(x) into P2 (P2 also serves as the first stage buffer), then v
-      if constexpr (EO) {
-        mirror3_all<D, N, R>(P0, lane);
-        fwd3_eon<N, Q1, D, R>(s_kf, s_rt, P0, P2, lane);
-        unfold_points<D * D, Q1, R>(P2, s_Sc, lane);
-      } else if constexpr (RB) {
-        fwd3_rb<N, Q1, D, R>(tB, tG, P0, P2, lane);
-      } else {
-        fwd3<N, Q1, D, R>(sB, sG, P0, P2, lane);
+    // the split Hessian action's v, loaded behind x and masked
+    constexpr int VPRE = (Cfg::SPLIT && FX) ? (NDOF + GT - 1) / GT : 0;
+    double vpre[VPRE > 0 ? VPRE * D : 1];
+#pragma unroll
+    for (int k = 0; k < VPRE; ++k) {
+      const int t = lane + k * GT;
+      if (t >= NDOF) break;
+      const int g = nodes(t);
+#pragma unroll
+      for (int c = 0; c < D; ++c) {
+        const size_t dof = (size_t)c * p.nnode + g;
+        const double vv = __ldg(p.v + dof);
+        vpre[k * D + c] = (p.fixed && __ldg(p.fixed + dof)) ? 0.0 : vv;
       }
-      for (int t = lane; t < NDOF; t += 32) {
+    }
+    int em[FX ? Cfg::NC : 1];
+    if constexpr (FX) fx_group_exp<G, Cfg::NC>(mag, em, s_mag[warp], bar);
+    else __syncwarp();
+    // ---- forward contraction: A (and dA) at every point
+    if constexpr (Cfg::SPLIT && FX) {
+      // A(x) into P2 (P2 also serves as the first stage buffer), then v into
+      // P1, by one copy of the code
+#pragma unroll 1
+      for (int f = 0;; ++f) {
+        fwd3_fx<N, Q1, D, G>(p.fx, em, P0, f == 0 ? P2 : P1, lane, bar);
+        if (f) break;
+#pragma unroll
+        for (int c = 0; c < D; ++c) mag[c] = 0;
+#pragma unroll
+        for (int k = 0; k < VPRE; ++k) {
+          const int t = lane + k * GT;
+          if (t >= NDOF) break;
+#pragma unroll
+          for (int c = 0; c < D; ++c) {
+            P0[nodal(c, t)] = vpre[k * D + c];
+            mag[c] = max(mag[c], fx_mag(vpre[k * D + c]));
+          }
+        }
+        fx_group_exp<G, D>(mag, em, s_mag[warp], bar);
+      }
+    } else if constexpr (Cfg::SPLIT) {
+      fwd3_rb<N, Q1, D, R>(tB, tG, P0, P2, lane);
+      for (int t = lane; t < NDOF; t += GT) {
         const int g = nodes(t);
 #pragma unroll
         for (int c = 0; c < D; ++c) {
@@ -264,33 +296,24 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP>::WARPS * 32, ElemCfg<
         }
       }
       __syncwarp();
-      if constexpr (EO) {
-        mirror3_all<D, N, R>(P0, lane);
-        fwd3_eon<N, Q1, D, R>(s_kf, s_rt, P0, P1, lane);
-        unfold_points<D * D, Q1, R>(P1, s_Sc, lane);
-      } else if constexpr (RB) {
-        fwd3_rb<N, Q1, D, R>(tB, tG, P0, P1, lane);
-      } else {
-        fwd3<N, Q1, D, R>(sB, sG, P0, P1, lane);
-      }
+      fwd3_rb<N, Q1, D, R>(tB, tG, P0, P1, lane);
     } else if constexpr (D == 2) {
-      fwd2<N, Q1, Cfg::NC, R>(sB, sG, P0, P1, lane);
-    } else if constexpr (EO) {
-      mirror3_all<Cfg::NC, N, R>(P0, lane);
-      fwd3_eon<N, Q1, Cfg::NC, R>(s_kf, s_rt, P0, P1, lane);
-      unfold_points<Cfg::NC * D, Q1, R>(P1, s_Sc, lane);
-    } else if constexpr (RB) {
-      fwd3_rb<N, Q1, Cfg::NC, R>(tB, tG, P0, P1, lane);
+      if constexpr (FX) fwd2_fx<N, Q1, Cfg::NC, G>(p.fx, em, P0, P1, lane, bar);
+      else fwd2<N, Q1, Cfg::NC, R>(sB, sG, P0, P1, lane);
     } else {
-      fwd3<N, Q1, Cfg::NC, R>(sB, sG, P0, P1, lane);
+      if constexpr (FX) fwd3_fx<N, Q1, Cfg::NC, G>(p.fx, em, P0, P1, lane, bar);
+      else fwd3_rb<N, Q1, Cfg::NC, R>(tB, tG, P0, P1, lane);
     }
     R* Abuf = Cfg::SPLIT ? P2 : ((D == 2) ? P0 : P1);     // A: [D][D][QP]
     R* dAbuf = Cfg::SPLIT ? P1 : Abuf + DD * QP;         // dA (Hessian action)
     R* Rbuf = Cfg::SPLIT ? P1 : Abuf;                    // per-point output of the adjoint
     // ---- pointwise
     double emin = INFINITY;
+    // FP64: largest magnitude (high word) per component of the fields the
+    // adjoint map takes (OP_GRAD_HESS: the gradient's, then the Hessian action's)
+    unsigned rmag[FX ? 2 * D : 1] = {};
     constexpr int NS = DD * (DD + 1) / 2;
-    for (int q = lane; q < QP; q += 32) {
+    for (int q = lane; q < QP; q += GT) {
       if constexpr (OP == OP_HESS_PA) {
         // y = H dA with the stored symmetric A-space Hessian (already scaled by w det W)
         const R* H = static_cast<const R*>(p.pa) + (size_t)e * p.pa_stride + q;
@@ -318,7 +341,10 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP>::WARPS * 32, ElemCfg<
             if (c != r) y[c] = fma(h[s], dA[r], y[c]);
           }
 #pragma unroll
-        for (int i = 0; i < DD; ++i) Abuf[i * QP + q] = y[i];
+        for (int i = 0; i < DD; ++i) {
+          Abuf[i * QP + q] = y[i];
+          if constexpr (FX) rmag[i / D] = max(rmag[i / D], fx_mag(y[i]));
+        }
         continue;
       }
       R A[DD];
@@ -415,8 +441,12 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP>::WARPS * 32, ElemCfg<
                 rh = fma(Sh[a * D + c], Wi[b * D + c], rh);
               }
             }
-            Abuf[(a * D + b) * QP + q] = ok ? rg : R(0);
-            dAbuf[(a * D + b) * QP + q] = ok ? rh : R(0);
+            rg = ok ? rg : R(0);
+            rh = ok ? rh : R(0);
+            Abuf[(a * D + b) * QP + q] = rg;
+            dAbuf[(a * D + b) * QP + q] = rh;
+            rmag[a] = max(rmag[a], fx_mag(rg));
+            rmag[D + a] = max(rmag[D + a], fx_mag(rh));
           }
         continue;
       }
@@ -611,7 +641,9 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP>::WARPS * 32, ElemCfg<
 #pragma unroll
               for (int c = 0; c < D; ++c) r = fma(S[a * D + c], Wi[b * D + c], r);
             }
-            Rbuf[(a * D + b) * QP + q] = ok ? r : R(0);
+            r = ok ? r : R(0);
+            Rbuf[(a * D + b) * QP + q] = r;
+            if constexpr (FX) rmag[a] = max(rmag[a], fx_mag(r));
           }
         if (p.metric2) {
           // + eta w det W2 S2 W2^-t (S2 = P2 or dP2 at T2 = A W2^-1)
@@ -640,7 +672,9 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP>::WARPS * 32, ElemCfg<
                 R r2 = R(0);
 #pragma unroll
                 for (int c = 0; c < D; ++c) r2 = fma(S2[a * D + c], R(p.Winv2[b * D + c]), r2);
-                Rbuf[(a * D + b) * QP + q] = fma(s2, r2, Rbuf[(a * D + b) * QP + q]);
+                r2 = fma(s2, r2, Rbuf[(a * D + b) * QP + q]);
+                Rbuf[(a * D + b) * QP + q] = r2;
+                if constexpr (FX) rmag[a] = max(rmag[a], fx_mag(r2));
               }
           }
         }
@@ -656,63 +690,64 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP>::WARPS * 32, ElemCfg<
         if (lane == 0) p.elem_min[e] = emin;
       }
     } else if constexpr (OP == OP_GRAD_HESS) {
-      __syncwarp();
       // ---- two adjoint contractions: 3D, the Hessian action's fields (P1)
       // into y, then the gradient's (P2) into g, each through P0 and its own
       // buffer; 2D, both at once (components 0..D-1 the gradient's fields,
       // D..2D-1 the Hessian action's)
       if constexpr (D == 2) {
-        adj2<N, Q1, 2 * D, R>(sB, sG, P0, P1, lane);
-        for (int t = lane; t < NDOF; t += 32) {
+        // P0 holds the gradient's fields (in place of A), then the Hessian action's (dA)
+        int er[2 * D];
+        fx_group_exp<G, 2 * D>(rmag, er, s_mag[warp], bar);
+        adj2_fx<N, Q1, 2 * D, G>(p.fx, er, P0, P1, lane, bar);
+        for (int t = lane; t < NDOF; t += GT) {
           const int gn = nodes(t);
 #pragma unroll
           for (int c = 0; c < D; ++c) {
             const size_t dof = (size_t)c * p.nnode + gn;
             if (p.fixed && __ldg(p.fixed + dof)) continue;
-            atomicAdd(p.g + dof, to_f64(P0[c * NDOF + t]));
-            atomicAdd(p.y + dof, to_f64(P0[(D + c) * NDOF + t]));
+            atomicAdd(p.g + dof, P0[nodal(c, t)]);
+            atomicAdd(p.y + dof, P0[nodal(D + c, t)]);
           }
         }
       } else {
+        int er2[2 * D];
+        fx_group_exp<G, 2 * D>(rmag, er2, s_mag[warp], bar);
 #pragma unroll 1
         for (int pass = 0; pass < 2; ++pass) {
           R* Rin = pass == 0 ? P1 : P2;
           double* out = pass == 0 ? p.y : p.g;
-          if constexpr (EO) {
-            mirror3_all<D * D, Q1, R>(Rin, lane);
-            adj3_eon<N, Q1, D, R>(sB, sG, s_aperm, s_arat, s_C, P0, Rin, lane);
-            unfold_nodes<D, N, R>(P0, s_ysc, lane);
-          } else {
-            adj3<N, Q1, D, R>(sB, sG, P0, Rin, lane);
-          }
-          for (int t = lane; t < NDOF; t += 32) {
+          int er[D];
+#pragma unroll
+          for (int c = 0; c < D; ++c) er[c] = pass == 0 ? er2[D + c] : er2[c];
+          adj3_fx<N, Q1, D, G>(p.fx, er, P0, Rin, lane, bar);
+          for (int t = lane; t < NDOF; t += GT) {
             const int gn = nodes(t);
 #pragma unroll
             for (int c = 0; c < D; ++c) {
               const size_t dof = (size_t)c * p.nnode + gn;
               if (p.fixed && __ldg(p.fixed + dof)) continue;
-              atomicAdd(out + dof, to_f64(P0[c * NDOF + t]));
+              atomicAdd(out + dof, P0[nodal(c, t)]);
             }
           }
-          __syncwarp();
+          group_sync<G>(bar);
         }
       }
     } else {
       if constexpr (EG) accMin = fmin(accMin, emin);
-      __syncwarp();
       // ---- adjoint contraction and scatter
-      if constexpr (D == 2) {
+      if constexpr (FX) {
+        int er[D];
+        fx_group_exp<G, D>(rmag, er, s_mag[warp], bar);
+        if constexpr (D == 2) adj2_fx<N, Q1, D, G>(p.fx, er, P0, P1, lane, bar);
+        else adj3_fx<N, Q1, D, G>(p.fx, er, P0, P1, lane, bar);
+      } else if constexpr (D == 2) {
+        __syncwarp();
         adj2<N, Q1, D, R>(sB, sG, P0, P1, lane);
-      } else if constexpr (EO) {
-        mirror3_all<D * D, Q1, R>(P1, lane);
-        adj3_eon<N, Q1, D, R>(sB, sG, s_aperm, s_arat, s_C, P0, P1, lane);
-        unfold_nodes<D, N, R>(P0, s_ysc, lane);
-      } else if constexpr (RB) {
-        adj3_rb<N, Q1, D, R>(tB, tG, P0, P1, lane);
       } else {
-        adj3<N, Q1, D, R>(sB, sG, P0, P1, lane);
+        __syncwarp();
+        adj3_rb<N, Q1, D, R>(tB, tG, P0, P1, lane);
       }
-      for (int t = lane; t < NDOF; t += 32) {
+      for (int t = lane; t < NDOF; t += GT) {
         const int g = nodes(t);
 #pragma unroll
         for (int c = 0; c < D; ++c) {
@@ -721,26 +756,26 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP>::WARPS * 32, ElemCfg<
           // (one colour per launch in the deterministic mode: no other
           // element of the launch adds to this node, so each node gets one
           // add per launch, in colour order)
-          if (PA_APPLY && p.y32) atomicAdd(p.y32 + dof, float(P0[c * NDOF + t]));   // FP32 Krylov vectors
-          else atomicAdd(p.y + dof, to_f64(P0[c * NDOF + t]));
+          if (PA_APPLY && p.y32) atomicAdd(p.y32 + dof, float(P0[nodal(c, t)]));   // FP32 Krylov vectors
+          else atomicAdd(p.y + dof, to_f64(P0[nodal(c, t)]));
         }
       }
     }
-    __syncwarp();
+    group_sync<G>(bar);
   }
 
   if constexpr (OP == OP_ENERGY || EG) {
-    __shared__ double redF[WARPS], redM[WARPS];
+    __shared__ double redF[WARPS * G], redM[WARPS * G];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
       accF += __shfl_xor_sync(0xffffffffu, accF, o);
       accMin = fmin(accMin, __shfl_xor_sync(0xffffffffu, accMin, o));
     }
-    if (lane == 0) { redF[warp] = accF; redM[warp] = accMin; }
+    if (threadIdx.x % 32 == 0) { redF[threadIdx.x / 32] = accF; redM[threadIdx.x / 32] = accMin; }
     __syncthreads();
     if (threadIdx.x == 0) {
       double f = 0.0, m = INFINITY;
-      for (int w = 0; w < WARPS; ++w) { f += redF[w]; m = fmin(m, redM[w]); }
+      for (int w = 0; w < WARPS * G; ++w) { f += redF[w]; m = fmin(m, redM[w]); }
       p.part_F[blockIdx.x] = f;
       p.part_min[blockIdx.x] = m;
     }
@@ -751,7 +786,7 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP>::WARPS * 32, ElemCfg<
 template <int D, int N, int Q1, class R, int OP>
 int launch_elem(const KParams& p, int grid, void* stream) {
   using Cfg = ElemCfg<D, N, Q1, R, OP>;
-  elem_kernel<D, N, Q1, R, OP><<<grid, Cfg::WARPS * 32, Cfg::smem_bytes(), (cudaStream_t)stream>>>(p);
+  elem_kernel<D, N, Q1, R, OP><<<grid, Cfg::WARPS * Cfg::G * 32, Cfg::smem_bytes(), (cudaStream_t)stream>>>(p);
   return (int)cudaGetLastError();
 }
 
@@ -765,7 +800,7 @@ int prepare_elem_impl(int nelem, int* grid) {
   if (err != cudaSuccess) return (int)err;
   int per_sm = 0, dev = 0, sms = 0;
   err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void*)elem_kernel<D, N, Q1, R, OP>,
-                                                      Cfg::WARPS * 32, smem);
+                                                      Cfg::WARPS * Cfg::G * 32, smem);
   if (err != cudaSuccess) return (int)err;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);

@@ -27,7 +27,18 @@ enum {
 constexpr int kCompactRec = 14;  // values per point of the compact record (3D)
 enum { WK_IDENTITY = 0, WK_CONST = 1, WK_PER_QP = 2 };
 
+// Tables of the FP64 kernels' fixed-point contractions (tmop_fixed.cuh): the
+// even and odd parts of B and of 2^-gexp G over the first half of the points
+// q and of the nodes i (index 3 q + i), each entry c as c 2^60 = H 2^30 + L.
+struct FxTab {
+  int BeH[12], BeL[12], BoH[12], BoL[12], GeH[12], GeL[12], GoH[12], GoL[12];
+  int gexp;   // max |G entries| <= 2^gexp
+  int xin;    // bits of the forward map's inputs below their common exponent
+  int rin;    // the same of the adjoint map
+};
+
 struct KParams {
+  FxTab fx;
   int dim, nelem, nnode, metric, wkind;
   int sx, sy, sz;                 // structured grid (sx > 0) or elem_nodes
   const int32_t* elem_nodes;      // [nelem][n^d]
@@ -103,5 +114,6 @@ bool rule_gl(int q, double* x, double* w);
 bool rule_gll(int q, double* x, double* w);
 void lagrange_bary(int n, const double* z, double s, double* phi, double* dphi);
 bool inv_h(int d, const double* W, double* Wi, double* detW);
+bool fx_tables(int dim, int n, int q, const double* B, const double* G, FxTab* T);
 
 }  // namespace tmop

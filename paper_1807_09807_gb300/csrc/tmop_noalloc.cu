@@ -98,6 +98,7 @@ extern "C" int tmop_energy_noalloc(int dim, int order, const int structured[3], 
     }
     p.w1[a] = qw[a];
   }
+  if (!fx_tables(dim, n, nq, p.B, p.G, &p.fx)) return TMOP_ERR_ARG;
   double Wc[9] = {0};
   switch (targets->kind) {
     case TMOP_W_IDENTITY:
