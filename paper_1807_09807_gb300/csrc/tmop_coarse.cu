@@ -155,61 +155,85 @@ __device__ __forceinline__ double block_sum_c(double v) {
 // (M x N = (M x Kd)(Kd x N)), with A(i, k) = A[b sAb + i lda + k],
 // B(k, j) = B[b sBb + k ldb + j], C(i, j) = C[b sCb + i ldc + j]: along x
 // (inner = 1) In [rows][L] times S (symmetric), along y or z S times every
-// [L][inner] slab. 64 x 64 output tiles over 16-deep chunks staged in shared
-// memory, 4 x 4 outputs per thread (rows ty + 16 r, columns tx + 16 c).
-constexpr int kTM = 64, kTN = 64, kTK = 16;
-
-template <class R>
-__global__ void __launch_bounds__(256, 2) k_dst(const R* __restrict__ A, const R* __restrict__ B, R* __restrict__ C,
-                                             int M, int N, int Kd, int batch, size_t sAb, int lda, size_t sBb,
-                                             int ldb, size_t sCb, int ldc) {
-  __shared__ R As[kTK][kTM + 1];
-  __shared__ R Bs[kTK][kTN];
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  const int tiles_n = (N + kTN - 1) / kTN, tiles_m = (M + kTM - 1) / kTM;
+// [L][inner] slab. Output tiles of T x T over KC-deep chunks staged in shared
+// memory, P x P outputs per thread (rows ty + (T/P) r, columns tx + (T/P) c).
+template <class R, int T, int P, int KC>
+__global__ void __launch_bounds__((T / P) * (T / P)) k_dst(const R* __restrict__ A, const R* __restrict__ B,
+                                                           R* __restrict__ C, int M, int N, int Kd, int batch,
+                                                           size_t sAb, int lda, size_t sBb, int ldb, size_t sCb,
+                                                           int ldc) {
+  constexpr int W = T / P, NT = W * W;
+  __shared__ R As[KC][T + 1];
+  __shared__ R Bs[KC][T];
+  const int tid = threadIdx.x, tx = tid % W, ty = tid / W;
+  const int tiles_n = (N + T - 1) / T, tiles_m = (M + T - 1) / T;
   for (int b = blockIdx.z; b < batch; b += gridDim.z)
     for (int tm = blockIdx.y; tm < tiles_m; tm += gridDim.y)
       for (int tn = blockIdx.x; tn < tiles_n; tn += gridDim.x) {
         const R* Ab = A + b * sAb;
         const R* Bb = B + b * sBb;
-        const int i0 = tm * kTM, j0 = tn * kTN;
-        R acc[4][4];
+        const int i0 = tm * T, j0 = tn * T;
+        R acc[P][P];
 #pragma unroll
-        for (int r = 0; r < 4; ++r)
+        for (int r = 0; r < P; ++r)
 #pragma unroll
-          for (int c = 0; c < 4; ++c) acc[r][c] = R(0);
-        for (int k0 = 0; k0 < Kd; k0 += kTK) {
+          for (int c = 0; c < P; ++c) acc[r][c] = R(0);
+        for (int k0 = 0; k0 < Kd; k0 += KC) {
 #pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            const int i = (tid >> 4) + 16 * q, k = tid & 15;   // A tile: 16 consecutive k per row
+          for (int q = tid; q < KC * T; q += NT) {
+            const int i = q / KC, k = q % KC;   // A tile: consecutive k per row
             As[k][i] = (i0 + i < M && k0 + k < Kd) ? Ab[(size_t)(i0 + i) * lda + k0 + k] : R(0);
-            const int kb = (tid >> 6) + 4 * q, j = tid & 63;   // B tile: 64 consecutive j per row
+            const int kb = q / T, j = q % T;    // B tile: consecutive j per row
             Bs[kb][j] = (k0 + kb < Kd && j0 + j < N) ? Bb[(size_t)(k0 + kb) * ldb + j0 + j] : R(0);
           }
           __syncthreads();
+#pragma unroll 16
+          for (int k = 0; k < KC; ++k) {
+            R a[P], bb[P];
 #pragma unroll
-          for (int k = 0; k < kTK; ++k) {
-            R a[4], bb[4];
+            for (int r = 0; r < P; ++r) a[r] = As[k][ty + W * r];
 #pragma unroll
-            for (int r = 0; r < 4; ++r) a[r] = As[k][ty + 16 * r];
+            for (int c = 0; c < P; ++c) bb[c] = Bs[k][tx + W * c];
 #pragma unroll
-            for (int c = 0; c < 4; ++c) bb[c] = Bs[k][tx + 16 * c];
+            for (int r = 0; r < P; ++r)
 #pragma unroll
-            for (int r = 0; r < 4; ++r)
-#pragma unroll
-              for (int c = 0; c < 4; ++c) acc[r][c] = fmaR(a[r], bb[c], acc[r][c]);
+              for (int c = 0; c < P; ++c) acc[r][c] = fmaR(a[r], bb[c], acc[r][c]);
           }
           __syncthreads();
         }
         R* Cb = C + b * sCb;
 #pragma unroll
-        for (int r = 0; r < 4; ++r)
+        for (int r = 0; r < P; ++r)
 #pragma unroll
-          for (int c = 0; c < 4; ++c) {
-            const int i = i0 + ty + 16 * r, j = j0 + tx + 16 * c;
+          for (int c = 0; c < P; ++c) {
+            const int i = i0 + ty + W * r, j = j0 + tx + W * c;
             if (i < M && j < N) Cb[(size_t)i * ldc + j] = acc[r][c];
           }
       }
+}
+
+template <class R, int T, int P, int KC>
+void launch_dst(const R* A, const R* B, R* C, int M, int N, int Kd, int batch, size_t sAb, int lda, size_t sBb,
+                int ldb, size_t sCb, int ldc, cudaStream_t s) {
+  const int tm = (M + T - 1) / T, tn = (N + T - 1) / T;
+  const dim3 g(tn < 65535 ? tn : 65535, tm < 65535 ? tm : 65535, batch < 65535 ? batch : 65535);
+  k_dst<R, T, P, KC><<<g, (T / P) * (T / P), 0, s>>>(A, B, C, M, N, Kd, batch, sAb, lda, sBb, ldb, sCb, ldc);
+}
+
+// The tile by the number of 64 x 64 tiles. With 60 or more of them (47^3
+// coarse vertices: 104 to 141) the 64 tile's fewer loads per multiply-add
+// win: two-level FP32 Newton on 48^3 order-3 hexes 89.6 ms against 92.3 ms
+// with 32 tiles. A small coarse grid leaves one or two 64 tiles, i.e. one or
+// two of 152 SMs, whose FP64 pipe (2 operations per clock) then bounds the
+// transform: 63^2 vertices, FP64, 71 us; with 16 tiles (32 blocks) 4 us, and
+// the two-level FP64 Newton solve on 64^2 order-3 quads takes 22.8 ms instead
+// of 110 ms.
+template <class R>
+void dst_product(const R* A, const R* B, R* C, int M, int N, int Kd, int batch, size_t sAb, int lda, size_t sBb,
+                 int ldb, size_t sCb, int ldc, cudaStream_t s) {
+  const double tiles = ceil(M / 64.0) * ceil(N / 64.0) * batch;
+  if (tiles >= 60) launch_dst<R, 64, 4, 16>(A, B, C, M, N, Kd, batch, sAb, lda, sBb, ldb, sCb, ldc, s);
+  else launch_dst<R, 16, 1, 64>(A, B, C, M, N, Kd, batch, sAb, lda, sBb, ldb, sCb, ldc, s);
 }
 
 // divide by alpha times the eigenvalue of K_c at every coarse point, in the
@@ -347,16 +371,10 @@ void dst_pass(CoarseSpace* cs, int a, const R* src, R* dst, cudaStream_t s) {
   const int L = cs->Lc[a];
   const R* S = tab_S<R>(cs, a);
   if (inner == 1) {   // [rows][L] S
-    const int M = (int)outer;
-    const int tm = (M + kTM - 1) / kTM, tn = (L + kTN - 1) / kTN;
-    const dim3 g(tn, tm < 65535 ? tm : 65535, 1);
-    k_dst<R><<<g, 256, 0, s>>>(src, S, dst, M, L, L, 1, 0, L, 0, L, 0, L);
+    dst_product<R>(src, S, dst, (int)outer, L, L, 1, 0, L, 0, L, 0, L, s);
   } else {            // S [L][inner] for every outer slab
-    const int N = (int)inner, batch = (int)outer;
-    const int tm = (L + kTM - 1) / kTM, tn = (N + kTN - 1) / kTN;
-    const dim3 g(tn < 65535 ? tn : 65535, tm < 65535 ? tm : 65535, batch < 65535 ? batch : 65535);
     const size_t slab = (size_t)L * inner;
-    k_dst<R><<<g, 256, 0, s>>>(S, src, dst, L, N, L, batch, 0, L, slab, N, slab, N);
+    dst_product<R>(S, src, dst, L, (int)inner, L, (int)outer, 0, L, slab, (int)inner, slab, (int)inner, s);
   }
 }
 
