@@ -172,7 +172,7 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP>::WARPS * ElemCfg<D, N
   __syncthreads();
 
   double accF = 0.0, accMin = INFINITY;
-  const int nwarps_total = gridDim.x * WARPS;
+  const int warps = blockDim.x / GT, nwarps_total = gridDim.x * warps;   // (small meshes: fewer than WARPS, launch_elem)
   // (the product from compact records, OP_HESS_PA_C, is pac_kernel in tmop_pa_compact.cu)
   constexpr bool PA_APPLY = OP == OP_HESS_PA;
   constexpr bool EG = OP == OP_ENERGY_GRAD;                // gradient + energy partials
@@ -186,7 +186,7 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP>::WARPS * ElemCfg<D, N
   static_assert(!FX || Cfg::NC * FxNodal<D, N>::CS <= Cfg::B0, "B0 too small for the padded nodal fields");
   NodeMap<N> nodes(p.elem_nodes, p.sx, p.sy, D == 3 ? N - 1 : 1);
   const int ecount = p.elist ? p.ecount : p.nelem;
-  for (int ei = blockIdx.x * WARPS + warp; ei < ecount; ei += nwarps_total) {
+  for (int ei = blockIdx.x * warps + warp; ei < ecount; ei += nwarps_total) {
     const int e = p.elist ? __ldg(p.elist + ei) : ei;
     nodes.element(e, NDOF);
     // Partially assembled product: the stored values of this lane's first
@@ -775,7 +775,7 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP>::WARPS * ElemCfg<D, N
     __syncthreads();
     if (threadIdx.x == 0) {
       double f = 0.0, m = INFINITY;
-      for (int w = 0; w < WARPS * G; ++w) { f += redF[w]; m = fmin(m, redM[w]); }
+      for (int w = 0; w < warps * G; ++w) { f += redF[w]; m = fmin(m, redM[w]); }
       p.part_F[blockIdx.x] = f;
       p.part_min[blockIdx.x] = m;
     }
@@ -786,7 +786,8 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP>::WARPS * ElemCfg<D, N
 template <int D, int N, int Q1, class R, int OP>
 int launch_elem(const KParams& p, int grid, void* stream) {
   using Cfg = ElemCfg<D, N, Q1, R, OP>;
-  elem_kernel<D, N, Q1, R, OP><<<grid, Cfg::WARPS * Cfg::G * 32, Cfg::smem_bytes(), (cudaStream_t)stream>>>(p);
+  const int w = (p.nelem + grid - 1) / grid, warps = w < Cfg::WARPS ? w : Cfg::WARPS;
+  elem_kernel<D, N, Q1, R, OP><<<grid, warps * Cfg::G * 32, Cfg::smem_bytes(), (cudaStream_t)stream>>>(p);
   return (int)cudaGetLastError();
 }
 
@@ -805,9 +806,17 @@ int prepare_elem_impl(int nelem, int* grid) {
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (per_sm < 1) return (int)cudaErrorInvalidConfiguration;
+  // Fewer full blocks than SMs: the elements are spread over all SMs in
+  // smaller blocks instead, since the warps of a block share one narrow FP64
+  // pipe.
   const int need = (nelem + Cfg::WARPS - 1) / Cfg::WARPS;
   const int full = per_sm * sms;
-  *grid = need < full ? need : full;
+  if (need < sms) {
+    const int w = (nelem + sms - 1) / sms;
+    *grid = (nelem + w - 1) / w;
+  } else {
+    *grid = need < full ? need : full;
+  }
   return 0;
 }
 

@@ -8,6 +8,7 @@
 // symmetric Hessian with the residual minimised through Givens rotations;
 // the scalar recurrences run on the device in a one-thread kernel, so a
 // step needs no host round trip. CG is the SPD alternative.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stddef.h>
@@ -65,15 +66,24 @@ __global__ void k_dot_part(const double* __restrict__ a, const double* __restric
   if (threadIdx.x == 0) part[blockIdx.x] = s;
 }
 
-// a . b over T vectors: each thread sums its elements in T (FP32 vectors:
-// ~30 elements per thread at full occupancy), the blocks in FP64
-template <class T>
-__global__ void k_dot_part_t(const T* __restrict__ a, const T* __restrict__ b, size_t n, double* __restrict__ part) {
-  T s = T(0);
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-    s = fma(a[i], b[i], s);
-  const double t = block_sum((double)s);
-  if (threadIdx.x == 0) part[blockIdx.x] = t;
+// Sum of the per-block partials by the block that finishes last (the same sum,
+// in the same order, as k_sum_final), which saves the launch of one more
+// kernel: true in all threads of that block, with the sum valid in thread 0.
+// counter: a zeroed slot of the state; atomicInc leaves it zero again.
+__device__ __forceinline__ bool last_block_sum(double v, double* part, int np, double* counter, double* sum) {
+  __shared__ bool last;
+  if (threadIdx.x == 0) {
+    part[blockIdx.x] = v;
+    __threadfence();
+    last = atomicInc(reinterpret_cast<unsigned*>(counter), gridDim.x - 1) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!last) return false;
+  __threadfence();
+  double s = 0.0;
+  for (int i = threadIdx.x; i < np; i += blockDim.x) s += __ldcg(part + i);
+  *sum = block_sum(s);
+  return true;
 }
 
 __global__ void k_sum_final(const double* __restrict__ part, int np, double* __restrict__ out) {
@@ -176,14 +186,30 @@ __global__ void k_minres_init(const double* __restrict__ b, T* v, T* vprev, T* A
   }
 }
 
+// st[KS_ALPHA] = a . b over T vectors: each thread sums its elements in T
+// (FP32 vectors: ~30 elements per thread at full occupancy), the blocks in FP64
+template <class T>
+__global__ void k_dot_alpha(const T* __restrict__ a, const T* __restrict__ b, size_t n, double* __restrict__ part,
+                            double* st) {
+  T s = T(0);
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
+    s = fma(a[i], b[i], s);
+  double sum;
+  if (last_block_sum(block_sum((double)s), part, gridDim.x, st + KS_COUNTER, &sum) && threadIdx.x == 0)
+    st[KS_ALPHA] = sum;
+}
+
+__device__ void minres_scalars(double* st, double beta_next2);
+
 // The next Lanczos vector, unnormalised, over Av, with per-block partials of
 // its squared norm. The arrays hold v / sv, vprev / svp and H (v / sv), so
 // H v - alpha v - beta vprev = sv Av - (alpha sv) v - (beta svp) vprev, and
 // alpha = v . H v = sv^2 (v array . Av) from the sum in st[KS_ALPHA]. vprev
 // is read here for the last time and zeroed: it is the next product's output.
+// The last block takes the scalar step.
 template <class T>
-__global__ void k_lanczos(T* __restrict__ Av, const T* __restrict__ v, T* __restrict__ vprev,
-                          const double* __restrict__ st, size_t n, double* __restrict__ part) {
+__global__ void k_lanczos(T* __restrict__ Av, const T* __restrict__ v, T* __restrict__ vprev, double* st, size_t n,
+                          double* __restrict__ part) {
   const double svd = st[KS_SV];
   const T sv = (T)svd, av = (T)(st[KS_ALPHA] * svd * svd * svd), bv = (T)(st[KS_BETA] * st[KS_SVP]);
   T s = T(0);
@@ -193,12 +219,20 @@ __global__ void k_lanczos(T* __restrict__ Av, const T* __restrict__ v, T* __rest
     vprev[i] = T(0);
     s = fma(r, r, s);
   }
-  const double t = block_sum((double)s);
-  if (threadIdx.x == 0) part[blockIdx.x] = t;
+  double sum;
+  if (last_block_sum(block_sum((double)s), part, gridDim.x, st + KS_COUNTER, &sum) && threadIdx.x == 0)
+    minres_scalars(st, sum);
 }
 
 // Apply the two previous rotations to the new tridiagonal column
 // (beta_k, alpha_k, beta_{k+1}), form the new rotation, update eta.
+// (All on one thread: what it costs is the chain of dependent FP64
+// operations, so square roots and quotients come from two independent
+// reciprocal square roots, 1 / beta and 1 / rho, instead of a square root, a
+// hypot and four divisions.)
+__device__ __forceinline__ double rsqrt_safe(double a) {   // 1 / sqrt(a), 0 for a = 0
+  return a > 0.0 ? rsqrt(a) : 0.0;
+}
 __device__ void minres_scalar_step(double* st) {
   if (st[KS_DONE] == 0.0 && st[KS_ITER] >= st[KS_MAXIT]) {  // the cap: freeze, not converged
     st[KS_DONE] = 1.0;
@@ -215,22 +249,28 @@ __device__ void minres_scalar_step(double* st) {
   }
   st[KS_ITER] += 1.0;
   const double beta = st[KS_BETA], alpha = st[KS_ALPHA] * st[KS_SV] * st[KS_SV];
-  const double beta_next = sqrt(fmax(st[KS_BETA_NEXT2], 0.0));
+  const double b2 = fmax(st[KS_BETA_NEXT2], 0.0);
   const double c_old = st[KS_C_OLD], s_old = st[KS_S_OLD], c = st[KS_C], s = st[KS_S];
   const double r1 = s_old * beta;
   const double tmp = c_old * beta;
   const double r2 = c * tmp + s * alpha;
   const double r3 = -s * tmp + c * alpha;
-  const double rho = hypot(r3, beta_next);
-  const double c_new = rho > 0.0 ? r3 / rho : 1.0, s_new = rho > 0.0 ? beta_next / rho : 0.0;
+  const double inv_bn = rsqrt_safe(b2), beta_next = b2 * inv_bn;
+  double inv_rho = rsqrt_safe(fma(r3, r3, b2));
+  if (!(fabs(r3) < 1e150 && (b2 > 1e-290 || fabs(r3) > 1e-145))) {   // squares near the ends of the range
+    const double rho = hypot(r3, beta_next);
+    inv_rho = rho > 0.0 ? 1.0 / rho : 0.0;
+  }
+  const bool zero = inv_rho == 0.0;
+  const double c_new = zero ? 1.0 : r3 * inv_rho, s_new = beta_next * inv_rho;
   const double eta = st[KS_ETA];
   st[KS_R1] = r1;
   st[KS_R2] = r2;
-  st[KS_INV_RHO] = rho > 0.0 ? 1.0 / rho : 0.0;
+  st[KS_INV_RHO] = inv_rho;
   st[KS_PHI] = c_new * eta;
   st[KS_ETA] = -s_new * eta;
   st[KS_RESID] = fabs(s_new * eta);
-  st[KS_INV_BETA_NEXT] = beta_next > 0.0 ? 1.0 / beta_next : 0.0;
+  st[KS_INV_BETA_NEXT] = inv_bn;
   st[KS_BETA_NEXT] = beta_next;
   st[KS_C_OLD] = c; st[KS_S_OLD] = s; st[KS_C] = c_new; st[KS_S] = s_new;
   st[KS_BETA] = beta_next;
@@ -240,14 +280,10 @@ __device__ void minres_scalar_step(double* st) {
   }
 }
 
-// one block: |next Lanczos vector|^2 from the Lanczos step's per-block
-// partials (the same sum as k_sum_final), then the scalar step in thread 0
-__global__ void k_minres_scalar(const double* __restrict__ part, int np, double* st) {
-  double sum = 0.0;
-  for (int i = threadIdx.x; i < np; i += blockDim.x) sum += part[i];
-  sum = block_sum(sum);
-  if (threadIdx.x != 0) return;
-  st[KS_BETA_NEXT2] = sum;
+// The scalar step from |next Lanczos vector|^2, and the scales and
+// coefficients of the passes after it.
+__device__ void minres_scalars(double* st, double beta_next2) {
+  st[KS_BETA_NEXT2] = beta_next2;
   minres_scalar_step(st);
   // scales of the unnormalised Lanczos vectors: the direction update takes v
   // at its present scale, then the arrays rotate and the next v is the new
@@ -297,18 +333,134 @@ __global__ void k_minres_vec_rot(const T* __restrict__ v, const T* __restrict__ 
   }
 }
 
+// ---------------------------------------------------------------- small problems
+// One cluster of blocks does all that follows a product: with few unknowns
+// an iteration is a chain of launches and reductions (2.5-7 us each for
+// microseconds of work), so the dot products are reduced through distributed
+// shared memory, in block order, and every block takes the scalar step itself
+// on a copy of the state in shared memory; block 0 writes it back after the
+// barrier behind which all blocks have read it.
+namespace cg = cooperative_groups;
+constexpr int kClBlocks = 8, kClPer = 4;
+constexpr size_t kClMax = (size_t)256 * kClBlocks * kClPer;   // unknowns: kClPer per thread of the larger form
+
+// sum over the cluster in a fixed order, to all threads; slot: [kClBlocks]
+// doubles of this call. (A shuffle and an FP64 add are ~110 cycles, so every
+// level is a tree.)
+template <int NT>
+__device__ __forceinline__ double cluster_sum(double v, double* slot, cg::cluster_group& cl) {
+  constexpr int W = NT / 32;
+  __shared__ double red[W];
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if (lane == 0) red[threadIdx.x >> 5] = v;
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    double s = lane < W ? red[lane] : 0.0;
+#pragma unroll
+    for (int o = (W > kClBlocks ? W : kClBlocks) / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane < kClBlocks) *cl.map_shared_rank(slot + cl.block_rank(), lane) = s;
+  }
+  cl.sync();
+  double s = slot[lane % kClBlocks];
+#pragma unroll
+  for (int o = kClBlocks / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  return s;
+}
+
+// the whole of a plain MINRES step after Av = H v (k_dot_part_t, k_lanczos,
+// k_minres_scalar and k_minres_vec_rot in one)
+template <class T, int NT>
+__global__ void __launch_bounds__(NT) k_minres_cluster(const T* __restrict__ v, T* __restrict__ vprev, T* __restrict__ Av,
+                                                       const T* __restrict__ w, T* __restrict__ wp,
+                                                       T* __restrict__ sol, double* st, int n) {
+  cg::cluster_group cl = cg::this_cluster();
+  __shared__ double sst[KS_COUNT];
+  __shared__ double slots[2][kClBlocks];
+  const int first = cl.block_rank() * NT + threadIdx.x;
+  constexpr int S = NT * kClBlocks;
+  // all that the step reads, at once: one trip to memory
+  T rv[kClPer], ra[kClPer], rp[kClPer], rw[kClPer], rwp[kClPer], rs[kClPer];
+#pragma unroll
+  for (int k = 0; k < kClPer; ++k) {
+    const int i = first + k * S;
+    const bool in = i < n;
+    rv[k] = in ? v[i] : T(0);
+    ra[k] = in ? Av[i] : T(0);
+    rp[k] = in ? vprev[i] : T(0);
+    rw[k] = in ? w[i] : T(0);
+    rwp[k] = in ? wp[i] : T(0);
+    rs[k] = in ? sol[i] : T(0);
+  }
+  if (threadIdx.x < KS_COUNT) sst[threadIdx.x] = st[threadIdx.x];
+  T a = T(0);
+#pragma unroll
+  for (int k = 0; k < kClPer; ++k)
+    if (first + k * S < n) a = fma(rv[k], ra[k], a);
+  const double alpha = cluster_sum<NT>((double)a, slots[0], cl);   // (its barriers cover sst too)
+  const double svd = sst[KS_SV];
+  const T sv = (T)svd, av = (T)(alpha * svd * svd * svd), bv = (T)(sst[KS_BETA] * sst[KS_SVP]);
+  T q = T(0);
+#pragma unroll
+  for (int k = 0; k < kClPer; ++k) {
+    const int i = first + k * S;
+    if (i >= n) break;
+    const T r = fma(sv, ra[k], -av * rv[k]) - bv * rp[k];
+    Av[i] = r;
+    vprev[i] = T(0);
+    q = fma(r, r, q);
+  }
+  const double b2 = cluster_sum<NT>((double)q, slots[1], cl);
+  if (threadIdx.x == 0) {
+    sst[KS_ALPHA] = alpha;
+    minres_scalars(sst, b2);
+  }
+  __syncthreads();
+  if (cl.block_rank() == 0 && threadIdx.x < KS_COUNT) st[threadIdx.x] = sst[threadIdx.x];
+  const T cu = (T)sst[KS_WU], cp = (T)sst[KS_WP], cw = (T)sst[KS_WW], phi = (T)sst[KS_PHI];
+#pragma unroll
+  for (int k = 0; k < kClPer; ++k) {
+    const int i = first + k * S;
+    if (i >= n) break;
+    const T wn = fma(-cw, rw[k], fma(-cp, rwp[k], rv[k] * cu));
+    wp[i] = wn;
+    sol[i] = fma(phi, wn, rs[k]);
+  }
+}
+
+template <class... P, class... A>
+int launch_cluster(void (*f)(P...), int threads, cudaStream_t s, A... a) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(kClBlocks);
+  cfg.blockDim = dim3(threads);
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = kClBlocks;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return (int)cudaLaunchKernelEx(&cfg, f, P(a)...);
+}
+
 template <class T>
 int minres_after_hv_rot(const T* v, T* vprev, T* Av, const T* w, T* wp, T* sol, double* st, double* part, size_t n,
                         cudaStream_t s, const double* vdot, int vdot_np) {
+  // (128 threads a block up to 2048 unknowns: with 4 warps instead of 8 to
+  // reduce, 12.4 against 14.1 us per iteration of 578 unknowns, product
+  // included; 20.3 us in separate kernels. 4802 unknowns: 16.1 against 24.4)
+  if (n <= 2048)
+    return launch_cluster(k_minres_cluster<T, 128>, 128, s, v, vprev, Av, w, wp, sol, st, (int)n);
+  if (n <= kClMax)
+    return launch_cluster(k_minres_cluster<T, 256>, 256, s, v, vprev, Av, w, wp, sol, st, (int)n);
   int g = red_grid(n);
   if (vdot) {  // alpha = v . (H v) from the product kernel's own partials
     k_sum_final<<<1, kThreads, 0, s>>>(vdot, vdot_np, st + KS_ALPHA);
   } else {
-    k_dot_part_t<T><<<g, kThreads, 0, s>>>(v, Av, n, part);
-    k_sum_final<<<1, kThreads, 0, s>>>(part, g, st + KS_ALPHA);
+    k_dot_alpha<T><<<g, kThreads, 0, s>>>(v, Av, n, part, st);
   }
   k_lanczos<T><<<g, kThreads, 0, s>>>(Av, v, vprev, st, n, part);
-  k_minres_scalar<<<1, kThreads, 0, s>>>(part, g, st);
   k_minres_vec_rot<T><<<g, kThreads, 0, s>>>(v, w, wp, sol, st, n);
   return (int)cudaGetLastError();
 }
@@ -366,53 +518,9 @@ __global__ void k_pm_init_scalar(double* st, double rtol, int maxit) {
   st[KS_BREAKDOWN] = 0.0;
 }
 
-// q <- q / beta - (beta / oldb) r1 (the r1 term from the second iteration
-// on), partials of u . q (alpha = their sum / beta)
-template <class T>
-__global__ void k_pm_a(T* __restrict__ q, const T* __restrict__ r1, const T* __restrict__ u,
-                       const double* __restrict__ st, size_t n, double* __restrict__ part) {
-  const double oldb = st[KS_OLDB];
-  const T ib = (T)st[KS_INV_BETA];
-  const T c = (T)(oldb > 0.0 ? st[KS_BETA] / oldb : 0.0);
-  T s = T(0);
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-    const T qi = fma(-c, r1[i], q[i] * ib);
-    q[i] = qi;
-    s = fma(u[i], qi, s);
-  }
-  const double t = block_sum((double)s);
-  if (threadIdx.x == 0) part[blockIdx.x] = t;
-}
-
-// out = (sum of the partials) * *scale
-__global__ void k_sum_scaled(const double* __restrict__ part, int np, const double* __restrict__ scale,
-                             double* __restrict__ out) {
-  double s = 0.0;
-  for (int i = threadIdx.x; i < np; i += blockDim.x) s += part[i];
-  s = block_sum(s);
-  if (threadIdx.x == 0) *out = s * *scale;
-}
-
-// t = q - (alpha / beta) r2 into r1's buffer (the old r1 is dead), then
-// q <- M^-1 t (diagonal part); partials of t . q
-template <class T>
-__global__ void k_pm_b(const T* __restrict__ minv, T* __restrict__ r1, const T* __restrict__ r2, T* __restrict__ q,
-                       const double* __restrict__ st, size_t n, double* __restrict__ part) {
-  const double beta = st[KS_BETA];
-  const T c = (T)(beta > 0.0 ? st[KS_ALPHA] / beta : 0.0);
-  T s = T(0);
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-    const T t = fma(-c, r2[i], q[i]);
-    r1[i] = t;
-    const T yi = minv[i] * t;
-    q[i] = yi;
-    s = fma(t, yi, s);
-  }
-  const double tt = block_sum((double)s);
-  if (threadIdx.x == 0) part[blockIdx.x] = tt;
-}
-
-__global__ void k_pm_scalar(double* st) {
+// (square roots and quotients from two independent reciprocal square roots, as
+// in minres_scalar_step)
+__device__ void pm_scalars(double* st) {
   if (st[KS_DONE] == 0.0 && st[KS_ITER] >= st[KS_MAXIT]) {
     st[KS_DONE] = 1.0;
     st[KS_HITMAX] = 1.0;
@@ -429,7 +537,7 @@ __global__ void k_pm_scalar(double* st) {
   st[KS_INV_BETA_OLD] = st[KS_INV_BETA];   // the direction update reads this iteration's v = u / beta
   st[KS_ITER] += 1.0;
   const double alpha = st[KS_ALPHA];
-  const double beta = sqrt(fmax(st[KS_BETA_NEXT2], 0.0));
+  const double b2 = fmax(st[KS_BETA_NEXT2], 0.0), inv_beta = rsqrt_safe(b2), beta = b2 * inv_beta;
   st[KS_OLDB] = st[KS_BETA];
   st[KS_BETA] = beta;
   const double cs = st[KS_CS], sn = st[KS_SN], dbar = st[KS_DBAR];
@@ -438,23 +546,84 @@ __global__ void k_pm_scalar(double* st) {
   const double gbar = sn * dbar - cs * alpha;
   st[KS_EPSLN] = sn * beta;
   st[KS_DBAR] = -cs * beta;
-  double gamma = hypot(gbar, beta);
-  if (!(gamma > 0.0)) gamma = 1e-300;
-  const double cs_new = gbar / gamma, sn_new = beta / gamma;
+  double inv_gamma = rsqrt_safe(fma(gbar, gbar, b2));
+  if (!(fabs(gbar) < 1e150 && (b2 > 1e-290 || fabs(gbar) > 1e-145))) {   // squares near the ends of the range
+    const double gamma = hypot(gbar, beta);
+    inv_gamma = gamma > 0.0 ? 1.0 / gamma : 1e300;
+  }
+  const double cs_new = gbar * inv_gamma, sn_new = beta * inv_gamma;
   st[KS_CS] = cs_new;
   st[KS_SN] = sn_new;
   const double phibar = st[KS_PHIBAR];
   st[KS_PHI] = cs_new * phibar;
   st[KS_PHIBAR] = sn_new * phibar;
   st[KS_RESID] = fabs(sn_new * phibar);
-  st[KS_INV_GAMMA] = 1.0 / gamma;
-  st[KS_WU] = st[KS_INV_BETA_OLD] / gamma;
-  st[KS_WP] = st[KS_OLDEPS] / gamma;
-  st[KS_WW] = st[KS_DELTA] / gamma;
-  st[KS_INV_BETA] = beta > 0.0 ? 1.0 / beta : 0.0;
+  st[KS_INV_GAMMA] = inv_gamma;
+  st[KS_WU] = st[KS_INV_BETA_OLD] * inv_gamma;
+  st[KS_WP] = st[KS_OLDEPS] * inv_gamma;
+  st[KS_WW] = st[KS_DELTA] * inv_gamma;
+  st[KS_INV_BETA] = inv_beta;
   if (fabs(sn_new * phibar) <= st[KS_TOL] || beta == 0.0) {
     st[KS_DONE] = 1.0;
     st[KS_CONV_IT] = st[KS_ITER];
+  }
+}
+
+// q <- q / beta - (beta / oldb) r1 (the r1 term from the second iteration
+// on); alpha = u . q / beta from the last block
+template <class T>
+__global__ void k_pm_a(T* __restrict__ q, const T* __restrict__ r1, const T* __restrict__ u, double* st, size_t n,
+                       double* __restrict__ part) {
+  const double oldb = st[KS_OLDB];
+  const T ib = (T)st[KS_INV_BETA];
+  const T c = (T)(oldb > 0.0 ? st[KS_BETA] / oldb : 0.0);
+  T s = T(0);
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+    const T qi = fma(-c, r1[i], q[i] * ib);
+    q[i] = qi;
+    s = fma(u[i], qi, s);
+  }
+  double sum;
+  if (last_block_sum(block_sum((double)s), part, gridDim.x, st + KS_COUNTER, &sum) && threadIdx.x == 0)
+    st[KS_ALPHA] = sum * st[KS_INV_BETA];
+}
+
+// t = q - (alpha / beta) r2 into r1's buffer (the old r1 is dead), then
+// q <- M^-1 t (diagonal part); partials of t . q. Without a further part of
+// the preconditioner (SCALARS) the last block takes the scalar step.
+template <class T, bool SCALARS>
+__global__ void k_pm_b(const T* __restrict__ minv, T* __restrict__ r1, const T* __restrict__ r2, T* __restrict__ q,
+                       double* st, size_t n, double* __restrict__ part) {
+  const double beta = st[KS_BETA];
+  const T c = (T)(beta > 0.0 ? st[KS_ALPHA] / beta : 0.0);
+  T s = T(0);
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+    const T t = fma(-c, r2[i], q[i]);
+    r1[i] = t;
+    const T yi = minv[i] * t;
+    q[i] = yi;
+    s = fma(t, yi, s);
+  }
+  const double tt = block_sum((double)s);
+  if constexpr (SCALARS) {
+    double sum;
+    if (last_block_sum(tt, part, gridDim.x, st + KS_COUNTER, &sum) && threadIdx.x == 0) {
+      st[KS_BETA_NEXT2] = sum;
+      pm_scalars(st);
+    }
+  } else if (threadIdx.x == 0) {
+    part[blockIdx.x] = tt;
+  }
+}
+
+// the scalar step from the partials of the diagonal and the coarse part
+__global__ void k_pm_scalar(const double* __restrict__ part, int np, double* st) {
+  double s = 0.0;
+  for (int i = threadIdx.x; i < np; i += blockDim.x) s += part[i];
+  s = block_sum(s);
+  if (threadIdx.x == 0) {
+    st[KS_BETA_NEXT2] = s;
+    pm_scalars(st);
   }
 }
 
@@ -500,16 +669,14 @@ int pminres_after_hv(const T* minv, T* r1, const T* r2, T* u, T* q, const T* w, 
                      double* part, size_t n, cudaStream_t s, const PrecondAdd* pc) {
   const int g = red_grid(n);
   k_pm_a<T><<<g, kThreads, 0, s>>>(q, r1, u, st, n, part);
-  k_sum_scaled<<<1, kThreads, 0, s>>>(part, g, st + KS_INV_BETA, st + KS_ALPHA);
-  int g2 = g;
-  k_pm_b<T><<<g, kThreads, 0, s>>>(minv, r1, r2, q, st, n, part);
   if (pc) {   // q += C t (t now in r1's buffer), and the partials of t . C t after the diagonal part's
+    k_pm_b<T, false><<<g, kThreads, 0, s>>>(minv, r1, r2, q, st, n, part);
     const int np = pc->apply_t(pc->obj, r1, q, part + g, s);
     if (np < 0) return (int)cudaErrorLaunchFailure;
-    g2 += np;
+    k_pm_scalar<<<1, kThreads, 0, s>>>(part, g + np, st);
+  } else {
+    k_pm_b<T, true><<<g, kThreads, 0, s>>>(minv, r1, r2, q, st, n, part);
   }
-  k_sum_final<<<1, kThreads, 0, s>>>(part, g2, st + KS_BETA_NEXT2);
-  k_pm_scalar<<<1, 1, 0, s>>>(st);
   k_pm_w<T><<<g, kThreads, 0, s>>>(u, w, wprev, sol, st, n);
   return (int)cudaGetLastError();
 }

@@ -27,6 +27,7 @@ enum {
   // preconditioned MINRES
   KS_OLDB, KS_DBAR, KS_EPSLN, KS_OLDEPS, KS_PHIBAR, KS_CS, KS_SN, KS_DELTA, KS_INV_GAMMA, KS_INV_BETA,
   KS_INV_BETA_OLD, KS_WU, KS_WP, KS_WW,   // direction update coefficients of v (u), w_{k-2}, w_{k-1}
+  KS_COUNTER,   // zero between kernels (an unsigned counter of finished blocks in its first bytes)
   KS_COUNT
 };
 
