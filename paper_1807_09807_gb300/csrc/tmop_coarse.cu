@@ -156,16 +156,19 @@ __device__ __forceinline__ double block_sum_c(double v) {
 // B(k, j) = B[b sBb + k ldb + j], C(i, j) = C[b sCb + i ldc + j]: along x
 // (inner = 1) In [rows][L] times S (symmetric), along y or z S times every
 // [L][inner] slab. Output tiles of T x T over KC-deep chunks staged in shared
-// memory, P x P outputs per thread (rows ty + (T/P) r, columns tx + (T/P) c).
-template <class R, int T, int P, int KC>
-__global__ void __launch_bounds__((T / P) * (T / P)) k_dst(const R* __restrict__ A, const R* __restrict__ B,
-                                                           R* __restrict__ C, int M, int N, int Kd, int batch,
-                                                           size_t sAb, int lda, size_t sBb, int ldb, size_t sCb,
-                                                           int ldc) {
-  constexpr int W = T / P, NT = W * W;
+// memory, P x P outputs per thread (rows ty + (T/P) r, columns tx + (T/P) c);
+// the terms of a chunk are split over KS groups of threads, whose sums are
+// added at the end (small tiles: a thread's chain of FP64 multiply-adds, 66
+// cycles each, and its loads are then a quarter as long).
+template <class R, int T, int P, int KC, int KS>
+__global__ void __launch_bounds__((T / P) * (T / P) * KS) k_dst(const R* __restrict__ A, const R* __restrict__ B,
+                                                                R* __restrict__ C, int M, int N, int Kd, int batch,
+                                                                size_t sAb, int lda, size_t sBb, int ldb, size_t sCb,
+                                                                int ldc) {
+  constexpr int W = T / P, NT = W * W * KS, KL = KC / KS;
   __shared__ R As[KC][T + 1];
   __shared__ R Bs[KC][T];
-  const int tid = threadIdx.x, tx = tid % W, ty = tid / W;
+  const int tid = threadIdx.x, tx = tid % W, ty = tid / W % W, ks = tid / (W * W);
   const int tiles_n = (N + T - 1) / T, tiles_m = (M + T - 1) / T;
   for (int b = blockIdx.z; b < batch; b += gridDim.z)
     for (int tm = blockIdx.y; tm < tiles_m; tm += gridDim.y)
@@ -179,16 +182,26 @@ __global__ void __launch_bounds__((T / P) * (T / P)) k_dst(const R* __restrict__
 #pragma unroll
           for (int c = 0; c < P; ++c) acc[r][c] = R(0);
         for (int k0 = 0; k0 < Kd; k0 += KC) {
+          // (all loads before the first store: one trip to memory)
+          constexpr int LD = KC * T / NT;
+          R la[LD], lb[LD];
 #pragma unroll
-          for (int q = tid; q < KC * T; q += NT) {
-            const int i = q / KC, k = q % KC;   // A tile: consecutive k per row
-            As[k][i] = (i0 + i < M && k0 + k < Kd) ? Ab[(size_t)(i0 + i) * lda + k0 + k] : R(0);
-            const int kb = q / T, j = q % T;    // B tile: consecutive j per row
-            Bs[kb][j] = (k0 + kb < Kd && j0 + j < N) ? Bb[(size_t)(k0 + kb) * ldb + j0 + j] : R(0);
+          for (int l = 0; l < LD; ++l) {
+            const int q = tid + l * NT, i = q / KC, k = q % KC;   // A tile: consecutive k per row
+            la[l] = (i0 + i < M && k0 + k < Kd) ? Ab[(size_t)(i0 + i) * lda + k0 + k] : R(0);
+            const int kb = q / T, j = q % T;                      // B tile: consecutive j per row
+            lb[l] = (k0 + kb < Kd && j0 + j < N) ? Bb[(size_t)(k0 + kb) * ldb + j0 + j] : R(0);
+          }
+#pragma unroll
+          for (int l = 0; l < LD; ++l) {
+            const int q = tid + l * NT;
+            As[q % KC][q / KC] = la[l];
+            Bs[q / T][q % T] = lb[l];
           }
           __syncthreads();
-#pragma unroll 16
-          for (int k = 0; k < KC; ++k) {
+#pragma unroll
+          for (int kk = 0; kk < KL; ++kk) {
+            const int k = ks * KL + kk;
             R a[P], bb[P];
 #pragma unroll
             for (int r = 0; r < P; ++r) a[r] = As[k][ty + W * r];
@@ -201,23 +214,33 @@ __global__ void __launch_bounds__((T / P) * (T / P)) k_dst(const R* __restrict__
           }
           __syncthreads();
         }
+        if constexpr (KS > 1) {   // (one output per thread) the groups' sums, through the A tile
+          static_assert(KS == 1 || (P == 1 && KS == 4 && KC * T >= 4 * T * T), "split sums");
+          R* red = &As[0][0];
+          red[tid] = acc[0][0];
+          __syncthreads();
+          if (ks == 0) acc[0][0] = (acc[0][0] + red[tid + W * W]) + (red[tid + 2 * W * W] + red[tid + 3 * W * W]);
+          __syncthreads();
+        }
         R* Cb = C + b * sCb;
+        if (ks == 0) {
 #pragma unroll
-        for (int r = 0; r < P; ++r)
+          for (int r = 0; r < P; ++r)
 #pragma unroll
-          for (int c = 0; c < P; ++c) {
-            const int i = i0 + ty + W * r, j = j0 + tx + W * c;
-            if (i < M && j < N) Cb[(size_t)i * ldc + j] = acc[r][c];
-          }
+            for (int c = 0; c < P; ++c) {
+              const int i = i0 + ty + W * r, j = j0 + tx + W * c;
+              if (i < M && j < N) Cb[(size_t)i * ldc + j] = acc[r][c];
+            }
+        }
       }
 }
 
-template <class R, int T, int P, int KC>
+template <class R, int T, int P, int KC, int KS>
 void launch_dst(const R* A, const R* B, R* C, int M, int N, int Kd, int batch, size_t sAb, int lda, size_t sBb,
                 int ldb, size_t sCb, int ldc, cudaStream_t s) {
   const int tm = (M + T - 1) / T, tn = (N + T - 1) / T;
   const dim3 g(tn < 65535 ? tn : 65535, tm < 65535 ? tm : 65535, batch < 65535 ? batch : 65535);
-  k_dst<R, T, P, KC><<<g, (T / P) * (T / P), 0, s>>>(A, B, C, M, N, Kd, batch, sAb, lda, sBb, ldb, sCb, ldc);
+  k_dst<R, T, P, KC, KS><<<g, (T / P) * (T / P) * KS, 0, s>>>(A, B, C, M, N, Kd, batch, sAb, lda, sBb, ldb, sCb, ldc);
 }
 
 // The tile by the number of 64 x 64 tiles. With 60 or more of them (47^3
@@ -225,15 +248,16 @@ void launch_dst(const R* A, const R* B, R* C, int M, int N, int Kd, int batch, s
 // win: two-level FP32 Newton on 48^3 order-3 hexes 89.6 ms against 92.3 ms
 // with 32 tiles. A small coarse grid leaves one or two 64 tiles, i.e. one or
 // two of 152 SMs, whose FP64 pipe (2 operations per clock) then bounds the
-// transform: 63^2 vertices, FP64, 71 us; with 16 tiles (32 blocks) 4 us, and
-// the two-level FP64 Newton solve on 64^2 order-3 quads takes 22.8 ms instead
-// of 110 ms.
+// transform: 63^2 vertices, FP64, 71 us. 8 tiles (128 blocks) of four thread
+// groups take 2.4 us, and one iteration of the two-level FP64 solve on 64^2
+// order-3 quads, which has four transforms, 49 us (65 us with 16 tiles of one
+// thread per output).
 template <class R>
 void dst_product(const R* A, const R* B, R* C, int M, int N, int Kd, int batch, size_t sAb, int lda, size_t sBb,
                  int ldb, size_t sCb, int ldc, cudaStream_t s) {
   const double tiles = ceil(M / 64.0) * ceil(N / 64.0) * batch;
-  if (tiles >= 60) launch_dst<R, 64, 4, 16>(A, B, C, M, N, Kd, batch, sAb, lda, sBb, ldb, sCb, ldc, s);
-  else launch_dst<R, 16, 1, 64>(A, B, C, M, N, Kd, batch, sAb, lda, sBb, ldb, sCb, ldc, s);
+  if (tiles >= 60) launch_dst<R, 64, 4, 16, 1>(A, B, C, M, N, Kd, batch, sAb, lda, sBb, ldb, sCb, ldc, s);
+  else launch_dst<R, 8, 1, 32, 4>(A, B, C, M, N, Kd, batch, sAb, lda, sBb, ldb, sCb, ldc, s);
 }
 
 // divide by alpha times the eigenvalue of K_c at every coarse point, in the

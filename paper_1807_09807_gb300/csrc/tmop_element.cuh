@@ -41,7 +41,7 @@ constexpr int round16(int words) {
   return ((words * (int)sizeof(R) + 15) / 16) * 16 / (int)sizeof(R);
 }
 
-template <int D, int N, int Q1, class R, int OP>
+template <int D, int N, int Q1, class R, int OP, bool WIDE = false>
 struct ElemCfg {
   // 3D Hessian action: x and v are contracted one after the other and only
   // A(x) is kept (buffer B2) while v runs through the stage buffers, so the
@@ -54,27 +54,35 @@ struct ElemCfg {
   static constexpr int B1 = round16<R>(Buf<D, N, Q1, NC>::B1);
   static constexpr int B2 = SPLIT ? round16<R>(D * D * Shape<D, N, Q1>::QP) : 0;
   static constexpr int PER_WARP = (int)sizeof(R) * (B0 + B1 + B2);
-  // Warps per element. The FP64 3D kernels with 4 or more points per
+  // Threads per element. The FP64 3D kernels with 4 or more points per
   // direction run two warps on an element, in a block of its own, as many
   // blocks per SM as shared memory holds: the contractions run on the integer
   // pipes beside the FP64 pipe, and with one warp per element only 2-3 warps
   // per scheduler hide their latency (48^3 order-3 hexes, gradient + Hessian
   // action: 8.30 ms with one warp, 6.87 ms with two, 5.53 ms with one copy of
   // the forward map's code for x and v, which took the misses of the
-  // instruction cache down).
+  // instruction cache down). In 2D a stage has 6 to 24 lines, one per thread:
+  // on meshes that fill the chip (WIDE) half a warp per element leaves fewer
+  // of them idle (150 x 117 order-4 quads, 6^2 points, gradient + Hessian
+  // action: 266 us with a warp, 195 us with half, 197 us with a quarter); on
+  // small ones, where an element's latency counts, a warp is faster (8^2
+  // order-2 quads, Newton: 5.22 against 5.51 ms).
   static constexpr bool FX3 = D == 3 && sizeof(R) == 8;
-  static constexpr int G = (FX3 && Q1 >= 4 && OP != OP_ENERGY && OP != OP_LINEARIZE) ? 2 : 1;
+  static constexpr bool HAS_WIDE = D == 2 && sizeof(R) == 8 && OP != OP_ENERGY;
+  static constexpr int GT = (HAS_WIDE && WIDE) ? 16
+                            : (FX3 && Q1 >= 4 && OP != OP_ENERGY && OP != OP_LINEARIZE) ? 64
+                                                                                       : 32;
   // Elements in flight per block: up to 8 within ~200 KB of shared memory;
   // the FP64 3D energy as two blocks of 6 per SM where they fit
   static constexpr bool TWO = FX3 && OP == OP_ENERGY && 12 * PER_WARP <= 200 * 1024;
   static constexpr int FIT = 200 * 1024 / PER_WARP;
-  static constexpr int WARPS = G == 2 ? 1 : (TWO ? 6 : (FIT >= 8 ? 8 : (FIT < 1 ? 1 : FIT)));
+  static constexpr int WARPS = GT == 64 ? 1 : (TWO ? 6 : (FIT >= 8 ? 8 : (FIT < 1 ? 1 : FIT)));
   // blocks per SM that bound the registers (0: no bound): 8 (128 registers),
   // 10 (96) for the gradient, whose pointwise stage needs fewer (32^3 order-2
   // hexes, mu302: 422 us with 8, 392 us with 10; the stored-Hessian product
   // 211 us with 8, 223 us with 12)
   static constexpr int WANT = (OP == OP_GRADIENT || OP == OP_ENERGY_GRAD) ? 10 : 8;
-  static constexpr int MINB = G == 2 ? (FIT >= WANT ? WANT : FIT) : (TWO ? 2 : 0);
+  static constexpr int MINB = GT == 64 ? (FIT >= WANT ? WANT : FIT) : (TWO ? 2 : 0);
   // after the 1D tables: the product weight w_q0 w_q1 (w_q2) of every point
   static constexpr int WQ_OFF = 2 * kMaxQ * kMaxN + kMaxQ;
   static constexpr int TABLE = round16<R>(WQ_OFF + Shape<D, N, Q1>::QP);
@@ -120,13 +128,13 @@ __device__ __forceinline__ bool metric_dP(int id, const R* T, const R* dT, R* S)
   return ok;
 }
 
-template <int D, int N, int Q1, class R, int OP>
-__global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP>::WARPS * ElemCfg<D, N, Q1, R, OP>::G * 32,
-                                  ElemCfg<D, N, Q1, R, OP>::MINB)
+template <int D, int N, int Q1, class R, int OP, bool WIDE>
+__global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP, WIDE>::WARPS * ElemCfg<D, N, Q1, R, OP, WIDE>::GT,
+                                  ElemCfg<D, N, Q1, R, OP, WIDE>::MINB)
     elem_kernel(const KParams p) {
-  using Cfg = ElemCfg<D, N, Q1, R, OP>;
+  using Cfg = ElemCfg<D, N, Q1, R, OP, WIDE>;
   constexpr int NDOF = Shape<D, N, Q1>::NDOF, QP = Shape<D, N, Q1>::QP, DD = D * D;
-  constexpr int WARPS = Cfg::WARPS, G = Cfg::G, GT = 32 * G;   // elements per block, warps and threads per element
+  constexpr int WARPS = Cfg::WARPS, GT = Cfg::GT;   // elements per block, threads per element
   extern __shared__ __align__(16) unsigned char smem_raw[];
   R* sB = reinterpret_cast<R*>(smem_raw);
   R* sG = sB + kMaxQ * kMaxN;
@@ -155,7 +163,8 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP>::WARPS * ElemCfg<D, N
     if constexpr (D == 3) w *= R(p.w1[t / (Q1 * Q1)]);
     sWq[t] = w;
   }
-  __shared__ unsigned s_mag[WARPS][G * 2 * D];   // per warp and component: largest magnitudes of the group's warps
+  constexpr int GW = GT > 32 ? GT / 32 : 1;   // warps per element
+  __shared__ unsigned s_mag[WARPS][GW * 2 * D];   // per warp and component: largest magnitudes of the group's warps
   R Wi[DD];
 #pragma unroll
   for (int i = 0; i < DD; ++i) Wi[i] = R(p.Winv[i]);
@@ -260,7 +269,7 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP>::WARPS * ElemCfg<D, N
       }
     }
     int em[FX ? Cfg::NC : 1];
-    if constexpr (FX) fx_group_exp<G, Cfg::NC>(mag, em, s_mag[warp], bar);
+    if constexpr (FX) fx_group_exp<GT, Cfg::NC>(mag, em, s_mag[warp], bar);
     else __syncwarp();
     // ---- forward contraction: A (and dA) at every point
     if constexpr (Cfg::SPLIT && FX) {
@@ -268,7 +277,7 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP>::WARPS * ElemCfg<D, N
       // P1, by one copy of the code
 #pragma unroll 1
       for (int f = 0;; ++f) {
-        fwd3_fx<N, Q1, D, G>(p.fx, em, P0, f == 0 ? P2 : P1, lane, bar);
+        fwd3_fx<N, Q1, D, GT>(p.fx, em, P0, f == 0 ? P2 : P1, lane, bar);
         if (f) break;
 #pragma unroll
         for (int c = 0; c < D; ++c) mag[c] = 0;
@@ -282,7 +291,7 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP>::WARPS * ElemCfg<D, N
             mag[c] = max(mag[c], fx_mag(vpre[k * D + c]));
           }
         }
-        fx_group_exp<G, D>(mag, em, s_mag[warp], bar);
+        fx_group_exp<GT, D>(mag, em, s_mag[warp], bar);
       }
     } else if constexpr (Cfg::SPLIT) {
       fwd3_rb<N, Q1, D, R>(tB, tG, P0, P2, lane);
@@ -298,10 +307,10 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP>::WARPS * ElemCfg<D, N
       __syncwarp();
       fwd3_rb<N, Q1, D, R>(tB, tG, P0, P1, lane);
     } else if constexpr (D == 2) {
-      if constexpr (FX) fwd2_fx<N, Q1, Cfg::NC, G>(p.fx, em, P0, P1, lane, bar);
+      if constexpr (FX) fwd2_fx<N, Q1, Cfg::NC, GT>(p.fx, em, P0, P1, lane, bar);
       else fwd2<N, Q1, Cfg::NC, R>(sB, sG, P0, P1, lane);
     } else {
-      if constexpr (FX) fwd3_fx<N, Q1, Cfg::NC, G>(p.fx, em, P0, P1, lane, bar);
+      if constexpr (FX) fwd3_fx<N, Q1, Cfg::NC, GT>(p.fx, em, P0, P1, lane, bar);
       else fwd3_rb<N, Q1, Cfg::NC, R>(tB, tG, P0, P1, lane);
     }
     R* Abuf = Cfg::SPLIT ? P2 : ((D == 2) ? P0 : P1);     // A: [D][D][QP]
@@ -681,12 +690,13 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP>::WARPS * ElemCfg<D, N
       }
     }
     if constexpr (OP == OP_LINEARIZE || OP == OP_LINEARIZE_C) {
-      __syncwarp();
+      group_sync<GT>(bar);
     } else if constexpr (OP == OP_ENERGY) {
       accMin = fmin(accMin, emin);
       if (p.elem_min) {
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) emin = fmin(emin, __shfl_xor_sync(0xffffffffu, emin, o));
+        for (int o = (GT < 32 ? GT : 32) / 2; o > 0; o >>= 1)
+          emin = fmin(emin, __shfl_xor_sync(group_mask<GT>(), emin, o));
         if (lane == 0) p.elem_min[e] = emin;
       }
     } else if constexpr (OP == OP_GRAD_HESS) {
@@ -697,8 +707,8 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP>::WARPS * ElemCfg<D, N
       if constexpr (D == 2) {
         // P0 holds the gradient's fields (in place of A), then the Hessian action's (dA)
         int er[2 * D];
-        fx_group_exp<G, 2 * D>(rmag, er, s_mag[warp], bar);
-        adj2_fx<N, Q1, 2 * D, G>(p.fx, er, P0, P1, lane, bar);
+        fx_group_exp<GT, 2 * D>(rmag, er, s_mag[warp], bar);
+        adj2_fx<N, Q1, 2 * D, GT>(p.fx, er, P0, P1, lane, bar);
         for (int t = lane; t < NDOF; t += GT) {
           const int gn = nodes(t);
 #pragma unroll
@@ -711,7 +721,7 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP>::WARPS * ElemCfg<D, N
         }
       } else {
         int er2[2 * D];
-        fx_group_exp<G, 2 * D>(rmag, er2, s_mag[warp], bar);
+        fx_group_exp<GT, 2 * D>(rmag, er2, s_mag[warp], bar);
 #pragma unroll 1
         for (int pass = 0; pass < 2; ++pass) {
           R* Rin = pass == 0 ? P1 : P2;
@@ -719,7 +729,7 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP>::WARPS * ElemCfg<D, N
           int er[D];
 #pragma unroll
           for (int c = 0; c < D; ++c) er[c] = pass == 0 ? er2[D + c] : er2[c];
-          adj3_fx<N, Q1, D, G>(p.fx, er, P0, Rin, lane, bar);
+          adj3_fx<N, Q1, D, GT>(p.fx, er, P0, Rin, lane, bar);
           for (int t = lane; t < NDOF; t += GT) {
             const int gn = nodes(t);
 #pragma unroll
@@ -729,7 +739,7 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP>::WARPS * ElemCfg<D, N
               atomicAdd(out + dof, P0[nodal(c, t)]);
             }
           }
-          group_sync<G>(bar);
+          group_sync<GT>(bar);
         }
       }
     } else {
@@ -737,9 +747,9 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP>::WARPS * ElemCfg<D, N
       // ---- adjoint contraction and scatter
       if constexpr (FX) {
         int er[D];
-        fx_group_exp<G, D>(rmag, er, s_mag[warp], bar);
-        if constexpr (D == 2) adj2_fx<N, Q1, D, G>(p.fx, er, P0, P1, lane, bar);
-        else adj3_fx<N, Q1, D, G>(p.fx, er, P0, P1, lane, bar);
+        fx_group_exp<GT, D>(rmag, er, s_mag[warp], bar);
+        if constexpr (D == 2) adj2_fx<N, Q1, D, GT>(p.fx, er, P0, P1, lane, bar);
+        else adj3_fx<N, Q1, D, GT>(p.fx, er, P0, P1, lane, bar);
       } else if constexpr (D == 2) {
         __syncwarp();
         adj2<N, Q1, D, R>(sB, sG, P0, P1, lane);
@@ -761,11 +771,12 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP>::WARPS * ElemCfg<D, N
         }
       }
     }
-    group_sync<G>(bar);
+    group_sync<GT>(bar);
   }
 
   if constexpr (OP == OP_ENERGY || EG) {
-    __shared__ double redF[WARPS * G], redM[WARPS * G];
+    constexpr int BW = (WARPS * GT + 31) / 32;
+    __shared__ double redF[BW], redM[BW];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
       accF += __shfl_xor_sync(0xffffffffu, accF, o);
@@ -775,7 +786,7 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP>::WARPS * ElemCfg<D, N
     __syncthreads();
     if (threadIdx.x == 0) {
       double f = 0.0, m = INFINITY;
-      for (int w = 0; w < warps * G; ++w) { f += redF[w]; m = fmin(m, redM[w]); }
+      for (int w = 0; w < (int)(blockDim.x / 32); ++w) { f += redF[w]; m = fmin(m, redM[w]); }
       p.part_F[blockIdx.x] = f;
       p.part_min[blockIdx.x] = m;
     }
@@ -783,25 +794,24 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP>::WARPS * ElemCfg<D, N
 }
 
 // Host-side launcher for one instantiation.
-template <int D, int N, int Q1, class R, int OP>
-int launch_elem(const KParams& p, int grid, void* stream) {
-  using Cfg = ElemCfg<D, N, Q1, R, OP>;
-  const int w = (p.nelem + grid - 1) / grid, warps = w < Cfg::WARPS ? w : Cfg::WARPS;
-  elem_kernel<D, N, Q1, R, OP><<<grid, warps * Cfg::G * 32, Cfg::smem_bytes(), (cudaStream_t)stream>>>(p);
+template <int D, int N, int Q1, class R, int OP, bool WIDE>
+int launch_elem_impl(const KParams& p, int grid, void* stream) {
+  using Cfg = ElemCfg<D, N, Q1, R, OP, WIDE>;
+  const int w = (p.nelem + grid - 1) / grid, threads = ((w < Cfg::WARPS ? w : Cfg::WARPS) * Cfg::GT + 31) / 32 * 32;
+  elem_kernel<D, N, Q1, R, OP, WIDE><<<grid, threads, Cfg::smem_bytes(), (cudaStream_t)stream>>>(p);
   return (int)cudaGetLastError();
 }
 
 // Occupancy-derived grid size, and the opt-in for > 48 KB of shared memory.
-template <int D, int N, int Q1, class R, int OP>
+template <int D, int N, int Q1, class R, int OP, bool WIDE>
 int prepare_elem_impl(int nelem, int* grid) {
-  using Cfg = ElemCfg<D, N, Q1, R, OP>;
+  using Cfg = ElemCfg<D, N, Q1, R, OP, WIDE>;
   const size_t smem = Cfg::smem_bytes();
-  cudaError_t err = cudaFuncSetAttribute((const void*)elem_kernel<D, N, Q1, R, OP>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const void* f = (const void*)elem_kernel<D, N, Q1, R, OP, WIDE>;
+  cudaError_t err = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (err != cudaSuccess) return (int)err;
   int per_sm = 0, dev = 0, sms = 0;
-  err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, (const void*)elem_kernel<D, N, Q1, R, OP>,
-                                                      Cfg::WARPS * Cfg::G * 32, smem);
+  err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, f, Cfg::WARPS * Cfg::GT, smem);
   if (err != cudaSuccess) return (int)err;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -820,9 +830,24 @@ int prepare_elem_impl(int nelem, int* grid) {
   return 0;
 }
 
+// The WIDE form where it exists and every SM has a full block (8 elements).
+template <int D, int N, int Q1, class R, int OP>
+bool use_wide(int nelem) {
+  return ElemCfg<D, N, Q1, R, OP>::HAS_WIDE && nelem >= 1216;
+}
+
+template <int D, int N, int Q1, class R, int OP>
+int launch_elem(const KParams& p, int grid, void* stream) {
+  constexpr bool W = ElemCfg<D, N, Q1, R, OP>::HAS_WIDE;
+  return use_wide<D, N, Q1, R, OP>(p.nelem) ? launch_elem_impl<D, N, Q1, R, OP, W>(p, grid, stream)
+                                            : launch_elem_impl<D, N, Q1, R, OP, false>(p, grid, stream);
+}
+
 template <int D, int N, int Q1, class R, int OP>
 int prepare_elem(int nelem, int* grid) {
-  return (int)prepare_elem_impl<D, N, Q1, R, OP>(nelem, grid);
+  constexpr bool W = ElemCfg<D, N, Q1, R, OP>::HAS_WIDE;
+  return use_wide<D, N, Q1, R, OP>(nelem) ? prepare_elem_impl<D, N, Q1, R, OP, W>(nelem, grid)
+                                          : prepare_elem_impl<D, N, Q1, R, OP, false>(nelem, grid);
 }
 
 }  // namespace tmop

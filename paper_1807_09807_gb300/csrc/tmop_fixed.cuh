@@ -34,34 +34,41 @@ namespace tmop {
 
 typedef long long fx_t;
 
-// Barrier of the G warps that share an element (named barrier `bar`).
-template <int G>
+// An element is worked on by GT threads: part of a warp, a warp or several.
+// The lanes of the group within its warp:
+template <int GT>
+__device__ __forceinline__ unsigned group_mask() {
+  if constexpr (GT >= 32) return 0xffffffffu;
+  else return ((1u << GT) - 1u) << (threadIdx.x & 31 & ~(GT - 1));
+}
+// Barrier of the group (named barrier `bar` where it is several warps).
+template <int GT>
 __device__ __forceinline__ void group_sync(int bar) {
-  if constexpr (G == 1) __syncwarp();
-  else asm volatile("bar.sync %0, %1;" ::"r"(bar), "n"(32 * G) : "memory");
+  if constexpr (GT <= 32) __syncwarp(group_mask<GT>());
+  else asm volatile("bar.sync %0, %1;" ::"r"(bar), "n"(GT) : "memory");
 }
 
-// exponent field of the largest magnitude among the high words `m` of a warp
-__device__ __forceinline__ int fx_warp_exp(unsigned m) { return (int)(__reduce_max_sync(0xffffffffu, m) >> 20); }
 __device__ __forceinline__ unsigned fx_mag(double v) { return (unsigned)__double2hiint(v) & 0x7fffffffu; }
 
-// The same over the G warps of an element for NC components, with the barrier
-// that makes the group's shared-memory writes before it visible. s: [G][NC]
-// words, rewritten only after a later barrier of the group.
-template <int G, int NC>
+// Exponent fields of the largest magnitudes (high words m) of NC components
+// among the group's threads, with the barrier that makes the group's
+// shared-memory writes before it visible. s: [warps of the group][NC] words,
+// rewritten only after a later barrier of the group.
+template <int GT, int NC>
 __device__ __forceinline__ void fx_group_exp(const unsigned* m, int* e, unsigned* s, int bar) {
-  if constexpr (G == 1) {
+  if constexpr (GT <= 32) {
 #pragma unroll
-    for (int c = 0; c < NC; ++c) e[c] = fx_warp_exp(m[c]);
-    __syncwarp();
+    for (int c = 0; c < NC; ++c) e[c] = (int)(__reduce_max_sync(group_mask<GT>(), m[c]) >> 20);
+    group_sync<GT>(bar);
   } else {
+    constexpr int G = GT / 32;
     const int w = (threadIdx.x >> 5) % G;
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
       const unsigned r = __reduce_max_sync(0xffffffffu, m[c]);
       if ((threadIdx.x & 31) == 0) s[w * NC + c] = r;
     }
-    group_sync<G>(bar);
+    group_sync<GT>(bar);
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
       unsigned r = s[c];
@@ -228,8 +235,8 @@ struct FxNodal {
 // 3D forward map of NC components. P0: X (FxNodal, double) -> P1: [NC][2][N][N][Q]
 // -> P0: [NC][3][N][Q][Q] -> P1: A[NC][3][Q][Q][Q] (double). em: exponent
 // field of the largest magnitude of each component. `lane`: the thread's
-// number among the 32 G of the element's warps.
-template <int N, int Q1, int NC, int G>
+// number among the GT of its group.
+template <int N, int Q1, int NC, int GT>
 __device__ __forceinline__ void fwd3_fx(const FxTab& T, const int (&em)[NC], double* P0d, double* P1d, int lane, int bar) {
   constexpr int NNQ = N * N * Q1, NQQ = N * Q1 * Q1, QQ = Q1 * Q1, QQQ = Q1 * Q1 * Q1;
   fx_t *P0 = reinterpret_cast<fx_t*>(P0d), *P1 = reinterpret_cast<fx_t*>(P1d);
@@ -240,7 +247,7 @@ __device__ __forceinline__ void fwd3_fx(const FxTab& T, const int (&em)[NC], dou
     return e;
   };
 #pragma unroll 1
-  for (int t = lane; t < NC * N * N; t += 32 * G) {               // (c, l, j): lines along x
+  for (int t = lane; t < NC * N * N; t += GT) {               // (c, l, j): lines along x
     const int c = t / (N * N), lj = t % (N * N), e = pick(c);
     fx_t v[N];
 #pragma unroll
@@ -251,9 +258,9 @@ __device__ __forceinline__ void fwd3_fx(const FxTab& T, const int (&em)[NC], dou
     fx_forward<N, Q1, false>(T, x, [&](int q, fx_t y) { o[q] = y; });
     fx_forward<N, Q1, true>(T, x, [&](int q, fx_t y) { o[NNQ + q] = y; });
   }
-  group_sync<G>(bar);
+  group_sync<GT>(bar);
 #pragma unroll 1
-  for (int t = lane; t < NC * N * Q1; t += 32 * G) {              // (c, l, q0): lines along y
+  for (int t = lane; t < NC * N * Q1; t += GT) {              // (c, l, q0): lines along y
     const int q0 = t % Q1, l = (t / Q1) % N, c = t / (Q1 * N);
     const fx_t* s = P1 + (c * 2) * NNQ + l * N * Q1 + q0;
     fx_t* o = P0 + (c * 3) * NQQ + l * QQ + q0;
@@ -269,9 +276,9 @@ __device__ __forceinline__ void fwd3_fx(const FxTab& T, const int (&em)[NC], dou
     x.set(v);
     fx_forward<N, Q1, false>(T, x, [&](int q, fx_t y) { o[2 * NQQ + q * Q1] = y; });
   }
-  group_sync<G>(bar);
+  group_sync<GT>(bar);
 #pragma unroll 1
-  for (int t = lane; t < NC * QQ; t += 32 * G) {                  // (c, q1, q0): lines along z
+  for (int t = lane; t < NC * QQ; t += GT) {                  // (c, q1, q0): lines along z
     const int c = t / QQ, q01 = t % QQ;
     const FxScale sc = fx_scale(pick(c), T.xin, T.gexp);
     const fx_t* s = P0 + (c * 3) * NQQ + q01;
@@ -290,12 +297,12 @@ __device__ __forceinline__ void fwd3_fx(const FxTab& T, const int (&em)[NC], dou
     x.set(v);
     fx_forward<N, Q1, true>(T, x, [&](int q, fx_t y) { o[2 * QQQ + q * QQ] = fx_to_f64(y, sc); });
   }
-  group_sync<G>(bar);
+  group_sync<GT>(bar);
 }
 
 // 3D adjoint map. P1: R[NC][3][Q][Q][Q] (double) -> P0: [NC][3][N][Q][Q] ->
 // P1: [NC][2][N][N][Q] -> P0: Y (FxNodal, double).
-template <int N, int Q1, int NC, int G>
+template <int N, int Q1, int NC, int GT>
 __device__ __forceinline__ void adj3_fx(const FxTab& T, const int (&em)[NC], double* P0d, double* P1d, int lane, int bar) {
   constexpr int NNQ = N * N * Q1, NQQ = N * Q1 * Q1, QQ = Q1 * Q1, QQQ = Q1 * Q1 * Q1;
   fx_t *P0 = reinterpret_cast<fx_t*>(P0d), *P1 = reinterpret_cast<fx_t*>(P1d);
@@ -306,7 +313,7 @@ __device__ __forceinline__ void adj3_fx(const FxTab& T, const int (&em)[NC], dou
     return e;
   };
 #pragma unroll 1
-  for (int t = lane; t < NC * QQ; t += 32 * G) {                  // (c, q1, q0): lines along z
+  for (int t = lane; t < NC * QQ; t += GT) {                  // (c, q1, q0): lines along z
     const int c = t / QQ, q01 = t % QQ, e = pick(c), sh = T.rin - 53;
     const double* s = P1d + (c * 3) * QQQ + q01;
     fx_t* o = P0 + (c * 3) * NQQ + q01;
@@ -324,9 +331,9 @@ __device__ __forceinline__ void adj3_fx(const FxTab& T, const int (&em)[NC], dou
     x.set(v);
     fx_adjoint<N, Q1, false, true>(T, x, x, [&](int l, fx_t y) { o[2 * NQQ + l * QQ] = y; });
   }
-  group_sync<G>(bar);
+  group_sync<GT>(bar);
 #pragma unroll 1
-  for (int t = lane; t < NC * N * Q1; t += 32 * G) {              // (c, l, q0): lines along y
+  for (int t = lane; t < NC * N * Q1; t += GT) {              // (c, l, q0): lines along y
     const int q0 = t % Q1, l = (t / Q1) % N, c = t / (Q1 * N);
     const fx_t* s = P0 + (c * 3) * NQQ + l * QQ + q0;
     fx_t* o = P1 + (c * 2) * NNQ + l * N * Q1 + q0;
@@ -344,9 +351,9 @@ __device__ __forceinline__ void adj3_fx(const FxTab& T, const int (&em)[NC], dou
     x.set(v);
     fx_adjoint<N, Q1, true, true>(T, x, g, [&](int j, fx_t y) { o[NNQ + j * Q1] = y; });        // pairs with B in x
   }
-  group_sync<G>(bar);
+  group_sync<GT>(bar);
 #pragma unroll 1
-  for (int t = lane; t < NC * N * N; t += 32 * G) {               // (c, l, j): lines along x
+  for (int t = lane; t < NC * N * N; t += GT) {               // (c, l, j): lines along x
     const int c = t / (N * N), lj = t % (N * N);
     const FxScale sc = fx_scale(pick(c), T.rin, T.gexp);
     const fx_t* s = P1 + (c * 2) * NNQ + lj * Q1;
@@ -361,11 +368,11 @@ __device__ __forceinline__ void adj3_fx(const FxTab& T, const int (&em)[NC], dou
     x.set(v);
     fx_adjoint<N, Q1, true, true>(T, x, g, [&](int i, fx_t y) { o[i * FxNodal<3, N>::LS] = fx_to_f64(y, sc); });
   }
-  group_sync<G>(bar);
+  group_sync<GT>(bar);
 }
 
 // 2D forward map. P0: X (FxNodal) -> P1: [NC][2][N][Q] -> P0: A[NC][2][Q][Q]
-template <int N, int Q1, int NC, int G>
+template <int N, int Q1, int NC, int GT>
 __device__ __forceinline__ void fwd2_fx(const FxTab& T, const int (&em)[NC], double* P0d, double* P1d, int lane, int bar) {
   constexpr int NQ = N * Q1, QQ = Q1 * Q1;
   fx_t* P1 = reinterpret_cast<fx_t*>(P1d);
@@ -376,7 +383,7 @@ __device__ __forceinline__ void fwd2_fx(const FxTab& T, const int (&em)[NC], dou
     return e;
   };
 #pragma unroll 1
-  for (int t = lane; t < NC * N; t += 32 * G) {                   // (c, j): lines along x
+  for (int t = lane; t < NC * N; t += GT) {                   // (c, j): lines along x
     const int c = t / N, j = t % N, e = pick(c);
     fx_t v[N];
 #pragma unroll
@@ -387,9 +394,9 @@ __device__ __forceinline__ void fwd2_fx(const FxTab& T, const int (&em)[NC], dou
     fx_forward<N, Q1, false>(T, x, [&](int q, fx_t y) { o[q] = y; });
     fx_forward<N, Q1, true>(T, x, [&](int q, fx_t y) { o[NQ + q] = y; });
   }
-  group_sync<G>(bar);
+  group_sync<GT>(bar);
 #pragma unroll 1
-  for (int t = lane; t < NC * Q1; t += 32 * G) {                  // (c, q0): lines along y
+  for (int t = lane; t < NC * Q1; t += GT) {                  // (c, q0): lines along y
     const int q0 = t % Q1, c = t / Q1;
     const FxScale sc = fx_scale(pick(c), T.xin, T.gexp);
     const fx_t* s = P1 + (c * 2) * NQ + q0;
@@ -405,11 +412,11 @@ __device__ __forceinline__ void fwd2_fx(const FxTab& T, const int (&em)[NC], dou
     x.set(v);
     fx_forward<N, Q1, true>(T, x, [&](int q, fx_t y) { o[QQ + q * Q1] = fx_to_f64(y, sc); });    // d/dxi_1
   }
-  group_sync<G>(bar);
+  group_sync<GT>(bar);
 }
 
 // 2D adjoint map. P0: R[NC][2][Q][Q] -> P1: [NC][2][N][Q] -> P0: Y (FxNodal)
-template <int N, int Q1, int NC, int G>
+template <int N, int Q1, int NC, int GT>
 __device__ __forceinline__ void adj2_fx(const FxTab& T, const int (&em)[NC], double* P0d, double* P1d, int lane, int bar) {
   constexpr int NQ = N * Q1, QQ = Q1 * Q1;
   fx_t* P1 = reinterpret_cast<fx_t*>(P1d);
@@ -420,7 +427,7 @@ __device__ __forceinline__ void adj2_fx(const FxTab& T, const int (&em)[NC], dou
     return e;
   };
 #pragma unroll 1
-  for (int t = lane; t < NC * Q1; t += 32 * G) {                  // (c, q0): lines along y
+  for (int t = lane; t < NC * Q1; t += GT) {                  // (c, q0): lines along y
     const int q0 = t % Q1, c = t / Q1, e = pick(c), sh = T.rin - 53;
     const double* s = P0d + (c * 2) * QQ + q0;
     fx_t* o = P1 + (c * 2) * NQ + q0;
@@ -435,9 +442,9 @@ __device__ __forceinline__ void adj2_fx(const FxTab& T, const int (&em)[NC], dou
     x.set(v);
     fx_adjoint<N, Q1, false, true>(T, x, x, [&](int j, fx_t y) { o[NQ + j * Q1] = y; });        // pairs with B in x
   }
-  group_sync<G>(bar);
+  group_sync<GT>(bar);
 #pragma unroll 1
-  for (int t = lane; t < NC * N; t += 32 * G) {                   // (c, j): lines along x
+  for (int t = lane; t < NC * N; t += GT) {                   // (c, j): lines along x
     const int c = t / N, j = t % N;
     const FxScale sc = fx_scale(pick(c), T.rin, T.gexp);
     const fx_t* s = P1 + (c * 2) * NQ + j * Q1;
@@ -452,7 +459,7 @@ __device__ __forceinline__ void adj2_fx(const FxTab& T, const int (&em)[NC], dou
     x.set(v);
     fx_adjoint<N, Q1, true, true>(T, x, g, [&](int i, fx_t y) { o[i * FxNodal<2, N>::LS] = fx_to_f64(y, sc); });
   }
-  group_sync<G>(bar);
+  group_sync<GT>(bar);
 }
 
 }  // namespace tmop

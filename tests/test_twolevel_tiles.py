@@ -1,5 +1,5 @@
 """The sine transforms of the two-level preconditioner at the edges of their
-tiles (16 outputs per side, 64-deep chunks): 16, 17, 33 and 65 interior
+tiles (8 outputs per side, 32-deep chunks): 16, 17, 33 and 65 interior
 vertices along an axis, against the dense definition in oracle/twolevel.py
 (1e-10: FP64 sums of at most 65 terms, times the condition number ~1e3 of the
 coarse Laplacian)."""
