@@ -77,11 +77,12 @@ struct ElemCfg {
   static constexpr bool TWO = FX3 && OP == OP_ENERGY && 12 * PER_WARP <= 200 * 1024;
   static constexpr int FIT = 200 * 1024 / PER_WARP;
   static constexpr int WARPS = GT == 64 ? 1 : (TWO ? 6 : (FIT >= 8 ? 8 : (FIT < 1 ? 1 : FIT)));
-  // blocks per SM that bound the registers (0: no bound): 8 (128 registers),
-  // 10 (96) for the gradient, whose pointwise stage needs fewer (32^3 order-2
-  // hexes, mu302: 422 us with 8, 392 us with 10; the stored-Hessian product
-  // 211 us with 8, 223 us with 12)
-  static constexpr int WANT = (OP == OP_GRADIENT || OP == OP_ENERGY_GRAD) ? 10 : 8;
+  // Blocks per SM that bound the registers (0: no bound): 6 (168 registers)
+  // for the kernels that hold T and dT, 7 (144) for the others. 48^3 order-3
+  // hexes, gradient + Hessian action: 4.61 ms with 8 (spills), 3.75 with 6,
+  // 3.72 with 5; 24^3, stored-Hessian product 329 us with 8, 324 with 7, 334
+  // with 6; energy + gradient 232 us with 9, 227 with 7.
+  static constexpr int WANT = HV ? 6 : 7;
   static constexpr int MINB = GT == 64 ? (FIT >= WANT ? WANT : FIT) : (TWO ? 2 : 0);
   // after the 1D tables: the product weight w_q0 w_q1 (w_q2) of every point
   static constexpr int WQ_OFF = 2 * kMaxQ * kMaxN + kMaxQ;
@@ -164,6 +165,12 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP, WIDE>::WARPS * ElemCf
     sWq[t] = w;
   }
   constexpr int GW = GT > 32 ? GT / 32 : 1;   // warps per element
+  // mu303 with W = I: the pointwise stage of these FP64 3D kernels in fixed point (fx_point303)
+  constexpr bool FX303 = FX && D == 3 && OP != OP_LINEARIZE && OP != OP_HESS_PA;
+  constexpr int NKEY = OP == OP_GRAD_HESS ? 2 : 1;
+  __shared__ short s_kq[FX303 ? WARPS : 1][FX303 ? NKEY * QP : 1];   // exponents of the points' results
+  __shared__ int s_key[FX303 ? WARPS : 1][GW * NKEY];
+  __shared__ unsigned s_top[WARPS][GW];
   __shared__ unsigned s_mag[WARPS][GW * 2 * D];   // per warp and component: largest magnitudes of the group's warps
   R Wi[DD];
 #pragma unroll
@@ -269,18 +276,32 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP, WIDE>::WARPS * ElemCf
       }
     }
     int em[FX ? Cfg::NC : 1];
+    int emx[FX ? D : 1];   // the split Hessian action's exponents of x
+    bool fx303 = false;    // mu303 with W = I: pointwise stage in fixed point
+    int upA = 0, upV = 0;  // and the bits T and dT have to spare there
     if constexpr (FX) fx_group_exp<GT, Cfg::NC>(mag, em, s_mag[warp], bar);
     else __syncwarp();
+    if constexpr (FX303) {
+      // one exponent for all components (at most 4 bits lost to one of them),
+      // where those of the products stay inside the FP64 range (fx_point303)
+      const int lo = min(em[0], min(em[1], em[2])), hi = max(em[0], max(em[1], em[2]));
+      fx303 = p.metric == 303 && p.wkind == WK_IDENTITY && !p.metric2 && lo > 600 && hi < 1400 && hi - lo <= 4;
+      if (fx303) em[0] = em[1] = em[2] = hi;
+    }
     // ---- forward contraction: A (and dA) at every point
     if constexpr (Cfg::SPLIT && FX) {
       // A(x) into P2 (P2 also serves as the first stage buffer), then v into
       // P1, by one copy of the code
 #pragma unroll 1
       for (int f = 0;; ++f) {
-        fwd3_fx<N, Q1, D, GT>(p.fx, em, P0, f == 0 ? P2 : P1, lane, bar);
+        const unsigned top = fwd3_fx<N, Q1, D, GT>(p.fx, em, P0, f == 0 ? P2 : P1, s_top[warp], lane, bar);
+        (f == 0 ? upA : upV) = fx_room(top);
         if (f) break;
 #pragma unroll
-        for (int c = 0; c < D; ++c) mag[c] = 0;
+        for (int c = 0; c < D; ++c) {
+          mag[c] = 0;
+          emx[c] = em[c];
+        }
 #pragma unroll
         for (int k = 0; k < VPRE; ++k) {
           const int t = lane + k * GT;
@@ -292,6 +313,11 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP, WIDE>::WARPS * ElemCf
           }
         }
         fx_group_exp<GT, D>(mag, em, s_mag[warp], bar);
+        if (fx303) {
+          const int hi = max(em[0], max(em[1], em[2]));
+          fx303 = hi > 300 && hi < 1750 && hi - emx[0] > -700 && hi - emx[0] < 700;
+          if (fx303) em[0] = em[1] = em[2] = hi;
+        }
       }
     } else if constexpr (Cfg::SPLIT) {
       fwd3_rb<N, Q1, D, R>(tB, tG, P0, P2, lane);
@@ -310,7 +336,7 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP, WIDE>::WARPS * ElemCf
       if constexpr (FX) fwd2_fx<N, Q1, Cfg::NC, GT>(p.fx, em, P0, P1, lane, bar);
       else fwd2<N, Q1, Cfg::NC, R>(sB, sG, P0, P1, lane);
     } else {
-      if constexpr (FX) fwd3_fx<N, Q1, Cfg::NC, GT>(p.fx, em, P0, P1, lane, bar);
+      if constexpr (FX) upA = fx_room(fwd3_fx<N, Q1, Cfg::NC, GT>(p.fx, em, P0, P1, s_top[warp], lane, bar));
       else fwd3_rb<N, Q1, Cfg::NC, R>(tB, tG, P0, P1, lane);
     }
     R* Abuf = Cfg::SPLIT ? P2 : ((D == 2) ? P0 : P1);     // A: [D][D][QP]
@@ -318,6 +344,23 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP, WIDE>::WARPS * ElemCf
     R* Rbuf = Cfg::SPLIT ? P1 : Abuf;                    // per-point output of the adjoint
     // ---- pointwise
     double emin = INFINITY;
+    // FP64 3D: A and dA are in fixed point
+    constexpr bool RAW = FX && D == 3;
+    FxScale sA[RAW ? D : 1], sV[RAW ? D : 1];
+    if constexpr (RAW) {
+#pragma unroll
+      for (int c = 0; c < D; ++c) {
+        sA[c] = fx_scale(Cfg::SPLIT ? emx[c] : em[c], p.fx.xin, p.fx.gexp);
+        sV[c] = fx_scale(em[c], p.fx.xin, p.fx.gexp);
+      }
+    }
+    auto load = [&](const R* buf, const FxScale* sc, int i, int q) -> R {
+      if constexpr (RAW) return fx_to_f64(reinterpret_cast<const fx_t*>(buf)[i * QP + q], sc[i / D]);
+      else return buf[i * QP + q];
+    };
+    int key[FX303 ? NKEY : 1];
+#pragma unroll
+    for (int k = 0; k < (FX303 ? NKEY : 1); ++k) key[k] = -4000;
     // FP64: largest magnitude (high word) per component of the fields the
     // adjoint map takes (OP_GRAD_HESS: the gradient's, then the Hessian action's)
     unsigned rmag[FX ? 2 * D : 1] = {};
@@ -338,7 +381,7 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP, WIDE>::WARPS * ElemCf
         R dA[DD], y[DD];
 #pragma unroll
         for (int i = 0; i < DD; ++i) {
-          dA[i] = Abuf[i * QP + q];
+          dA[i] = load(Abuf, sA, i, q);
           y[i] = R(0);
         }
         int s = 0;
@@ -356,11 +399,34 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP, WIDE>::WARPS * ElemCf
         }
         continue;
       }
+      if constexpr (FX303) {
+        if (fx303) {
+          FxPoint pt[2];   // of the gradient's fields, of the Hessian action's
+          double mu, tau;
+          const double s = sWq[q] * p.detW;
+          const bool ok = fx_point303<QP, GRADLIKE || OP == OP_GRAD_HESS, Cfg::HV>(
+              reinterpret_cast<fx_t*>(Abuf) + q, reinterpret_cast<fx_t*>(dAbuf) + q, upA, upV, sA[0].kb, sV[0].kb, s,
+              pt[0], pt[NKEY - 1], mu, tau);
+          if constexpr (OP != OP_ENERGY) {
+#pragma unroll
+            for (int k = 0; k < NKEY; ++k) {
+              key[k] = max(key[k], fx_point_key(pt[k]));
+              s_kq[warp][k * QP + q] = (short)(pt[k].mag ? pt[k].E : -16000);
+            }
+          }
+          if constexpr (EG || OP == OP_ENERGY) {
+            emin = fmin(emin, tau);
+            if (ok) accF += s * mu;
+            else accF = INFINITY;
+          }
+          continue;
+        }
+      }
       R A[DD];
 #pragma unroll
       for (int a = 0; a < D; ++a)
 #pragma unroll
-        for (int b = 0; b < D; ++b) A[a * D + b] = Abuf[(a * D + b) * QP + q];
+        for (int b = 0; b < D; ++b) A[a * D + b] = load(Abuf, sA, a * D + b, q);
       const R wq = sWq[q];
       R detW = R(p.detW);
       if (p.wkind == WK_PER_QP) {
@@ -393,7 +459,7 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP, WIDE>::WARPS * ElemCf
         const R s = wq * detW;
         R dA[DD], dT[DD], Sg[DD], Sh[DD];
 #pragma unroll
-        for (int i = 0; i < DD; ++i) dA[i] = dAbuf[i * QP + q];
+        for (int i = 0; i < DD; ++i) dA[i] = load(dAbuf, sV, i, q);
         if (p.wkind == WK_IDENTITY) {
 #pragma unroll
           for (int i = 0; i < DD; ++i) dT[i] = dA[i];
@@ -609,7 +675,7 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP, WIDE>::WARPS * ElemCf
         } else {
           R dT[DD];
 #pragma unroll
-          for (int i = 0; i < DD; ++i) dA[i] = dAbuf[i * QP + q];
+          for (int i = 0; i < DD; ++i) dA[i] = load(dAbuf, sV, i, q);
           if (p.wkind == WK_IDENTITY) {
 #pragma unroll
             for (int i = 0; i < DD; ++i) dT[i] = dA[i];
@@ -721,7 +787,8 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP, WIDE>::WARPS * ElemCf
         }
       } else {
         int er2[2 * D];
-        fx_group_exp<GT, 2 * D>(rmag, er2, s_mag[warp], bar);
+        if (FX303 && fx303) fx_group_max<GT, NKEY>(key, s_key[warp], bar);
+        else fx_group_exp<GT, 2 * D>(rmag, er2, s_mag[warp], bar);
 #pragma unroll 1
         for (int pass = 0; pass < 2; ++pass) {
           R* Rin = pass == 0 ? P1 : P2;
@@ -729,7 +796,13 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP, WIDE>::WARPS * ElemCf
           int er[D];
 #pragma unroll
           for (int c = 0; c < D; ++c) er[c] = pass == 0 ? er2[D + c] : er2[c];
-          adj3_fx<N, Q1, D, GT>(p.fx, er, P0, Rin, lane, bar);
+          if (FX303 && fx303) {
+            const int k = pass == 0 ? 1 : 0, L = pass == 0 ? key[NKEY - 1] : key[0];
+            er[0] = er[1] = er[D - 1] = fx_point_emax(L);
+            adj3_fx<N, Q1, D, GT, true>(p.fx, er, P0, Rin, lane, bar, s_kq[warp] + k * QP, L);
+          } else {
+            adj3_fx<N, Q1, D, GT>(p.fx, er, P0, Rin, lane, bar);
+          }
           for (int t = lane; t < NDOF; t += GT) {
             const int gn = nodes(t);
 #pragma unroll
@@ -747,9 +820,17 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP, WIDE>::WARPS * ElemCf
       // ---- adjoint contraction and scatter
       if constexpr (FX) {
         int er[D];
-        fx_group_exp<GT, D>(rmag, er, s_mag[warp], bar);
-        if constexpr (D == 2) adj2_fx<N, Q1, D, GT>(p.fx, er, P0, P1, lane, bar);
-        else adj3_fx<N, Q1, D, GT>(p.fx, er, P0, P1, lane, bar);
+        if (FX303 && fx303) {
+          if constexpr (FX303) {
+            fx_group_max<GT, 1>(key, s_key[warp], bar);
+            er[0] = er[1] = er[2] = fx_point_emax(key[0]);
+            adj3_fx<N, Q1, D, GT, true>(p.fx, er, P0, P1, lane, bar, s_kq[warp], key[0]);
+          }
+        } else {
+          fx_group_exp<GT, D>(rmag, er, s_mag[warp], bar);
+          if constexpr (D == 2) adj2_fx<N, Q1, D, GT>(p.fx, er, P0, P1, lane, bar);
+          else adj3_fx<N, Q1, D, GT>(p.fx, er, P0, P1, lane, bar);
+        }
       } else if constexpr (D == 2) {
         __syncwarp();
         adj2<N, Q1, D, R>(sB, sG, P0, P1, lane);

@@ -1,16 +1,19 @@
 // FP64 tensor-product contractions in 64-bit fixed point.
 //
-// Why: GB300 executes 2 FP64 operations per SM and clock, and 64 IMAD.WIDE
-// (32 x 32 + 64 -> 64 bit) per SM and clock (measured: 1.90 and 56.7 lane
-// operations at the 2.07 GHz maximum clock), with the integer pipe running
-// beside the FP64 pipe (one DFMA and 16 IMAD.WIDE take no longer than the
-// DFMA alone). A contraction is a sum of products of field values with
-// constant table entries, so its operands share one exponent per element and
-// component: written as integers of ~57 bits relative to the largest value,
-// a multiply-add is three IMAD.WIDE with no carry handling, and the result
-// is as accurate as FP64 arithmetic (whose intermediate sums round at 2^-53
-// of their magnitude; the dropped parts here lie at ~2^-57 of the largest
-// value). The FP64 pipe keeps the pointwise metric work only.
+// Why: an FP64 multiply-add takes GB300's FP64 pipe 17 cycles per warp and SM
+// (an add or a multiply 20), a 32 x 32 + 64 -> 64 bit IMAD.WIDE the integer
+// pipe 4 cycles per warp and scheduler, i.e. 1 per SM, and the two pipes run
+// beside one another (measured). A contraction is a sum of products of field
+// values with constant table entries, so its operands can share one exponent
+// per element and component: written as integers of ~57 bits relative to the
+// largest value, a multiply-add is three IMAD.WIDE with no carry handling, and
+// the result is as accurate as FP64 arithmetic (whose intermediate sums round
+// at 2^-53 of their magnitude; the dropped parts here lie at ~2^-57 of the
+// largest value). The same holds for the products of matrix entries in the
+// pointwise stage of mu303 (fx_point303), of which only the scalars stay in
+// FP64. 48^3 order-3 hexes, gradient + Hessian action: 11.13 ms with FP64
+// contractions, 5.53 ms with these, 3.75 ms with the pointwise products too
+// (FP64 instructions per element and warp 1490, 654, 98).
 //
 // Numbers: a value v of a component whose largest magnitude is below 2^E is
 // held as round-toward-zero(v 2^(X - E)), X = xin (forward) or rin (adjoint)
@@ -28,6 +31,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "tmop_device.cuh"
 #include "tmop_kparams.h"
 
 namespace tmop {
@@ -50,6 +54,11 @@ __device__ __forceinline__ void group_sync(int bar) {
 
 __device__ __forceinline__ unsigned fx_mag(double v) { return (unsigned)__double2hiint(v) & 0x7fffffffu; }
 
+// The exponents used: not below 64, so that a component of zeros (or of
+// magnitudes below 2^-1016 and less) becomes zeros and the exponent field of a
+// result cannot fall below 1.
+__device__ __forceinline__ int fx_floor(unsigned e) { return e < 64u ? 64 : (int)e; }
+
 // Exponent fields of the largest magnitudes (high words m) of NC components
 // among the group's threads, with the barrier that makes the group's
 // shared-memory writes before it visible. s: [warps of the group][NC] words,
@@ -58,7 +67,7 @@ template <int GT, int NC>
 __device__ __forceinline__ void fx_group_exp(const unsigned* m, int* e, unsigned* s, int bar) {
   if constexpr (GT <= 32) {
 #pragma unroll
-    for (int c = 0; c < NC; ++c) e[c] = (int)(__reduce_max_sync(group_mask<GT>(), m[c]) >> 20);
+    for (int c = 0; c < NC; ++c) e[c] = fx_floor(__reduce_max_sync(group_mask<GT>(), m[c]) >> 20);
     group_sync<GT>(bar);
   } else {
     constexpr int G = GT / 32;
@@ -74,13 +83,13 @@ __device__ __forceinline__ void fx_group_exp(const unsigned* m, int* e, unsigned
       unsigned r = s[c];
 #pragma unroll
       for (int k = 1; k < G; ++k) r = max(r, s[k * NC + c]);
-      e[c] = (int)(r >> 20);
+      e[c] = fx_floor(r >> 20);
     }
   }
 }
 
 // v -> fixed point with `lsh` + 53 bits below 2^(emax - 1022), emax >= the
-// exponent field of v (emax < 64: the value is irrelevant, see fx_to_f64).
+// exponent field of v and >= 64.
 __device__ __forceinline__ fx_t fx_from_f64(double v, int emax, int lsh) {
   const unsigned hi = (unsigned)__double2hiint(v), lo = (unsigned)__double2loint(v);
   const unsigned mh = (hi & 0xfffffu) | 0x100000u;
@@ -89,40 +98,36 @@ __device__ __forceinline__ fx_t fx_from_f64(double v, int emax, int lsh) {
   return (fx_t)(m ^ (unsigned long long)(long long)((int)hi >> 31));   // (complement: off by one unit)
 }
 
-// Scale of a component's results: the exponent field of a result whose
-// leading bit is bit b is b + kb. Components with a non-finite value become
-// NaN, those below 2^-958 zero; these, and the exponents near the ends of the
-// FP64 range, take the slow conversion (lim = all ones).
+// Scale of a component's values: the exponent field of a value whose leading
+// bit is bit b is b + kb. A component with a non-finite value (or one above
+// 2^1013, whose results might not be finite) becomes NaN.
 struct FxScale {
   int kb;
-  unsigned lim;
-  int emax;
+  unsigned nan;
 };
+__device__ __forceinline__ unsigned fx_nan(int emax) { return emax >= 2036 ? 0x7ff80000u : 0u; }
 __device__ __forceinline__ FxScale fx_scale(int emax, int bits, int gexp) {
-  FxScale s;
-  s.kb = 1 + gexp + emax - bits;
-  s.lim = (emax > 1900 || emax < 150) ? 0xffffffffu : 0u;
-  s.emax = emax;
-  return s;
+  return {1 + gexp + emax - bits, fx_nan(emax)};
 }
 
+// |y| < 2^62 -> FP64, rounded to nearest (values below 2^31 in magnitude are
+// exact but for their last bit). Without branches, so that several
+// conversions overlap.
 __device__ __forceinline__ double fx_to_f64(fx_t y, const FxScale& s) {
   const int neg = (int)(y >> 32) >> 31;
   // (the complement for the negative: off by one unit of ~2^-57)
-  unsigned long long u = (unsigned long long)y ^ (unsigned long long)(long long)neg;
-  const unsigned uh = (unsigned)(u >> 32);
-  if (uh <= s.lim) {   // small against the component's largest value, or an extreme exponent
-    const int k = s.kb - 1023, k1 = k / 2, k2 = k - k1;
-    const double v = (double)y * __hiloint2double((1023 + k1) << 20, 0) * __hiloint2double((1023 + k2) << 20, 0);
-    if (s.emax == 0x7ff) return __longlong_as_double(0x7ff8000000000000LL);
-    return s.emax < 64 ? 0.0 : v;
-  }
-  unsigned b;                          // leading bit of uh, <= 29: |y| < 2^62
+  unsigned uh = (unsigned)((int)(y >> 32) ^ neg), ul = (unsigned)((int)y ^ neg);
+  const bool low = uh == 0;            // the leading bit is in the low word
+  uh = low ? ul >> 1 : uh;
+  ul = low ? ul << 31 : ul;
+  unsigned b;                          // leading bit of uh, <= 30
   asm("bfind.u32 %0, %1;" : "=r"(b) : "r"(uh));
-  u = (u << (30 - b)) + 0x200u;        // leading bit 62; round the 10 low bits
-  u >>= 10;
-  const unsigned hi = (unsigned)(u >> 32) + (b << 20) + ((unsigned)(31 + s.kb) << 20);   // the leading bit adds one
-  return __hiloint2double((int)(hi | ((unsigned)neg & 0x80000000u)), (int)(unsigned)u);
+  unsigned long long u = ((((unsigned long long)uh << 32) | ul) << (30 - b)) + 0x200u;   // leading bit 62; round the
+  u >>= 10;                                                                               // 10 low bits
+  const unsigned f = (b << 20) + ((unsigned)(s.kb + (low ? 0 : 31)) << 20);              // the leading bit adds one
+  unsigned hi = (unsigned)(u >> 32) + f;
+  hi = uh == 0 ? 0u : hi;
+  return __hiloint2double((int)(hi | ((unsigned)neg & 0x80000000u) | s.nan), (int)(unsigned)u);
 }
 
 // 30-bit limbs of a value
@@ -233,11 +238,19 @@ struct FxNodal {
 };
 
 // 3D forward map of NC components. P0: X (FxNodal, double) -> P1: [NC][2][N][N][Q]
-// -> P0: [NC][3][N][Q][Q] -> P1: A[NC][3][Q][Q][Q] (double). em: exponent
-// field of the largest magnitude of each component. `lane`: the thread's
+// -> P0: [NC][3][N][Q][Q] -> P1: A[NC][3][Q][Q][Q] (fixed point at fx_scale(em,
+// xin, gexp): the pointwise stage converts them, one point per thread). em:
+// exponent field of the largest magnitude of each component. Returns the
+// largest magnitude of the results (their high words); s_top: a word per warp. `lane`: the thread's
 // number among the GT of its group.
 template <int N, int Q1, int NC, int GT>
-__device__ __forceinline__ void fwd3_fx(const FxTab& T, const int (&em)[NC], double* P0d, double* P1d, int lane, int bar) {
+__device__ __forceinline__ unsigned fwd3_fx(const FxTab& T, const int (&em)[NC], double* P0d, double* P1d,
+                                            unsigned* s_top, int lane, int bar) {
+  unsigned top = 0;
+  auto keep = [&](fx_t* o, fx_t y) {
+    *o = y;
+    top = max(top, (unsigned)((int)(y >> 32) ^ ((int)(y >> 32) >> 31)));
+  };
   constexpr int NNQ = N * N * Q1, NQQ = N * Q1 * Q1, QQ = Q1 * Q1, QQQ = Q1 * Q1 * Q1;
   fx_t *P0 = reinterpret_cast<fx_t*>(P0d), *P1 = reinterpret_cast<fx_t*>(P1d);
   auto pick = [&](int c) {
@@ -280,9 +293,8 @@ __device__ __forceinline__ void fwd3_fx(const FxTab& T, const int (&em)[NC], dou
 #pragma unroll 1
   for (int t = lane; t < NC * QQ; t += GT) {                  // (c, q1, q0): lines along z
     const int c = t / QQ, q01 = t % QQ;
-    const FxScale sc = fx_scale(pick(c), T.xin, T.gexp);
     const fx_t* s = P0 + (c * 3) * NQQ + q01;
-    double* o = P1d + (c * 3) * QQQ + q01;
+    fx_t* o = P1 + (c * 3) * QQQ + q01;
     fx_t v[N];
     FxLine<N> x;
 #pragma unroll 1
@@ -290,20 +302,38 @@ __device__ __forceinline__ void fwd3_fx(const FxTab& T, const int (&em)[NC], dou
 #pragma unroll
       for (int l = 0; l < N; ++l) v[l] = s[(2 - k) * NQQ + l * QQ];
       x.set(v);
-      fx_forward<N, Q1, false>(T, x, [&](int q, fx_t y) { o[k * QQQ + q * QQ] = fx_to_f64(y, sc); });
+      fx_forward<N, Q1, false>(T, x, [&](int q, fx_t y) { keep(o + k * QQQ + q * QQ, y); });
     }
 #pragma unroll
     for (int l = 0; l < N; ++l) v[l] = s[l * QQ];
     x.set(v);
-    fx_forward<N, Q1, true>(T, x, [&](int q, fx_t y) { o[2 * QQQ + q * QQ] = fx_to_f64(y, sc); });
+    fx_forward<N, Q1, true>(T, x, [&](int q, fx_t y) { keep(o + 2 * QQQ + q * QQ, y); });
   }
-  group_sync<GT>(bar);
+  top = __reduce_max_sync(group_mask<GT>(), top);
+  if constexpr (GT > 32) {
+    if ((threadIdx.x & 31) == 0) s_top[(threadIdx.x >> 5) % (GT / 32)] = top;
+    group_sync<GT>(bar);
+#pragma unroll
+    for (int w = 0; w < GT / 32; ++w) top = max(top, s_top[w]);
+  } else {
+    group_sync<GT>(bar);
+  }
+  return top;
+}
+
+// y shifted left by sh bits (right, with its sign, for sh < 0)
+__device__ __forceinline__ fx_t fx_align(fx_t y, int sh) {
+  const int r = min(max(-sh, 0), 63), l = max(sh, 0);
+  return (fx_t)((unsigned long long)y << l) >> r;
 }
 
 // 3D adjoint map. P1: R[NC][3][Q][Q][Q] (double) -> P0: [NC][3][N][Q][Q] ->
 // P1: [NC][2][N][N][Q] -> P0: Y (FxNodal, double).
-template <int N, int Q1, int NC, int GT>
-__device__ __forceinline__ void adj3_fx(const FxTab& T, const int (&em)[NC], double* P0d, double* P1d, int lane, int bar) {
+// RAW: R is in fixed point instead, point q at exponent kq[q] (FxPoint::E) of an
+// element whose largest key is L (all components then share one exponent).
+template <int N, int Q1, int NC, int GT, bool RAW = false>
+__device__ __forceinline__ void adj3_fx(const FxTab& T, const int (&em)[NC], double* P0d, double* P1d, int lane, int bar,
+                                        const short* kq = nullptr, int L = 0) {
   constexpr int NNQ = N * N * Q1, NQQ = N * Q1 * Q1, QQ = Q1 * Q1, QQQ = Q1 * Q1 * Q1;
   fx_t *P0 = reinterpret_cast<fx_t*>(P0d), *P1 = reinterpret_cast<fx_t*>(P1d);
   auto pick = [&](int c) {
@@ -319,15 +349,24 @@ __device__ __forceinline__ void adj3_fx(const FxTab& T, const int (&em)[NC], dou
     fx_t* o = P0 + (c * 3) * NQQ + q01;
     fx_t v[Q1];
     FxLine<Q1> x;
+    int al[RAW ? Q1 : 1];
+    if constexpr (RAW) {
+#pragma unroll
+      for (int q = 0; q < Q1; ++q) al[q] = kq[q * QQ + q01] - L + T.rin - 33;
+    }
+    auto in = [&](int i, int q) {
+      if constexpr (RAW) return fx_align(reinterpret_cast<const fx_t*>(s)[i], al[q]);
+      else return fx_from_f64(s[i], e, sh);
+    };
 #pragma unroll 1
     for (int k = 0; k < 2; ++k) {
 #pragma unroll
-      for (int q = 0; q < Q1; ++q) v[q] = fx_from_f64(s[k * QQQ + q * QQ], e, sh);
+      for (int q = 0; q < Q1; ++q) v[q] = in(k * QQQ + q * QQ, q);
       x.set(v);
       fx_adjoint<N, Q1, true, false>(T, x, x, [&](int l, fx_t y) { o[k * NQQ + l * QQ] = y; });
     }
 #pragma unroll
-    for (int q = 0; q < Q1; ++q) v[q] = fx_from_f64(s[2 * QQQ + q * QQ], e, sh);
+    for (int q = 0; q < Q1; ++q) v[q] = in(2 * QQQ + q * QQ, q);
     x.set(v);
     fx_adjoint<N, Q1, false, true>(T, x, x, [&](int l, fx_t y) { o[2 * NQQ + l * QQ] = y; });
   }
@@ -462,4 +501,150 @@ __device__ __forceinline__ void adj2_fx(const FxTab& T, const int (&em)[NC], dou
   group_sync<GT>(bar);
 }
 
+// Bits to shift the entries of a field up by: to |entries| < 2^59 by the
+// largest one of the element (top: its high word), or none (< 2^59.4 by
+// fx_tables).
+__device__ __forceinline__ int fx_room(unsigned top) { return max(__clz((int)top) - 5, 0); }
+
+// mu303 at one point in fixed point (W = I): s P (GRAD, in place of T) and s dP
+// in direction V (HESS, in place of V), s = w det W, with
+//   P = cA T + ct C,  dP = cA V + bT T + bC C + ct dC[V]   (MetricAct),
+// where only the scalars (from |T|^2, det T, T:V and C:V) are FP64: one FP64
+// operation takes as long as ~17 IMAD.WIDE. T, V: entries [3][3] at stride ST,
+// of one scale each (FxScale::kb kT, kV), shifted up by upT, upV (fx_room).
+// Magnitudes: |T|, |V|, |C| < 2^59, |dC| < 2^60, coefficients < 2^59 under a
+// common exponent per point, so all sums of limb products are < 2^63 and the
+// results < 2^61; a product loses ~2^-56 of the largest one.
+// A result is y 2^(E - 2044); E and the leading bit of the largest entry's high
+// word (0: all zero) per point are returned for the adjoint map, which gives
+// the element one exponent.
+struct FxPoint {
+  int E;          // exponent of the point's results
+  unsigned mag;   // largest magnitude (high words)
+};
+template <int ST, bool GRAD, bool HESS>
+__device__ __forceinline__ bool fx_point303(fx_t* T, fx_t* V, int upT, int upV, int kT, int kV, double s, FxPoint& pg,
+                                            FxPoint& ph, double& mu, double& tau) {
+  Limbs a[9], c[9], v[HESS ? 9 : 1];
+  kT -= upT;
+  kV -= upV;
+  const int kC = 2 * kT + 60 - 1023;
+  long long H = 0, M = 0;
+#pragma unroll
+  for (int i = 0; i < 9; ++i) {
+    a[i] = fx_split((fx_t)((unsigned long long)T[i * ST] << upT));
+    asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(H) : "r"(a[i].h), "r"(a[i].h));
+    asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(M) : "r"(a[i].h), "r"(a[i].l));
+  }
+  const double I1 = fx_to_f64(H + (M >> 29), {kC, 0u});
+  auto minor = [](const Limbs* x, const Limbs* y, int i, FxAcc& p, FxAcc& m) {   // x_p y_q and x_m y_n of entry i
+    const int r1 = 3 * ((i / 3 + 1) % 3), r2 = 3 * ((i / 3 + 2) % 3), c1 = (i % 3 + 1) % 3, c2 = (i % 3 + 2) % 3;
+    fx_mac(p, x[r1 + c1], y[r2 + c2].h, y[r2 + c2].l);
+    fx_mac(m, x[r1 + c2], y[r2 + c1].h, y[r2 + c1].l);
+  };
+  FxAcc at{0, 0};
+#pragma unroll
+  for (int i = 0; i < 9; ++i) {
+    FxAcc p{0, 0}, m{0, 0};
+    minor(a, a, i, p, m);
+    c[i] = fx_split((p.H - m.H) + ((p.M - m.M) >> 30));
+    if (i < 3) fx_mac(at, a[i], c[i].h, c[i].l);
+  }
+  tau = fx_to_f64(fx_value(at), {kT + kC + 60 - 1023, 0u});
+  const bool ok = tau > 0.0;
+  double t = 0.0, d = 0.0;
+  if constexpr (HESS) {
+    long long Ht = 0, Ma = 0, Mb = 0, Hd = 0, Mc = 0, Md = 0;   // (9 cross terms per sum)
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+      v[i] = fx_split((fx_t)((unsigned long long)V[i * ST] << upV));
+      asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(Ht) : "r"(a[i].h), "r"(v[i].h));
+      asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(Ma) : "r"(a[i].h), "r"(v[i].l));
+      asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(Mb) : "r"(a[i].l), "r"(v[i].h));
+      asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(Hd) : "r"(c[i].h), "r"(v[i].h));
+      asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(Mc) : "r"(c[i].h), "r"(v[i].l));
+      asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(Md) : "r"(c[i].l), "r"(v[i].h));
+    }
+    t = fx_to_f64(Ht + (Ma >> 30) + (Mb >> 30), {kT + kV + 60 - 1023, 0u});
+    d = fx_to_f64(Hd + (Mc >> 30) + (Md >> 30), {kC + kV + 60 - 1023, 0u});
+  }
+  // the scalars, as in MetricAct::init and dP
+  const double r = rcbrt_nr(ok ? tau : 1.0), r2 = r * r, it = r2 * r;
+  const double cA = ok ? ((2.0 / 3.0) * s) * r2 : 0.0;
+  const double c1t = cA * ((-2.0 / 3.0) * it);
+  const double ct = c1t * (0.5 * I1);
+  mu = fma((1.0 / 3.0) * I1, r2, -1.0);
+  auto ex = [](double x) { return (int)((unsigned)__double2hiint(x) >> 20 & 0x7ffu); };
+  if constexpr (GRAD) {
+    const int E = max(ex(cA) + kT, ex(ct) + kC);
+    const Limbs gT = fx_split(fx_from_f64(cA, E - kT, 6)), gC = fx_split(fx_from_f64(ct, E - kC, 6));
+    unsigned m = 0;
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+      FxAcc z{0, 0};
+      fx_mac(z, a[i], gT.h, gT.l);
+      fx_mac(z, c[i], gC.h, gC.l);
+      const fx_t y = ok ? fx_value(z) : 0;
+      T[i * ST] = y;
+      m = max(m, (unsigned)((int)(y >> 32) ^ ((int)(y >> 32) >> 31)));
+    }
+    pg = {E, m};
+  }
+  if constexpr (HESS) {
+    const double ctt = (ct * it) * (-5.0 / 3.0);
+    const double bT = c1t * d, bC = fma(c1t, t, ctt * d);
+    const int kD = kT + kV + 60 - 1023;
+    const int E = max(max(ex(cA) + kV, ex(bT) + kT), max(ex(bC) + kC, ex(ct) + kD));
+    const Limbs hV = fx_split(fx_from_f64(cA, E - kV, 6)), hT = fx_split(fx_from_f64(bT, E - kT, 6));
+    const Limbs hC = fx_split(fx_from_f64(bC, E - kC, 6)), hD = fx_split(fx_from_f64(ct, E - kD, 6));
+    unsigned m = 0;
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+      FxAcc p{0, 0}, n{0, 0}, z{0, 0};
+      minor(v, a, i, p, n);
+      minor(a, v, i, p, n);
+      const Limbs dc = fx_split((p.H - n.H) + ((p.M - n.M) >> 30));
+      fx_mac(z, dc, hD.h, hD.l);
+      fx_mac(z, v[i], hV.h, hV.l);
+      fx_mac(z, a[i], hT.h, hT.l);
+      fx_mac(z, c[i], hC.h, hC.l);
+      const fx_t y = ok ? fx_value(z) : 0;
+      V[i * ST] = y;
+      m = max(m, (unsigned)((int)(y >> 32) ^ ((int)(y >> 32) >> 31)));
+    }
+    ph = {E, m};
+  }
+  return ok;
+}
+
+// Largest values of NK keys over the group, with a barrier (as fx_group_exp).
+template <int GT, int NK>
+__device__ __forceinline__ void fx_group_max(int* key, int* s, int bar) {
+#pragma unroll
+  for (int k = 0; k < NK; ++k) key[k] = __reduce_max_sync(group_mask<GT>(), key[k]);
+  if constexpr (GT > 32) {
+    constexpr int G = GT / 32;
+    const int w = (threadIdx.x >> 5) % G;
+    if ((threadIdx.x & 31) == 0) {
+#pragma unroll
+      for (int k = 0; k < NK; ++k) s[w * NK + k] = key[k];
+    }
+    group_sync<GT>(bar);
+#pragma unroll
+    for (int k = 0; k < NK; ++k)
+#pragma unroll
+      for (int w2 = 0; w2 < G; ++w2) key[k] = max(key[k], s[w2 * NK + k]);
+  } else {
+    group_sync<GT>(bar);
+  }
+}
+
+// The key whose maximum over the points gives the element's exponent (L), and
+// the exponent field of the largest magnitude (as fx_group_exp's) from it.
+__device__ __forceinline__ int fx_point_key(const FxPoint& p) {
+  unsigned b;
+  asm("bfind.u32 %0, %1;" : "=r"(b) : "r"(p.mag));
+  return p.mag ? p.E + (int)b : -4000;
+}
+__device__ __forceinline__ int fx_point_emax(int L) { return L + 33 - 2044 + 1022; }
 }  // namespace tmop
