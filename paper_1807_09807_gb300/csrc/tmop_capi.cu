@@ -270,6 +270,7 @@ struct tmop_ctx {
   double* d_vec = nullptr;    // Krylov / Newton vectors, allocated on first use
   int nvec = 0;
   void* d_pa = nullptr;       // packed per-point Hessians (partial assembly), allocated on first use
+  short4* d_pa_exp = nullptr; // FP64 3D: exponents of the packed Hessians
   bool pa_valid = false;      // d_pa holds the linearisation of some x
   bool pa_compact = false;    // ... as compact records (OP_LINEARIZE_C / OP_HESS_PA_C)
   double* d_eta2 = nullptr;   // per-point weights of the composite second term
@@ -482,12 +483,19 @@ int linearize(tmop_ctx* c, const double* x, cudaStream_t s) {
     const size_t stride = (size_t)pa_stride_for(c->dim, c->Q, elt);
     CUDA_TRY(cudaMalloc(&c->d_pa, (size_t)elt * stride * (size_t)c->nelem));
   }
+  const bool pack = c->dim == 3 && c->precision == TMOP_FP64;   // for the fixed-point product
+  if (pack && !c->d_pa_exp) {
+    CUDA_TRY(cudaMalloc(&c->d_pa_exp, sizeof(short4) * (size_t)c->Q * (size_t)c->nelem));
+    c->base.pa_exp = c->d_pa_exp;
+  }
   c->pa_compact = c->ent[OP_LINEARIZE_C] && c->ent[OP_HESS_PA_C] && metric_is_lin(c->base.metric) &&
                   c->base.metric2 == 0 && c->base.wkind != WK_PER_QP;
   c->base.pa_stride = pa_stride_for(c->dim, c->Q, elt, c->pa_compact);
   c->pa_valid = false;
   int rc = launch_op(c, OP_LINEARIZE, x, nullptr, nullptr, nullptr, s);
   if (rc) return rc;
+  if (pack && pa_pack(static_cast<double*>(c->d_pa), c->base.pa_stride, c->d_pa_exp, c->nelem, c->Q, s) != 0)
+    return TMOP_ERR_CUDA;
   c->pa_valid = true;
   return TMOP_OK;
 }
@@ -529,6 +537,7 @@ int hessian_diagonal(tmop_ctx* c, bool inverse, cudaStream_t s) {
   dp.elem_nodes = b.elem_nodes;
   dp.pa = c->d_pa;
   dp.pa_stride = b.pa_stride;
+  dp.pa_exp = c->d_pa_exp;
   dp.diag = c->d_diag;
   memcpy(dp.B, b.B, sizeof(dp.B));
   memcpy(dp.G, b.G, sizeof(dp.G));
@@ -868,6 +877,7 @@ void tmop_destroy(tmop_ctx* c) {
   cudaFree(c->d_res);
   cudaFree(c->d_vec);
   cudaFree(c->d_pa);
+  cudaFree(c->d_pa_exp);
   cudaFree(c->d_eta2);
   cudaFree(c->d_x_init);
   cudaFree(c->d_diag);

@@ -16,6 +16,7 @@
 
 #include "tmop_device.cuh"
 #include "tmop_diag.h"
+#include "tmop_fixed.cuh"
 #include "tmop_kparams.h"
 
 namespace tmop {
@@ -169,7 +170,18 @@ __global__ void __launch_bounds__(kDiagWarps * 32) diag_kernel(const DiagParams 
             // packed index of (row a*DIM+b, column a*DIM+c), row <= column
             const int rr = a * DIM + b, cc = a * DIM + c;
             const int s = rr * DD - rr * (rr - 1) / 2 + (cc - rr);
-            for (int q = lane; q < QP; q += 32) r[q] = m * (A)He[(size_t)s * QP + q];
+            for (int q = lane; q < QP; q += 32) {
+              if constexpr (DIM == 3 && sizeof(R) == 8) {   // packed: (h 2^30 + l) 2^(E + 2 s_a - 57)
+                const short4 ex = __ldg(p.pa_exp + (size_t)e * QP + q);
+                const double v = He[(size_t)s * QP + q];
+                const long long i = ((long long)__double2hiint(v) << 30) + __double2loint(v);
+                const int sa = a == 0 ? ex.x : (a == 1 ? ex.y : ex.z);
+                r[q] = ex.w == kPaNan ? __longlong_as_double(0x7ff8000000000000LL)
+                                      : ldexp(m * (double)i, ex.w == kPaZero ? 0 : ex.w + 2 * sa - 57);
+              } else {
+                r[q] = m * (A)He[(size_t)s * QP + q];
+              }
+            }
           }
           __syncwarp();
           const A* T0 = tab[(b == 0) + (c == 0)];

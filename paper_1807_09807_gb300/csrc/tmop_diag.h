@@ -13,6 +13,7 @@ struct DiagParams {
   const int32_t* elem_nodes;  // [nelem][n^d] (unstructured) or null
   const void* pa;             // packed Hessians [nelem][pa_stride] (float or double)
   int pa_stride;
+  const short4* pa_exp;       // FP64 3D: exponents of the packed Hessians (tmop_fixed.cuh)
   double* diag;               // [d][nnode], accumulated (zero it first)
   double B[kMaxQ * kMaxN], G[kMaxQ * kMaxN], w1[kMaxQ];
   double delta, detW;         // restricted-movement term (delta = 0: none)

@@ -78,11 +78,11 @@ struct ElemCfg {
   static constexpr int FIT = 200 * 1024 / PER_WARP;
   static constexpr int WARPS = GT == 64 ? 1 : (TWO ? 6 : (FIT >= 8 ? 8 : (FIT < 1 ? 1 : FIT)));
   // Blocks per SM that bound the registers (0: no bound): 6 (168 registers)
-  // for the kernels that hold T and dT, 7 (144) for the others. 48^3 order-3
-  // hexes, gradient + Hessian action: 4.61 ms with 8 (spills), 3.75 with 6,
-  // 3.72 with 5; 24^3, stored-Hessian product 329 us with 8, 324 with 7, 334
-  // with 6; energy + gradient 232 us with 9, 227 with 7.
-  static constexpr int WANT = HV ? 6 : 7;
+  // for the kernels that hold T and dT, 7 or 8 (128) for the others. 48^3
+  // order-3 hexes, gradient + Hessian action: 4.61 ms with 8 (spills), 3.75
+  // with 6, 3.72 with 5; 24^3, stored-Hessian product 227 us with 8, 242 with
+  // 10; energy + gradient 232 us with 9, 227 with 7.
+  static constexpr int WANT = HV ? 6 : (OP == OP_HESS_PA ? 8 : 7);
   static constexpr int MINB = GT == 64 ? (FIT >= WANT ? WANT : FIT) : (TWO ? 2 : 0);
   // after the 1D tables: the product weight w_q0 w_q1 (w_q2) of every point
   static constexpr int WQ_OFF = 2 * kMaxQ * kMaxN + kMaxQ;
@@ -167,9 +167,11 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP, WIDE>::WARPS * ElemCf
   constexpr int GW = GT > 32 ? GT / 32 : 1;   // warps per element
   // mu303 with W = I: the pointwise stage of these FP64 3D kernels in fixed point (fx_point303)
   constexpr bool FX303 = FX && D == 3 && OP != OP_LINEARIZE && OP != OP_HESS_PA;
-  constexpr int NKEY = OP == OP_GRAD_HESS ? 2 : 1;
-  __shared__ short s_kq[FX303 ? WARPS : 1][FX303 ? NKEY * QP : 1];   // exponents of the points' results
-  __shared__ int s_key[FX303 ? WARPS : 1][GW * NKEY];
+  constexpr bool FXPA = FX && D == 3 && OP == OP_HESS_PA;   // and the product of the stored Hessians (fx_stored_product)
+  constexpr int NKEY = FXPA ? D : (OP == OP_GRAD_HESS ? 2 : 1);
+  constexpr int NKQ = (FXPA || (FX303 && OP != OP_ENERGY)) ? NKEY * QP : 1;
+  __shared__ short s_kq[NKQ > 1 ? WARPS : 1][NKQ];   // exponents of the points' results
+  __shared__ int s_key[NKQ > 1 ? WARPS : 1][GW * NKEY];
   __shared__ unsigned s_top[WARPS][GW];
   __shared__ unsigned s_mag[WARPS][GW * 2 * D];   // per warp and component: largest magnitudes of the group's warps
   R Wi[DD];
@@ -207,9 +209,12 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP, WIDE>::WARPS * ElemCf
     nodes.element(e, NDOF);
     // Partially assembled product: the stored values of this lane's first
     // point are loaded now, so their latency overlaps the gather and the
-    // v-contraction.
-    R hpre[NSH];
-    if constexpr (PA_APPLY) {
+    // v-contraction. (With two warps per element the registers they take cost
+    // more than they hide: 273 against 227 us on 24^3 order-3 hexes; a prefetch
+    // of the element's block into L2 instead: 236 us.)
+    constexpr bool HPRE = PA_APPLY && GT <= 32;
+    R hpre[HPRE ? NSH : 1];
+    if constexpr (HPRE) {
       if (lane < Shape<D, N, Q1>::QP) {
         const R* H0 = static_cast<const R*>(p.pa) + (size_t)e * p.pa_stride + lane;
 #pragma unroll
@@ -358,9 +363,9 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP, WIDE>::WARPS * ElemCf
       if constexpr (RAW) return fx_to_f64(reinterpret_cast<const fx_t*>(buf)[i * QP + q], sc[i / D]);
       else return buf[i * QP + q];
     };
-    int key[FX303 ? NKEY : 1];
+    int key[D];
 #pragma unroll
-    for (int k = 0; k < (FX303 ? NKEY : 1); ++k) key[k] = -4000;
+    for (int k = 0; k < D; ++k) key[k] = -4000;
     // FP64: largest magnitude (high word) per component of the fields the
     // adjoint map takes (OP_GRAD_HESS: the gradient's, then the Hessian action's)
     unsigned rmag[FX ? 2 * D : 1] = {};
@@ -371,12 +376,24 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP, WIDE>::WARPS * ElemCf
         const R* H = static_cast<const R*>(p.pa) + (size_t)e * p.pa_stride + q;
         // all NS loads are issued before the first use, so their latencies overlap
         R h[NS];
-        if (q == lane) {
+        if (HPRE && q == lane) {
 #pragma unroll
-          for (int t = 0; t < NS; ++t) h[t] = hpre[t];
+          for (int t = 0; t < NS; ++t) h[t] = hpre[HPRE ? t : 0];
         } else {
 #pragma unroll
           for (int t = 0; t < NS; ++t) h[t] = __ldg(H + (size_t)t * QP);
+        }
+        if constexpr (FXPA) {
+          const short4 ex = __ldg(p.pa_exp + (size_t)e * QP + q);
+          FxPoint pt[D];
+          fx_stored_product<QP>(reinterpret_cast<fx_t*>(Abuf) + q, h, ex, upA, sA, pt);
+          const bool bad = ex.w == kPaNan || sA[0].nan || sA[1].nan || sA[2].nan;   // NaN everywhere
+#pragma unroll
+          for (int a = 0; a < D; ++a) {
+            key[a] = max(key[a], bad ? 32000 : fx_point_key(pt[a]));
+            s_kq[warp][a * QP + q] = (short)(pt[a].mag ? pt[a].E : -16000);
+          }
+          continue;
         }
         R dA[DD], y[DD];
 #pragma unroll
@@ -797,9 +814,10 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP, WIDE>::WARPS * ElemCf
 #pragma unroll
           for (int c = 0; c < D; ++c) er[c] = pass == 0 ? er2[D + c] : er2[c];
           if (FX303 && fx303) {
-            const int k = pass == 0 ? 1 : 0, L = pass == 0 ? key[NKEY - 1] : key[0];
+            const int k = pass == 0 ? 1 : 0, L = pass == 0 ? key[1] : key[0];
+            const int Ls[3] = {L, L, L};
             er[0] = er[1] = er[D - 1] = fx_point_emax(L);
-            adj3_fx<N, Q1, D, GT, true>(p.fx, er, P0, Rin, lane, bar, s_kq[warp] + k * QP, L);
+            adj3_fx<N, Q1, D, GT, true>(p.fx, er, P0, Rin, lane, bar, s_kq[warp] + k * QP, 0, Ls);
           } else {
             adj3_fx<N, Q1, D, GT>(p.fx, er, P0, Rin, lane, bar);
           }
@@ -820,11 +838,13 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP, WIDE>::WARPS * ElemCf
       // ---- adjoint contraction and scatter
       if constexpr (FX) {
         int er[D];
-        if (FX303 && fx303) {
-          if constexpr (FX303) {
-            fx_group_max<GT, 1>(key, s_key[warp], bar);
-            er[0] = er[1] = er[2] = fx_point_emax(key[0]);
-            adj3_fx<N, Q1, D, GT, true>(p.fx, er, P0, P1, lane, bar, s_kq[warp], key[0]);
+        if (FXPA || (FX303 && fx303)) {
+          if constexpr (FXPA || FX303) {
+            fx_group_max<GT, NKEY>(key, s_key[warp], bar);
+            if constexpr (!FXPA) key[1] = key[2] = key[0];
+#pragma unroll
+            for (int c = 0; c < D; ++c) er[c] = fx_point_emax(key[c]);
+            adj3_fx<N, Q1, D, GT, true>(p.fx, er, P0, P1, lane, bar, s_kq[warp], FXPA ? QP : 0, key);
           }
         } else {
           fx_group_exp<GT, D>(rmag, er, s_mag[warp], bar);

@@ -329,11 +329,11 @@ __device__ __forceinline__ fx_t fx_align(fx_t y, int sh) {
 
 // 3D adjoint map. P1: R[NC][3][Q][Q][Q] (double) -> P0: [NC][3][N][Q][Q] ->
 // P1: [NC][2][N][N][Q] -> P0: Y (FxNodal, double).
-// RAW: R is in fixed point instead, point q at exponent kq[q] (FxPoint::E) of an
-// element whose largest key is L (all components then share one exponent).
+// RAW: R is in fixed point instead, point q of component c at exponent
+// kq[c kst + q] (FxPoint::E) in an element whose largest key is L[c].
 template <int N, int Q1, int NC, int GT, bool RAW = false>
 __device__ __forceinline__ void adj3_fx(const FxTab& T, const int (&em)[NC], double* P0d, double* P1d, int lane, int bar,
-                                        const short* kq = nullptr, int L = 0) {
+                                        const short* kq = nullptr, int kst = 0, const int* L = nullptr) {
   constexpr int NNQ = N * N * Q1, NQQ = N * Q1 * Q1, QQ = Q1 * Q1, QQQ = Q1 * Q1 * Q1;
   fx_t *P0 = reinterpret_cast<fx_t*>(P0d), *P1 = reinterpret_cast<fx_t*>(P1d);
   auto pick = [&](int c) {
@@ -341,6 +341,12 @@ __device__ __forceinline__ void adj3_fx(const FxTab& T, const int (&em)[NC], dou
 #pragma unroll
     for (int k = 1; k < NC; ++k) e = c == k ? em[k] : e;
     return e;
+  };
+  auto pickL = [&](int c) {
+    int l = L[0];
+#pragma unroll
+    for (int k = 1; k < NC; ++k) l = c == k ? L[k] : l;
+    return l;
   };
 #pragma unroll 1
   for (int t = lane; t < NC * QQ; t += GT) {                  // (c, q1, q0): lines along z
@@ -352,9 +358,9 @@ __device__ __forceinline__ void adj3_fx(const FxTab& T, const int (&em)[NC], dou
     int al[RAW ? Q1 : 1];
     if constexpr (RAW) {
 #pragma unroll
-      for (int q = 0; q < Q1; ++q) al[q] = kq[q * QQ + q01] - L + T.rin - 33;
+      for (int q = 0; q < Q1; ++q) al[q] = kq[c * kst + q * QQ + q01] - pickL(c) + T.rin - 33;
     }
-    auto in = [&](int i, int q) {
+    auto in = [&](int i, int q) -> fx_t {
       if constexpr (RAW) return fx_align(reinterpret_cast<const fx_t*>(s)[i], al[q]);
       else return fx_from_f64(s[i], e, sh);
     };
@@ -636,6 +642,49 @@ __device__ __forceinline__ void fx_group_max(int* key, int* s, int bar) {
       for (int w2 = 0; w2 < G; ++w2) key[k] = max(key[k], s[w2 * NK + k]);
   } else {
     group_sync<GT>(bar);
+  }
+}
+
+// ---------------------------------------------------------------- stored Hessians
+// The FP64 3D stored Hessians are packed for the fixed-point product by
+// pa_pack (tmop_pa_pack.cu): the 45 entries H_(r,c) of a point, r = 3 a + b, as
+//   H_(r,c) = (h 2^30 + l) 2^(E + s_a + s_c - 57),  |h| <= 2^27, 0 <= l < 2^30,
+// (h, l) in the place of the double's high and low word, and {s_0, s_1, s_2, E}
+// beside them; s_a is half the exponent of block (a, a), so that directions
+// along which elements are long or short keep their digits.
+constexpr int kPaNan = 32767, kPaZero = -20000;   // E of a point with a non-finite entry, of one without any
+
+// y = H dA at one point: h the packed entries, ex their exponents; A: dA in
+// fixed point at stride ST (rows' scales kb), shifted up by up (fx_room); the
+// rows are first brought to one exponent under the scaling of H. y replaces
+// dA; pt: per row.
+template <int ST>
+__device__ __forceinline__ void fx_stored_product(fx_t* A, const double* h, short4 ex, int up, const FxScale* sA,
+                                                  FxPoint* pt) {
+  const int s[3] = {ex.x, ex.y, ex.z};
+  int m[3], mx = -100000;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    m[a] = sA[a].kb + s[a];
+    mx = max(mx, m[a]);
+  }
+  Limbs d[9];
+#pragma unroll
+  for (int i = 0; i < 9; ++i)
+    d[i] = fx_split((fx_t)((unsigned long long)A[i * ST] << up) >> min(mx - m[i / 3], 63));
+#pragma unroll
+  for (int a = 0; a < 3; ++a) pt[a] = {s[a] + ex.w + mx - up + 1024, 0u};
+#pragma unroll
+  for (int r = 0; r < 9; ++r) {
+    FxAcc z{0, 0};   // 9 terms: |H| < 9 2^56, |M| < 9 (2^59 + 2^57) < 2^63
+#pragma unroll
+    for (int c = 0; c < 9; ++c) {
+      const int lo = r < c ? r : c, hi = r < c ? c : r, t = lo * 9 - lo * (lo - 1) / 2 + hi - lo;
+      fx_mac(z, d[c], __double2hiint(h[t]), __double2loint(h[t]));
+    }
+    const fx_t y = fx_value(z);
+    A[r * ST] = y;
+    pt[r / 3].mag = max(pt[r / 3].mag, (unsigned)((int)(y >> 32) ^ ((int)(y >> 32) >> 31)));
   }
 }
 

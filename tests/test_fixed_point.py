@@ -88,3 +88,29 @@ def test_a_value_that_is_not_finite_spoils_its_elements_only(dim, order, nq, met
     free = m.fixed == 0
     assert np.isnan(z[free & hit[None, :]]).all()
     assert np.array_equal(z[free & ~hit[None, :]], y[free & ~hit[None, :]])
+
+
+@pytest.mark.parametrize("dim,order,nq,metric", CASES)
+def test_stored_product_with_values_that_are_not_finite(dim, order, nq, metric):
+    """A direction that is not finite at one node spoils that node's elements
+    only."""
+    import torch
+    from paper_1807_09807_gb300 import tmop as tm
+    m = _mesh(dim, order, nq, metric)
+    ctx = tm.Context.from_mesh(m)
+    ctx.set_deterministic(True)
+    x = torch.tensor(m.x, device="cuda")
+    v = torch.tensor(np.random.default_rng(3).standard_normal(m.x.shape), device="cuda")
+    ctx.linearize(x)
+    y = ctx.hess_apply_pa(v).cpu().numpy()
+    node = int(np.flatnonzero(m.fixed[0] == 0)[0])
+    hit = np.zeros(m.nnode, dtype=bool)
+    for row in m.elem_nodes:
+        if node in row:
+            hit[row] = True
+    free = m.fixed == 0
+    w = v.clone()
+    w[:, node] = float("nan")   # (every component: a stored Hessian need not mix them)
+    z = ctx.hess_apply_pa(w).cpu().numpy()
+    assert np.isnan(z[free & hit[None, :]]).all()
+    assert np.array_equal(z[free & ~hit[None, :]], y[free & ~hit[None, :]])
