@@ -190,7 +190,9 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP, WIDE>::WARPS * ElemCf
   __syncthreads();
 
   double accF = 0.0, accMin = INFINITY;
-  const int warps = blockDim.x / GT, nwarps_total = gridDim.x * warps;   // (small meshes: fewer than WARPS, launch_elem)
+  // elements in flight per block (FP64, small meshes: fewer than WARPS, launch_elem_impl)
+  const int warps = FX ? (int)blockDim.x / GT : WARPS;
+  const int nwarps_total = gridDim.x * warps;
   // (the product from compact records, OP_HESS_PA_C, is pac_kernel in tmop_pa_compact.cu)
   constexpr bool PA_APPLY = OP == OP_HESS_PA;
   constexpr bool EG = OP == OP_ENERGY_GRAD;                // gradient + energy partials
@@ -887,7 +889,7 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP, WIDE>::WARPS * ElemCf
     __syncthreads();
     if (threadIdx.x == 0) {
       double f = 0.0, m = INFINITY;
-      for (int w = 0; w < (int)(blockDim.x / 32); ++w) { f += redF[w]; m = fmin(m, redM[w]); }
+      for (int w = 0; w < (FX ? (int)blockDim.x / 32 : BW); ++w) { f += redF[w]; m = fmin(m, redM[w]); }
       p.part_F[blockIdx.x] = f;
       p.part_min[blockIdx.x] = m;
     }
@@ -898,7 +900,9 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP, WIDE>::WARPS * ElemCf
 template <int D, int N, int Q1, class R, int OP, bool WIDE>
 int launch_elem_impl(const KParams& p, int grid, void* stream) {
   using Cfg = ElemCfg<D, N, Q1, R, OP, WIDE>;
-  const int w = (p.nelem + grid - 1) / grid, threads = ((w < Cfg::WARPS ? w : Cfg::WARPS) * Cfg::GT + 31) / 32 * 32;
+  const int w = (p.nelem + grid - 1) / grid;
+  const int threads = sizeof(R) == 4 ? Cfg::WARPS * Cfg::GT
+                                     : ((w < Cfg::WARPS ? w : Cfg::WARPS) * Cfg::GT + 31) / 32 * 32;
   elem_kernel<D, N, Q1, R, OP, WIDE><<<grid, threads, Cfg::smem_bytes(), (cudaStream_t)stream>>>(p);
   return (int)cudaGetLastError();
 }
@@ -917,12 +921,12 @@ int prepare_elem_impl(int nelem, int* grid) {
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (per_sm < 1) return (int)cudaErrorInvalidConfiguration;
-  // Fewer full blocks than SMs: the elements are spread over all SMs in
+  // FP64, fewer full blocks than SMs: the elements are spread over all SMs in
   // smaller blocks instead, since the warps of a block share one narrow FP64
   // pipe.
   const int need = (nelem + Cfg::WARPS - 1) / Cfg::WARPS;
   const int full = per_sm * sms;
-  if (need < sms) {
+  if (sizeof(R) == 8 && need < sms) {
     const int w = (nelem + sms - 1) / sms;
     *grid = (nelem + w - 1) / w;
   } else {
