@@ -2,8 +2,9 @@
 //
 //  * Dual<R>: forward-mode dual numbers. The Hessian action needs
 //    d^2mu/dT^2 : dT (Section 3.4); evaluating the first derivative P(T) on
-//    T + eps dT in dual arithmetic yields exactly that directional derivative,
-//    so every metric is written once, generically in its scalar type.
+//    T + eps dT in dual arithmetic yields exactly that directional derivative
+//    (mu302 and mu98 in the FP32 kernels; MetricLin, MetricAct and Metric302
+//    write it out).
 //  * metric_P: mu and P = dmu/dT for the Table 3.1 / Section 3.2 metrics in
 //    the invariants I1 = |T|^2, tau = det T, C = cof T.
 //  * fwd2/fwd3, adj2/adj3: sum-factorised tensor-product contractions of one
@@ -321,7 +322,8 @@ __device__ __forceinline__ bool metric_P(int id, const S* T, S& mu, S* P) {
 }
 
 // ---------------------------------------------------------------- linearised metric
-// For metrics written in I1 = |T|^2 and tau = det T (all but mu302), the
+// For metrics written in I1 = |T|^2 (mu98: |T - I|^2, with X = T - I for T
+// in P and in the first and second term of dP) and tau = det T (all but mu302), the
 // first derivative is P = 2 mu_1 T + mu_t C and, with dI1 = 2 T:dT and
 // dtau = C:dT (C = cof T, the derivative of det),
 //   dP = 2 mu_1 dT + 2 (mu_11 dI1 + mu_1t dtau) T + (mu_1t dI1 + mu_tt dtau) C + mu_t dC,
@@ -332,15 +334,24 @@ template <int D, class R>
 struct MetricLin {
   static constexpr int DD = D * D;
   R T[DD], C[DD];
+  R X[D];   // diagonal of the matrix I1 is the norm of: T, or T - I (mu98)
   R m1, mt, m11, m1t, mtt;
   bool ok;
+
+  __device__ __forceinline__ R x(int i) const { return i % (D + 1) == 0 ? X[i / (D + 1)] : T[i]; }
 
   __device__ __forceinline__ bool init(int id, const R* Tin) {
 #pragma unroll
     for (int i = 0; i < DD; ++i) T[i] = Tin[i];
+#pragma unroll
+    for (int d = 0; d < D; ++d) X[d] = T[d * (D + 1)];
+    if (sizeof(R) == 8 && id == 98) {
+#pragma unroll
+      for (int d = 0; d < D; ++d) X[d] -= R(1);
+    }
     R I1 = R(0);
 #pragma unroll
-    for (int i = 0; i < DD; ++i) I1 = fma(T[i], T[i], I1);
+    for (int i = 0; i < DD; ++i) I1 = fma(x(i), x(i), I1);
     cof_m<D>(T, C);
     R tau = R(0);
 #pragma unroll
@@ -362,6 +373,8 @@ struct MetricLin {
       m1 = R(1) + it2; mt = R(-2) * I1 * it2 * it; m1t = R(-2) * it2 * it; mtt = R(6) * I1 * it2 * it2;
     } else if (id == 9) {     // tau I1 + I1 / tau - 4 tau (2D)
       m1 = tau + it; mt = I1 - I1 * it2 - R(4); m1t = R(1) - it2; mtt = R(2) * I1 * it2 * it;
+    } else if (sizeof(R) == 8 && id == 98) {    // |T - I|^2 / tau = I1 / tau with I1 = |T - I|^2
+      m1 = it; mt = -I1 * it2; m1t = -it2; mtt = R(2) * I1 * it2 * it;
     } else if (id == 77) {    // (tau - 1/tau)^2 / 2
       const R sdiff = tau - it, ds = R(1) + it2;
       mt = sdiff * ds; mtt = ds * ds - R(2) * sdiff * it2 * it;
@@ -376,7 +389,7 @@ struct MetricLin {
     R dI1 = R(0), dtau = R(0);
 #pragma unroll
     for (int i = 0; i < DD; ++i) {
-      dI1 = fma(T[i], dT[i], dI1);
+      dI1 = fma(x(i), dT[i], dI1);
       dtau = fma(C[i], dT[i], dtau);
     }
     dI1 *= R(2);
@@ -406,7 +419,7 @@ struct MetricLin {
 #undef TMOP_DMINOR
     }
 #pragma unroll
-    for (int i = 0; i < DD; ++i) out[i] = fma(a, dT[i], fma(bT, T[i], fma(bC, C[i], mdC[i])));
+    for (int i = 0; i < DD; ++i) out[i] = fma(a, dT[i], fma(bT, x(i), fma(bC, C[i], mdC[i])));
   }
 };
 
@@ -421,13 +434,18 @@ template <int D, class R>
 struct MetricAct {
   static constexpr int DD = D * D;
   R T[DD], C[DD];
+  R X[D];   // as MetricLin's
   R cA, c11, c1t, ctt, ct;
+
+  __device__ __forceinline__ R x(int i) const { return i % (D + 1) == 0 ? X[i / (D + 1)] : T[i]; }
 
   __device__ __forceinline__ bool init(int id, const R* Tin, R s) {
     if constexpr (D == 3) {
       if (id == 303) {  // I1 tau^{-2/3} / 3 - 1: mu_11 = 0
 #pragma unroll
         for (int i = 0; i < DD; ++i) T[i] = Tin[i];
+#pragma unroll
+        for (int d = 0; d < D; ++d) X[d] = T[d * (D + 1)];
         R I1 = R(0);
 #pragma unroll
         for (int i = 0; i < DD; ++i) I1 = fma(T[i], T[i], I1);
@@ -454,6 +472,8 @@ struct MetricAct {
       T[i] = L.T[i];
       C[i] = L.C[i];
     }
+#pragma unroll
+    for (int d = 0; d < D; ++d) X[d] = L.X[d];
     const R s2 = R(2) * s;
     cA = s2 * L.m1;
     c11 = (R(2) * s2) * L.m11;
@@ -467,7 +487,7 @@ struct MetricAct {
     R t = R(0), d = R(0);
 #pragma unroll
     for (int i = 0; i < DD; ++i) {
-      t = fma(T[i], dT[i], t);
+      t = fma(x(i), dT[i], t);
       d = fma(C[i], dT[i], d);
     }
     const R bT = fma(c11, t, c1t * d);
@@ -492,7 +512,78 @@ struct MetricAct {
 #undef TMOP_DMINOR
     }
 #pragma unroll
-    for (int i = 0; i < DD; ++i) out[i] = fma(cA, dT[i], fma(bT, T[i], fma(bC, C[i], mdC[i])));
+    for (int i = 0; i < DD; ++i) out[i] = fma(cA, dT[i], fma(bT, x(i), fma(bC, C[i], mdC[i])));
+  }
+};
+
+// mu302 = I1 K / (9 tau^2) - 1 (3D), K = |C|^2, C = cof T: with the
+// symmetric bilinear form cof'(A)[B] (the derivative of the cofactor matrix at A
+// in direction B) dK/dT = 2 N, N = cof'(T)[C], and
+//   P = a T + b N - c C,  a = 2 K / (9 tau^2), b = 2 I1 / (9 tau^2), c = 2 I1 K / (9 tau^3),
+//   dP = a dT + b dN - c dC + da T + db N - dc C,
+//   dC = cof'(T)[dT], dN = cof'(dT)[C] + cof'(T)[dC].
+// s scales P and dP.
+template <class R>
+struct Metric302 {
+  R T[9], C[9], N[9], I1, K, it, a, b, c, f;
+
+  // out += cof'(A)[B]
+  static __device__ __forceinline__ void dcof(const R* A, const R* B, R* out) {
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+      const int r1 = 3 * ((i / 3 + 1) % 3), r2 = 3 * ((i / 3 + 2) % 3), c1 = (i % 3 + 1) % 3, c2 = (i % 3 + 2) % 3;
+      out[i] = fma(A[r1 + c1], B[r2 + c2], out[i]);
+      out[i] = fma(B[r1 + c1], A[r2 + c2], out[i]);
+      out[i] = fma(-A[r1 + c2], B[r2 + c1], out[i]);
+      out[i] = fma(-B[r1 + c2], A[r2 + c1], out[i]);
+    }
+  }
+  __device__ __forceinline__ bool init(const R* Tin, R s) {
+    I1 = R(0);
+    K = R(0);
+    R tau = R(0);
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+      T[i] = Tin[i];
+      N[i] = R(0);
+    }
+    cof_m<3>(T, C);
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+      I1 = fma(T[i], T[i], I1);
+      K = fma(C[i], C[i], K);
+      if (i < 3) tau = fma(T[i], C[i], tau);
+    }
+    if (!(tau > R(0))) return false;
+    dcof(T, C, N);
+    it = R(1) / tau;
+    f = R(2.0 / 9.0) * s * it * it;
+    a = f * K;
+    b = f * I1;
+    c = a * I1 * it;
+    return true;
+  }
+  __device__ __forceinline__ R P(int i) const { return fma(a, T[i], fma(b, N[i], -c * C[i])); }
+  __device__ __forceinline__ void dP(const R* dT, R* out) const {
+    R t = R(0), n = R(0), d = R(0);   // dI1 / 2, dK / 2, dtau
+    R dC[9];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+      t = fma(T[i], dT[i], t);
+      n = fma(N[i], dT[i], n);
+      d = fma(C[i], dT[i], d);
+      dC[i] = R(0);
+      out[i] = R(0);
+    }
+    const R dt = R(2) * it * d;   // 2 dtau / tau
+    const R da = fma(R(2) * f, n, -a * dt), db = fma(R(2) * f, t, -b * dt);
+    const R dc = it * fma(R(2), fma(a, t, b * n), -R(3) * c * d);
+    dcof(T, dT, dC);
+    dcof(dT, C, out);
+    dcof(T, dC, out);
+#pragma unroll
+    for (int i = 0; i < 9; ++i)
+      out[i] = fma(b, out[i], fma(a, dT[i], fma(-c, dC[i], fma(da, T[i], fma(db, N[i], -dc * C[i])))));
   }
 };
 

@@ -79,10 +79,11 @@ struct ElemCfg {
   static constexpr int WARPS = GT == 64 ? 1 : (TWO ? 6 : (FIT >= 8 ? 8 : (FIT < 1 ? 1 : FIT)));
   // Blocks per SM that bound the registers (0: no bound): 6 (168 registers)
   // for the kernels that hold T and dT, 7 or 8 (128) for the others. 48^3
-  // order-3 hexes, gradient + Hessian action: 4.61 ms with 8 (spills), 3.75
-  // with 6, 3.72 with 5; 24^3, stored-Hessian product 227 us with 8, 242 with
-  // 10; energy + gradient 232 us with 9, 227 with 7.
-  static constexpr int WANT = HV ? 6 : (OP == OP_HESS_PA ? 8 : 7);
+  // order-3 hexes (5 points per axis), gradient + Hessian action: 4.61 ms with
+  // 8 (spills), 3.83 with 6, 3.70 with 5; 32^3 order 2 (4 points) 0.54-0.59
+  // with 6; 24^3, stored-Hessian product 227 us with 8, 242 with 10; energy +
+  // gradient 232 us with 9, 227 with 7.
+  static constexpr int WANT = HV ? (OP == OP_GRAD_HESS && Q1 == 5 ? 5 : 6) : (OP == OP_HESS_PA ? 8 : 7);
   static constexpr int MINB = GT == 64 ? (FIT >= WANT ? WANT : FIT) : (TWO ? 2 : 0);
   // after the 1D tables: the product weight w_q0 w_q1 (w_q2) of every point
   static constexpr int WQ_OFF = 2 * kMaxQ * kMaxN + kMaxQ;
@@ -105,23 +106,35 @@ __device__ __forceinline__ void times_w2(const KParams& p, const R* M, R* out) {
     }
 }
 
-// Metrics not written in I1 = |T|^2 and tau = det T alone (mu302 also needs
-// |cof T|^2, mu98 needs T - I): their second derivative comes from
-// forward-mode dual numbers instead of MetricLin.
-__device__ __forceinline__ bool metric_dual(int id) { return id == 302 || id == 98; }
+// The FP32 kernels take the second derivative of mu302 and mu98 from
+// forward-mode dual numbers: the closed forms' rounding is larger there (order-1
+// hexes, mu302: 1.6e-7 against 1.3e-7 of FP64). In FP64 it is smaller
+// (Metric302, and MetricLin for mu98: 1.8e-15 against 2.9e-15 on order-2
+// hexes), and the 45 entries of mu302 at 24^3 5^3 points take 1.9 ms, not 15.6.
+template <class R>
+__device__ __forceinline__ bool metric_dual(int id) { return sizeof(R) == 4 && (id == 302 || id == 98); }
 
-// dP of metric `id` at T in direction dT (closed form, or dual numbers)
+// dP of metric `id` at T in direction dT
 template <int D, class R>
 __device__ __forceinline__ bool metric_dP(int id, const R* T, const R* dT, R* S) {
-  constexpr int DD = D * D;
-  if (metric_dual(id)) {
-    Dual<R> Td[DD], Pd[DD], mud;
+  if constexpr (sizeof(R) == 4) {
+    if (metric_dual<R>(id)) {
+      Dual<R> Td[D * D], Pd[D * D], mud;
 #pragma unroll
-    for (int i = 0; i < DD; ++i) Td[i] = Dual<R>{T[i], dT[i]};
-    const bool ok = metric_P<D>(id, Td, mud, Pd);
+      for (int i = 0; i < D * D; ++i) Td[i] = Dual<R>{T[i], dT[i]};
+      const bool ok = metric_P<D>(id, Td, mud, Pd);
 #pragma unroll
-    for (int i = 0; i < DD; ++i) S[i] = Pd[i].d;
-    return ok;
+      for (int i = 0; i < D * D; ++i) S[i] = Pd[i].d;
+      return ok;
+    }
+  }
+  if constexpr (D == 3 && sizeof(R) == 8) {
+    if (id == 302) {
+      Metric302<R> L;
+      const bool ok = L.init(T, R(1));
+      if (ok) L.dP(dT, S);
+      return ok;
+    }
   }
   MetricLin<D, R> L;
   const bool ok = L.init(id, T);
@@ -474,7 +487,7 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP, WIDE>::WARPS * ElemCf
         // the metric's terms for both. For an (|T|^2, det T) metric
         // P = 2 mu_1 T + mu_t C, i.e. s P = cA T + ct C with MetricAct's scaled
         // coefficients (mu14 = |T - I|^2 is the exception: its P from metric_P);
-        // the other metrics take P and dP from one dual-number evaluation.
+        // mu302 from the terms of Metric302.
         const R s = wq * detW;
         R dA[DD], dT[DD], Sg[DD], Sh[DD];
 #pragma unroll
@@ -494,15 +507,15 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP, WIDE>::WARPS * ElemCf
             }
         }
         bool ok;
-        if (metric_dual(p.metric)) {
-          Dual<R> Td[DD], Pd[DD], mud;
+        if (D == 3 && p.metric == 302) {   // (FP64 kernels only)
+          if constexpr (D == 3) {
+            Metric302<R> L;
+            ok = L.init(T, s);
+            if (ok) {
+              L.dP(dT, Sh);
 #pragma unroll
-          for (int i = 0; i < DD; ++i) Td[i] = Dual<R>{T[i], dT[i]};
-          ok = metric_P<D>(p.metric, Td, mud, Pd);
-#pragma unroll
-          for (int i = 0; i < DD; ++i) {
-            Sg[i] = s * Pd[i].v;
-            Sh[i] = s * Pd[i].d;
+              for (int i = 0; i < DD; ++i) Sg[i] = L.P(i);
+            }
           }
         } else {
           MetricAct<D, R> L;
@@ -514,7 +527,7 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP, WIDE>::WARPS * ElemCf
               metric_P<D>(p.metric, T, mu, Sg, s);
             } else {
 #pragma unroll
-              for (int i = 0; i < DD; ++i) Sg[i] = fma(L.cA, L.T[i], L.ct * L.C[i]);
+              for (int i = 0; i < DD; ++i) Sg[i] = fma(L.cA, L.x(i), L.ct * L.C[i]);
             }
           }
         }
@@ -565,8 +578,55 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP, WIDE>::WARPS * ElemCf
         R* H = static_cast<R*>(p.pa) + (size_t)e * p.pa_stride + q;
         const R s = wq * detW;
         MetricLin<D, R> L;
-        const bool lin = !metric_dual(p.metric);
+        const bool lin = p.metric != 302 && !metric_dual<R>(p.metric);
         bool ok = lin ? L.init(p.metric, T) : true;
+        if constexpr (D == 3 && sizeof(R) == 8) {
+          if (!lin && p.wkind == WK_IDENTITY && !p.metric2) {
+            // mu302 with W = I, in closed form: with G = T^t T, M = I1 T - T G
+            // (= dK/dT / 2), a = 2 s K / (9 tau^2), b = 2 s I1 / (9 tau^2),
+            // c = 2 s I1 K / (9 tau^3) as in Metric302,
+            //   H[(a,b),(c,d)] = (a + b I1) d_ac d_bd + (da_cd + 2 b T_cd) T_ab + db_cd M_ab - dc_cd C_ab
+            //                    - b (d_ac G_bd + d_bd (T T^t)_ac + T_ad T_cb) - c dC_ab/dT_cd,
+            // da, db, dc the derivatives of a, b, c by T_cd (nine directions of
+            // dP took 15.6 ms, 1.9 now, on 24^3 order-3 hexes)
+            Metric302<R> Q;
+            ok = Q.init(T, s);
+            R G[9], TT[9];
+#pragma unroll
+            for (int i = 0; i < 9; ++i) {
+              const int r = i / 3, c = i % 3;
+              G[i] = fma(T[r], T[c], fma(T[3 + r], T[3 + c], T[6 + r] * T[6 + c]));
+              TT[i] = fma(T[3 * r], T[3 * c], fma(T[3 * r + 1], T[3 * c + 1], T[3 * r + 2] * T[3 * c + 2]));
+            }
+            int off3 = 0;
+#pragma unroll
+            for (int kl = 0; kl < 9; ++kl) {
+              const int c = kl / 3, d = kl % 3;
+              const R dt = R(-2) * Q.it * Q.C[kl];
+              const R pT = fma(R(2) * Q.f, Q.N[kl], fma(Q.a, dt, R(2) * Q.b * T[kl]));
+              const R pM = fma(R(2) * Q.f, T[kl], Q.b * dt);
+              const R pC = -Q.it * fma(R(2), fma(Q.a, T[kl], Q.b * Q.N[kl]), R(-3) * Q.c * Q.C[kl]);
+#pragma unroll
+              for (int mn = kl; mn < 9; ++mn) {
+                const int a = mn / 3, b = mn % 3;
+                R v = fma(pT, T[mn], fma(pM, Q.N[mn], pC * Q.C[mn]));
+                R u = T[a * 3 + d] * T[c * 3 + b];
+                if (a == c) u += G[b * 3 + d];
+                if (b == d) u += TT[a * 3 + c];
+                v = fma(-Q.b, u, v);
+                if (mn == kl) v += fma(Q.b, Q.I1, Q.a);
+                if (a != c && b != d) {
+                  const int ee = 3 - a - c, ff = 3 - b - d;
+                  const bool plus = (c == (a + 1) % 3) == (d == (b + 1) % 3);
+                  v = fma(plus ? -Q.c : Q.c, T[ee * 3 + ff], v);
+                }
+                H[(size_t)(off3 + mn - kl) * QP] = ok ? v : R(0);
+              }
+              off3 += 9 - kl;
+            }
+            continue;
+          }
+        }
         if constexpr (D == 3) {
           if (lin && p.wkind == WK_IDENTITY && !p.metric2) {
             // W = I, an (|T|^2, det T) metric: the 45 entries in closed form,
@@ -580,12 +640,12 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP, WIDE>::WARPS * ElemCf
 #pragma unroll
             for (int kl = 0; kl < 9; ++kl) {
               const int c = kl / 3, d = kl % 3;
-              const R Pc = fma(R(4) * m11, T[kl], R(2) * m1t * L.C[kl]);
-              const R Qc = fma(R(2) * m1t, T[kl], mtt * L.C[kl]);
+              const R Pc = fma(R(4) * m11, L.x(kl), R(2) * m1t * L.C[kl]);
+              const R Qc = fma(R(2) * m1t, L.x(kl), mtt * L.C[kl]);
 #pragma unroll
               for (int mn = kl; mn < 9; ++mn) {
                 const int a = mn / 3, b = mn % 3;
-                R v = fma(Pc, T[mn], Qc * L.C[mn]);
+                R v = fma(Pc, L.x(mn), Qc * L.C[mn]);
                 if (mn == kl) v += R(2) * m1;
                 if (a != c && b != d) {
                   const int ee = 3 - a - c, ff = 3 - b - d;
@@ -611,13 +671,15 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP, WIDE>::WARPS * ElemCf
               dT[a * D + b] = a == k ? (p.wkind == WK_IDENTITY ? R(l == b) : Wi[l * D + b]) : R(0);
           if (lin) {
             if (ok) L.dP(dT, S);
-          } else {
+          } else if constexpr (sizeof(R) == 4) {
             Dual<R> Td[DD], Pd[DD], mud;
 #pragma unroll
             for (int i = 0; i < DD; ++i) Td[i] = Dual<R>{T[i], dT[i]};
             ok = metric_P<D>(p.metric, Td, mud, Pd);
 #pragma unroll
             for (int i = 0; i < DD; ++i) S[i] = Pd[i].d;
+          } else {
+            ok = metric_dP<D>(p.metric, T, dT, S);
           }
           // second term: dT2 = E_kl W2^-1
           R S2[DD];
@@ -709,14 +771,19 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP, WIDE>::WARPS * ElemCf
                 dT[a * D + b] = acc;
               }
           }
-          if (metric_dual(p.metric)) {
-            // not an (I1, tau) metric: forward-mode dual numbers
+          if (metric_dual<R>(p.metric)) {
             Dual<R> Td[DD], Pd[DD], mud;
 #pragma unroll
             for (int i = 0; i < DD; ++i) Td[i] = Dual<R>{T[i], dT[i]};
             ok = metric_P<D>(p.metric, Td, mud, Pd);
 #pragma unroll
             for (int i = 0; i < DD; ++i) S[i] = s * Pd[i].d;
+          } else if (D == 3 && sizeof(R) == 8 && p.metric == 302) {
+            if constexpr (D == 3 && sizeof(R) == 8) {
+              Metric302<R> L;
+              ok = L.init(T, s);
+              if (ok) L.dP(dT, S);
+            }
           } else {
             MetricAct<D, R> L;
             ok = L.init(p.metric, T, s);

@@ -95,7 +95,8 @@ inline int pa_stride_for(int dim, int Q, int elt, bool compact = false) {
   return bytes / elt;
 }
 
-// Metrics whose second derivative MetricLin writes in (|T|^2, det T).
+// Metrics whose second derivative MetricLin writes in (|T|^2, det T): those
+// with compact records (mu98 is written in |T - I|^2).
 inline bool metric_is_lin(int id) { return id != 302 && id != 98; }
 
 typedef int (*elem_launch_fn)(const KParams& p, int grid, void* stream);

@@ -317,6 +317,8 @@ __device__ __forceinline__ void pac_point(const float (&h)[kCompactRec], const f
   MetricLin<3, float> M;
 #pragma unroll
   for (int i = 0; i < 9; ++i) M.T[i] = h[i];
+#pragma unroll
+  for (int d = 0; d < 3; ++d) M.X[d] = h[4 * d];
   cof_m<3>(M.T, M.C);
   M.m1 = h[9]; M.mt = h[10]; M.m11 = h[11]; M.m1t = h[12]; M.mtt = h[13];
   float2* zp = reinterpret_cast<float2*>(buf) + q;
