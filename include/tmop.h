@@ -164,7 +164,9 @@ int tmop_gradient_hess_apply(tmop_ctx* ctx, const double* x, const double* v, do
  *   H_q = w_q det W (d^2mu/dT^2 composed with W^-1 on both sides)
  * (dim^2 (dim^2 + 1) / 2 values per point, FP64 under TMOP_FP64 and FP32
  * under the FP32 forms) in the context (allocated on first use:
- * nelem * Q * 45 * 8 bytes for order-k hexes in FP64). A 3D FP32 context
+ * nelem * Q * 45 * 8 bytes for order-k hexes in FP64, and 8 bytes per point
+ * of exponents: a 3D FP64 context keeps each value as a signed 60-bit integer
+ * in two 32-bit limbs, scaled by powers of two of its point). A 3D FP32 context
  * whose metric is written in |T|^2 and det T (1, 14, 303), with a constant
  * target and no second term, stores instead 14 values per point from which
  * the product rebuilds H_q (see tmop_pa_layout). Asynchronous. */
@@ -195,7 +197,8 @@ int tmop_hess_apply_pa_add_f32(tmop_ctx* ctx, const float* v, float* y, void* st
  * target and no second term, the 14-value record T, w det W (mu_1, mu_t,
  * mu_11, mu_1t, mu_tt) the product rebuilds the Hessian from), the element
  * stride in values (each element's block [value][point], padded to 16 bytes)
- * and the bytes per value (8 FP64, 4 FP32). Any pointer may be NULL.
+ * and the bytes per value (8 FP64, 4 FP32; the 8 bytes of a 3D FP64 context
+ * are a fixed-point number whose exponents are kept apart). Any pointer may be NULL.
  * Errors: TMOP_ERR_ARG if nothing is stored. */
 int tmop_pa_layout(const tmop_ctx* ctx, int* values_per_point, int* stride, int* elt_bytes);
 
