@@ -2,7 +2,7 @@
 kernels change: half a warp per 2D element from 1216 elements on, the
 fixed-point pointwise stage of mu303 against the general one, the closed-form
 second derivatives of mu302 and mu98, the one-cluster MINRES up to 2048 and
-8192 unknowns."""
+8192 unknowns, the scalar step in its own kernel above 150000."""
 import numpy as np
 import pytest
 
@@ -124,7 +124,8 @@ def test_second_derivatives_of_mu302_and_mu98(dim, order, nq, metric, target, pr
     assert _rel(ctx.hess_apply_pa(vd).cpu().numpy(), yo) <= tol
 
 
-@pytest.mark.parametrize("nx,unknowns", [((2, 2), 18), ((31, 31), 2048), ((40, 24), 2050), ((63, 63), 8192), ((40, 99), 8200)])
+@pytest.mark.parametrize("nx,unknowns", [((2, 2), 18), ((31, 31), 2048), ((40, 24), 2050), ((63, 63), 8192), ((40, 99), 8200),
+                                         ((273, 273), 150152)])
 @pytest.mark.parametrize("precision", ["fp64", "fp32"])
 def test_minres_vectors_in_one_cluster(nx, unknowns, precision):
     """After twelve iterations the oracle's iterate (rounding grows little in
@@ -145,6 +146,8 @@ def test_minres_vectors_in_one_cluster(nx, unknowns, precision):
         p, _ = ctx.krylov_solve(x, bd, krylov_rtol=1e-14, krylov_maxit=12)
         po, _ = orc.minres(m.x, b, rtol=1e-14, maxit=12)
         assert _rel(p.cpu().numpy(), po) <= (1e-10 if fp64 else 1e-4)
+    if unknowns > 100000:
+        return
     p, it = ctx.krylov_solve(x, bd, krylov_rtol=1e-9 if fp64 else 1e-5, krylov_maxit=5000)
     assert it > 0
     assert _rel(orc.hess_apply(m.x, p.cpu().numpy()), b) <= (1e-8 if fp64 else 1e-4 * 10)
