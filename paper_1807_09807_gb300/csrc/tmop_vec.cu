@@ -364,9 +364,10 @@ constexpr size_t kClMax = (size_t)256 * kClBlocks * kClPer;   // unknowns: kClPe
 
 // sum over the cluster in a fixed order, to all threads; slot: [kClBlocks]
 // doubles of this call. (A shuffle and an FP64 add are ~110 cycles, so every
-// level is a tree.)
-template <int NT>
-__device__ __forceinline__ double cluster_sum(double v, double* slot, cg::cluster_group& cl) {
+// level is a tree.) before(): what has to come before the first store to the
+// other blocks' shared memory.
+template <int NT, class WAIT>
+__device__ __forceinline__ double cluster_sum(double v, double* slot, cg::cluster_group& cl, WAIT&& before) {
   constexpr int W = NT / 32;
   __shared__ double red[W];
   const int lane = threadIdx.x & 31;
@@ -374,6 +375,7 @@ __device__ __forceinline__ double cluster_sum(double v, double* slot, cg::cluste
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   if (lane == 0) red[threadIdx.x >> 5] = v;
   __syncthreads();
+  before();
   if (threadIdx.x < 32) {
     double s = lane < W ? red[lane] : 0.0;
 #pragma unroll
@@ -387,13 +389,17 @@ __device__ __forceinline__ double cluster_sum(double v, double* slot, cg::cluste
   return s;
 }
 
-// the whole of a plain MINRES step after Av = H v (k_dot_part_t, k_lanczos,
-// k_minres_scalar and k_minres_vec_rot in one)
+// the whole of a plain MINRES step after Av = H v (k_dot_alpha, k_lanczos,
+// k_minres_scalar and k_minres_vec_rot in one). A block's shared memory may be
+// written by another one only after it has begun to run: every block arrives
+// at the cluster's barrier on entry and waits for it before the first such
+// store, so the step's loads hide the wait.
 template <class T, int NT>
 __global__ void __launch_bounds__(NT) k_minres_cluster(const T* __restrict__ v, T* __restrict__ vprev, T* __restrict__ Av,
                                                        const T* __restrict__ w, T* __restrict__ wp,
                                                        T* __restrict__ sol, double* st, int n) {
   cg::cluster_group cl = cg::this_cluster();
+  cl.barrier_arrive();
   __shared__ double sst[KS_COUNT];
   __shared__ double slots[2][kClBlocks];
   const int first = cl.block_rank() * NT + threadIdx.x;
@@ -416,7 +422,8 @@ __global__ void __launch_bounds__(NT) k_minres_cluster(const T* __restrict__ v, 
 #pragma unroll
   for (int k = 0; k < kClPer; ++k)
     if (first + k * S < n) a = fma(rv[k], ra[k], a);
-  const double alpha = cluster_sum<NT>((double)a, slots[0], cl);   // (its barriers cover sst too)
+  const double alpha = cluster_sum<NT>((double)a, slots[0], cl, [&] { cl.barrier_wait(); });
+  // (its barriers cover sst too)
   const double svd = sst[KS_SV];
   const T sv = (T)svd, av = (T)(alpha * svd * svd * svd), bv = (T)(sst[KS_BETA] * sst[KS_SVP]);
   T q = T(0);
@@ -429,7 +436,7 @@ __global__ void __launch_bounds__(NT) k_minres_cluster(const T* __restrict__ v, 
     vprev[i] = T(0);
     q = fma(r, r, q);
   }
-  const double b2 = cluster_sum<NT>((double)q, slots[1], cl);
+  const double b2 = cluster_sum<NT>((double)q, slots[1], cl, [] {});
   if (threadIdx.x == 0) {
     sst[KS_ALPHA] = alpha;
     minres_scalars(sst, b2);
