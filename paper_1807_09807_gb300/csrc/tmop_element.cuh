@@ -185,7 +185,6 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP, WIDE>::WARPS * ElemCf
   constexpr int NKQ = (FXPA || (FX303 && OP != OP_ENERGY)) ? NKEY * QP : 1;
   __shared__ short s_kq[NKQ > 1 ? WARPS : 1][NKQ];   // exponents of the points' results
   __shared__ int s_key[NKQ > 1 ? WARPS : 1][GW * NKEY];
-  __shared__ unsigned s_top[WARPS][GW];
   __shared__ unsigned s_mag[WARPS][GW * 2 * D];   // per warp and component: largest magnitudes of the group's warps
   R Wi[DD];
 #pragma unroll
@@ -298,7 +297,6 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP, WIDE>::WARPS * ElemCf
     int em[FX ? Cfg::NC : 1];
     int emx[FX ? D : 1];   // the split Hessian action's exponents of x
     bool fx303 = false;    // mu303 with W = I: pointwise stage in fixed point
-    int upA = 0, upV = 0;  // and the bits T and dT have to spare there
     if constexpr (FX) fx_group_exp<GT, Cfg::NC>(mag, em, s_mag[warp], bar);
     else __syncwarp();
     if constexpr (FX303) {
@@ -314,8 +312,7 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP, WIDE>::WARPS * ElemCf
       // P1, by one copy of the code
 #pragma unroll 1
       for (int f = 0;; ++f) {
-        const unsigned top = fwd3_fx<N, Q1, D, GT>(p.fx, em, P0, f == 0 ? P2 : P1, s_top[warp], lane, bar);
-        (f == 0 ? upA : upV) = fx_room(top);
+        fwd3_fx<N, Q1, D, GT>(p.fx, em, P0, f == 0 ? P2 : P1, lane, bar);
         if (f) break;
 #pragma unroll
         for (int c = 0; c < D; ++c) {
@@ -356,7 +353,7 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP, WIDE>::WARPS * ElemCf
       if constexpr (FX) fwd2_fx<N, Q1, Cfg::NC, GT>(p.fx, em, P0, P1, lane, bar);
       else fwd2<N, Q1, Cfg::NC, R>(sB, sG, P0, P1, lane);
     } else {
-      if constexpr (FX) upA = fx_room(fwd3_fx<N, Q1, Cfg::NC, GT>(p.fx, em, P0, P1, s_top[warp], lane, bar));
+      if constexpr (FX) fwd3_fx<N, Q1, Cfg::NC, GT>(p.fx, em, P0, P1, lane, bar);
       else fwd3_rb<N, Q1, Cfg::NC, R>(tB, tG, P0, P1, lane);
     }
     R* Abuf = Cfg::SPLIT ? P2 : ((D == 2) ? P0 : P1);     // A: [D][D][QP]
@@ -401,7 +398,7 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP, WIDE>::WARPS * ElemCf
         if constexpr (FXPA) {
           const short4 ex = __ldg(p.pa_exp + (size_t)e * QP + q);
           FxPoint pt[D];
-          fx_stored_product<QP>(reinterpret_cast<fx_t*>(Abuf) + q, h, ex, upA, sA, pt);
+          fx_stored_product<QP>(reinterpret_cast<fx_t*>(Abuf) + q, h, ex, sA, pt);
           const bool bad = ex.w == kPaNan || sA[0].nan || sA[1].nan || sA[2].nan;   // NaN everywhere
 #pragma unroll
           for (int a = 0; a < D; ++a) {
@@ -437,8 +434,8 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP, WIDE>::WARPS * ElemCf
           double mu, tau;
           const double s = sWq[q] * p.detW;
           const bool ok = fx_point303<QP, GRADLIKE || OP == OP_GRAD_HESS, Cfg::HV>(
-              reinterpret_cast<fx_t*>(Abuf) + q, reinterpret_cast<fx_t*>(dAbuf) + q, upA, upV, sA[0].kb, sV[0].kb, s,
-              pt[0], pt[NKEY - 1], mu, tau);
+              reinterpret_cast<fx_t*>(Abuf) + q, reinterpret_cast<fx_t*>(dAbuf) + q, sA[0].kb, sV[0].kb, s, pt[0],
+              pt[NKEY - 1], mu, tau);
           if constexpr (OP != OP_ENERGY) {
 #pragma unroll
             for (int k = 0; k < NKEY; ++k) {

@@ -240,17 +240,10 @@ struct FxNodal {
 // 3D forward map of NC components. P0: X (FxNodal, double) -> P1: [NC][2][N][N][Q]
 // -> P0: [NC][3][N][Q][Q] -> P1: A[NC][3][Q][Q][Q] (fixed point at fx_scale(em,
 // xin, gexp): the pointwise stage converts them, one point per thread). em:
-// exponent field of the largest magnitude of each component. Returns the
-// largest magnitude of the results (their high words); s_top: a word per warp. `lane`: the thread's
-// number among the GT of its group.
+// exponent field of the largest magnitude of each component. `lane`: the
+// thread's number among the GT of its group.
 template <int N, int Q1, int NC, int GT>
-__device__ __forceinline__ unsigned fwd3_fx(const FxTab& T, const int (&em)[NC], double* P0d, double* P1d,
-                                            unsigned* s_top, int lane, int bar) {
-  unsigned top = 0;
-  auto keep = [&](fx_t* o, fx_t y) {
-    *o = y;
-    top = max(top, (unsigned)((int)(y >> 32) ^ ((int)(y >> 32) >> 31)));
-  };
+__device__ __forceinline__ void fwd3_fx(const FxTab& T, const int (&em)[NC], double* P0d, double* P1d, int lane, int bar) {
   constexpr int NNQ = N * N * Q1, NQQ = N * Q1 * Q1, QQ = Q1 * Q1, QQQ = Q1 * Q1 * Q1;
   fx_t *P0 = reinterpret_cast<fx_t*>(P0d), *P1 = reinterpret_cast<fx_t*>(P1d);
   auto pick = [&](int c) {
@@ -302,23 +295,14 @@ __device__ __forceinline__ unsigned fwd3_fx(const FxTab& T, const int (&em)[NC],
 #pragma unroll
       for (int l = 0; l < N; ++l) v[l] = s[(2 - k) * NQQ + l * QQ];
       x.set(v);
-      fx_forward<N, Q1, false>(T, x, [&](int q, fx_t y) { keep(o + k * QQQ + q * QQ, y); });
+      fx_forward<N, Q1, false>(T, x, [&](int q, fx_t y) { o[k * QQQ + q * QQ] = y; });
     }
 #pragma unroll
     for (int l = 0; l < N; ++l) v[l] = s[l * QQ];
     x.set(v);
-    fx_forward<N, Q1, true>(T, x, [&](int q, fx_t y) { keep(o + 2 * QQQ + q * QQ, y); });
+    fx_forward<N, Q1, true>(T, x, [&](int q, fx_t y) { o[2 * QQQ + q * QQ] = y; });
   }
-  top = __reduce_max_sync(group_mask<GT>(), top);
-  if constexpr (GT > 32) {
-    if ((threadIdx.x & 31) == 0) s_top[(threadIdx.x >> 5) % (GT / 32)] = top;
-    group_sync<GT>(bar);
-#pragma unroll
-    for (int w = 0; w < GT / 32; ++w) top = max(top, s_top[w]);
-  } else {
-    group_sync<GT>(bar);
-  }
-  return top;
+  group_sync<GT>(bar);
 }
 
 // y shifted left by sh bits (right, with its sign, for sh < 0)
@@ -507,17 +491,27 @@ __device__ __forceinline__ void adj2_fx(const FxTab& T, const int (&em)[NC], dou
   group_sync<GT>(bar);
 }
 
-// Bits to shift the entries of a field up by: to |entries| < 2^59 by the
-// largest one of the element (top: its high word), or none (< 2^59.4 by
-// fx_tables).
-__device__ __forceinline__ int fx_room(unsigned top) { return max(__clz((int)top) - 5, 0); }
+// Bits to shift the nine entries of a point up by: to |entries| < 2^59 by the
+// largest one, or none (< 2^59.4 by fx_tables). By the point's own largest
+// entry: products of entries have a fixed number of bits, so at a point whose T
+// is r times smaller than the element's largest one would lose r^2 of the
+// cofactors and r^3 of det T to that one's scale (order-3 hexes graded to r =
+// 100: det T to 5e-10).
+template <int ST>
+__device__ __forceinline__ int fx_room(const fx_t* T) {
+  unsigned top = 0;   // (the same leading bit as the largest magnitude)
+#pragma unroll
+  for (int i = 0; i < 9; ++i) top |= (unsigned)((int)(T[i * ST] >> 32) ^ ((int)(T[i * ST] >> 32) >> 31));
+  return max(__clz((int)top) - 5, 0);
+}
 
 // mu303 at one point in fixed point (W = I): s P (GRAD, in place of T) and s dP
 // in direction V (HESS, in place of V), s = w det W, with
 //   P = cA T + ct C,  dP = cA V + bT T + bC C + ct dC[V]   (MetricAct),
 // where only the scalars (from |T|^2, det T, T:V and C:V) are FP64: one FP64
 // operation takes as long as ~17 IMAD.WIDE. T, V: entries [3][3] at stride ST,
-// of one scale each (FxScale::kb kT, kV), shifted up by upT, upV (fx_room).
+// of one scale each (FxScale::kb kT, kV), shifted up by what the point has to
+// spare (fx_room).
 // Magnitudes: |T|, |V|, |C| < 2^59, |dC| < 2^60, coefficients < 2^59 under a
 // common exponent per point, so all sums of limb products are < 2^63 and the
 // results < 2^61; a product loses ~2^-56 of the largest one.
@@ -529,9 +523,10 @@ struct FxPoint {
   unsigned mag;   // largest magnitude (high words)
 };
 template <int ST, bool GRAD, bool HESS>
-__device__ __forceinline__ bool fx_point303(fx_t* T, fx_t* V, int upT, int upV, int kT, int kV, double s, FxPoint& pg,
-                                            FxPoint& ph, double& mu, double& tau) {
+__device__ __forceinline__ bool fx_point303(fx_t* T, fx_t* V, int kT, int kV, double s, FxPoint& pg, FxPoint& ph,
+                                            double& mu, double& tau) {
   Limbs a[9], c[9], v[HESS ? 9 : 1];
+  const int upT = fx_room<ST>(T), upV = HESS ? fx_room<ST>(V) : 0;
   kT -= upT;
   kV -= upV;
   const int kC = 2 * kT + 60 - 1023;
@@ -655,13 +650,12 @@ __device__ __forceinline__ void fx_group_max(int* key, int* s, int bar) {
 constexpr int kPaNan = 32767, kPaZero = -20000;   // E of a point with a non-finite entry, of one without any
 
 // y = H dA at one point: h the packed entries, ex their exponents; A: dA in
-// fixed point at stride ST (rows' scales kb), shifted up by up (fx_room); the
-// rows are first brought to one exponent under the scaling of H. y replaces
-// dA; pt: per row.
+// fixed point at stride ST (rows' scales kb), shifted up by what the point has
+// to spare (fx_room); the rows are first brought to one exponent under the
+// scaling of H. y replaces dA; pt: per row.
 template <int ST>
-__device__ __forceinline__ void fx_stored_product(fx_t* A, const double* h, short4 ex, int up, const FxScale* sA,
-                                                  FxPoint* pt) {
-  const int s[3] = {ex.x, ex.y, ex.z};
+__device__ __forceinline__ void fx_stored_product(fx_t* A, const double* h, short4 ex, const FxScale* sA, FxPoint* pt) {
+  const int s[3] = {ex.x, ex.y, ex.z}, up = fx_room<ST>(A);
   int m[3], mx = -100000;
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
