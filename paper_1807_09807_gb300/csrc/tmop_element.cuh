@@ -377,7 +377,7 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP, WIDE>::WARPS * ElemCf
     };
     int key[D];
 #pragma unroll
-    for (int k = 0; k < D; ++k) key[k] = -4000;
+    for (int k = 0; k < D; ++k) key[k] = kFxKeyMin;
     // FP64: largest magnitude (high word) per component of the fields the
     // adjoint map takes (OP_GRAD_HESS: the gradient's, then the Hessian action's)
     unsigned rmag[FX ? 2 * D : 1] = {};

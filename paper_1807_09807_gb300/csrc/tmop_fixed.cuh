@@ -95,7 +95,8 @@ __device__ __forceinline__ fx_t fx_from_f64(double v, int emax, int lsh) {
   const unsigned mh = (hi & 0xfffffu) | 0x100000u;
   unsigned long long m = (((unsigned long long)mh << 32) | lo) << lsh;
   asm("shr.u64 %0, %1, %2;" : "=l"(m) : "l"(m), "r"(emax - (int)((hi >> 20) & 0x7ffu)));   // clamps at 64
-  return (fx_t)(m ^ (unsigned long long)(long long)((int)hi >> 31));   // (complement: off by one unit)
+  const long long neg = (int)hi >> 31;   // (the exact negative: -0.0 and what is shifted out become 0)
+  return ((fx_t)m ^ neg) - neg;
 }
 
 // Scale of a component's values: the exponent field of a value whose leading
@@ -683,11 +684,15 @@ __device__ __forceinline__ void fx_stored_product(fx_t* A, const double* h, shor
 }
 
 // The key whose maximum over the points gives the element's exponent (L), and
-// the exponent field of the largest magnitude (as fx_group_exp's) from it.
+// the exponent field of the largest magnitude (as fx_group_exp's) from it. Not
+// below kFxKeyMin, whose field is fx_floor's 64: what lies below (fields that
+// are zero, products that underflow) becomes zero, and the exponent field of a
+// result cannot leave its range.
+constexpr int kFxKeyMin = 64 + 2044 - 1022 - 33;
 __device__ __forceinline__ int fx_point_key(const FxPoint& p) {
   unsigned b;
   asm("bfind.u32 %0, %1;" : "=r"(b) : "r"(p.mag));
-  return p.mag ? p.E + (int)b : -4000;
+  return p.mag ? p.E + (int)b : kFxKeyMin;
 }
 __device__ __forceinline__ int fx_point_emax(int L) { return L + 33 - 2044 + 1022; }
 }  // namespace tmop
