@@ -403,7 +403,7 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP, WIDE>::WARPS * ElemCf
 #pragma unroll
           for (int a = 0; a < D; ++a) {
             key[a] = max(key[a], bad ? 32000 : fx_point_key(pt[a]));
-            s_kq[warp][a * QP + q] = (short)(pt[a].mag ? pt[a].E : -16000);
+            s_kq[warp][a * QP + q] = (short)(pt[a].zero() ? -16000 : pt[a].E);
           }
           continue;
         }
@@ -440,7 +440,7 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP, WIDE>::WARPS * ElemCf
 #pragma unroll
             for (int k = 0; k < NKEY; ++k) {
               key[k] = max(key[k], fx_point_key(pt[k]));
-              s_kq[warp][k * QP + q] = (short)(pt[k].mag ? pt[k].E : -16000);
+              s_kq[warp][k * QP + q] = (short)(pt[k].zero() ? -16000 : pt[k].E);
             }
           }
           if constexpr (EG || OP == OP_ENERGY) {

@@ -516,12 +516,19 @@ __device__ __forceinline__ int fx_room(const fx_t* T) {
 // Magnitudes: |T|, |V|, |C| < 2^59, |dC| < 2^60, coefficients < 2^59 under a
 // common exponent per point, so all sums of limb products are < 2^63 and the
 // results < 2^61; a product loses ~2^-56 of the largest one.
-// A result is y 2^(E - 2044); E and the leading bit of the largest entry's high
-// word (0: all zero) per point are returned for the adjoint map, which gives
-// the element one exponent.
+// A result is y 2^(E - 2044); E and the bits of the magnitudes per point are
+// returned for the adjoint map, which gives the element one exponent.
 struct FxPoint {
-  int E;          // exponent of the point's results
-  unsigned mag;   // largest magnitude (high words)
+  int E;                       // exponent of the point's results
+  unsigned hi = 0, lo = 0;     // the magnitudes' words, or-ed: the leading bit of the largest one
+  // (Both words: where the terms of P or of a product cancel, as near an ideal
+  // mesh, all entries can lie below 2^32 and still hold 25 good bits.)
+  __device__ __forceinline__ void add(fx_t y) {
+    const int neg = (int)(y >> 32) >> 31;
+    hi |= (unsigned)((int)(y >> 32) ^ neg);
+    lo |= (unsigned)((int)y ^ neg);
+  }
+  __device__ __forceinline__ bool zero() const { return (hi | lo) == 0; }
 };
 template <int ST, bool GRAD, bool HESS>
 __device__ __forceinline__ bool fx_point303(fx_t* T, fx_t* V, int kT, int kV, double s, FxPoint& pg, FxPoint& ph,
@@ -580,7 +587,7 @@ __device__ __forceinline__ bool fx_point303(fx_t* T, fx_t* V, int kT, int kV, do
   if constexpr (GRAD) {
     const int E = max(ex(cA) + kT, ex(ct) + kC);
     const Limbs gT = fx_split(fx_from_f64(cA, E - kT, 6)), gC = fx_split(fx_from_f64(ct, E - kC, 6));
-    unsigned m = 0;
+    pg = {E};
 #pragma unroll
     for (int i = 0; i < 9; ++i) {
       FxAcc z{0, 0};
@@ -588,9 +595,8 @@ __device__ __forceinline__ bool fx_point303(fx_t* T, fx_t* V, int kT, int kV, do
       fx_mac(z, c[i], gC.h, gC.l);
       const fx_t y = ok ? fx_value(z) : 0;
       T[i * ST] = y;
-      m = max(m, (unsigned)((int)(y >> 32) ^ ((int)(y >> 32) >> 31)));
+      pg.add(y);
     }
-    pg = {E, m};
   }
   if constexpr (HESS) {
     const double ctt = (ct * it) * (-5.0 / 3.0);
@@ -599,7 +605,7 @@ __device__ __forceinline__ bool fx_point303(fx_t* T, fx_t* V, int kT, int kV, do
     const int E = max(max(ex(cA) + kV, ex(bT) + kT), max(ex(bC) + kC, ex(ct) + kD));
     const Limbs hV = fx_split(fx_from_f64(cA, E - kV, 6)), hT = fx_split(fx_from_f64(bT, E - kT, 6));
     const Limbs hC = fx_split(fx_from_f64(bC, E - kC, 6)), hD = fx_split(fx_from_f64(ct, E - kD, 6));
-    unsigned m = 0;
+    ph = {E};
 #pragma unroll
     for (int i = 0; i < 9; ++i) {
       FxAcc p{0, 0}, n{0, 0}, z{0, 0};
@@ -612,9 +618,8 @@ __device__ __forceinline__ bool fx_point303(fx_t* T, fx_t* V, int kT, int kV, do
       fx_mac(z, c[i], hC.h, hC.l);
       const fx_t y = ok ? fx_value(z) : 0;
       V[i * ST] = y;
-      m = max(m, (unsigned)((int)(y >> 32) ^ ((int)(y >> 32) >> 31)));
+      ph.add(y);
     }
-    ph = {E, m};
   }
   return ok;
 }
@@ -668,7 +673,7 @@ __device__ __forceinline__ void fx_stored_product(fx_t* A, const double* h, shor
   for (int i = 0; i < 9; ++i)
     d[i] = fx_split((fx_t)((unsigned long long)A[i * ST] << up) >> min(mx - m[i / 3], 63));
 #pragma unroll
-  for (int a = 0; a < 3; ++a) pt[a] = {s[a] + ex.w + mx - up + 1024, 0u};
+  for (int a = 0; a < 3; ++a) pt[a] = {s[a] + ex.w + mx - up + 1024};
 #pragma unroll
   for (int r = 0; r < 9; ++r) {
     FxAcc z{0, 0};   // 9 terms: |H| < 9 2^56, |M| < 9 (2^59 + 2^57) < 2^63
@@ -679,7 +684,7 @@ __device__ __forceinline__ void fx_stored_product(fx_t* A, const double* h, shor
     }
     const fx_t y = fx_value(z);
     A[r * ST] = y;
-    pt[r / 3].mag = max(pt[r / 3].mag, (unsigned)((int)(y >> 32) ^ ((int)(y >> 32) >> 31)));
+    pt[r / 3].add(y);
   }
 }
 
@@ -690,9 +695,9 @@ __device__ __forceinline__ void fx_stored_product(fx_t* A, const double* h, shor
 // result cannot leave its range.
 constexpr int kFxKeyMin = 64 + 2044 - 1022 - 33;
 __device__ __forceinline__ int fx_point_key(const FxPoint& p) {
-  unsigned b;
-  asm("bfind.u32 %0, %1;" : "=r"(b) : "r"(p.mag));
-  return p.mag ? p.E + (int)b : kFxKeyMin;
+  unsigned b;   // leading bit of the word
+  asm("bfind.u32 %0, %1;" : "=r"(b) : "r"(p.hi ? p.hi : p.lo));
+  return p.zero() ? kFxKeyMin : p.E + (int)b - (p.hi ? 0 : 32);
 }
 __device__ __forceinline__ int fx_point_emax(int L) { return L + 33 - 2044 + 1022; }
 }  // namespace tmop
