@@ -301,9 +301,10 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP, WIDE>::WARPS * ElemCf
     else __syncwarp();
     if constexpr (FX303) {
       // one exponent for all components (at most 4 bits lost to one of them),
-      // where those of the products stay inside the FP64 range (fx_point303)
+      // where the scalars stay inside the FP64 range (kFx303X)
       const int lo = min(em[0], min(em[1], em[2])), hi = max(em[0], max(em[1], em[2]));
-      fx303 = p.metric == 303 && p.wkind == WK_IDENTITY && !p.metric2 && lo > 600 && hi < 1400 && hi - lo <= 4;
+      fx303 = p.metric == 303 && p.wkind == WK_IDENTITY && !p.metric2 &&
+              hi >= 1023 - kFx303X && hi <= 1023 + kFx303X && hi - lo <= 4;
       if (fx303) em[0] = em[1] = em[2] = hi;
     }
     // ---- forward contraction: A (and dA) at every point
@@ -332,7 +333,7 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP, WIDE>::WARPS * ElemCf
         fx_group_exp<GT, D>(mag, em, s_mag[warp], bar);
         if (fx303) {
           const int hi = max(em[0], max(em[1], em[2]));
-          fx303 = hi > 300 && hi < 1750 && hi - emx[0] > -700 && hi - emx[0] < 700;
+          fx303 = hi >= 1023 - kFx303V && hi <= 1023 + kFx303V;
           if (fx303) em[0] = em[1] = em[2] = hi;
         }
       }
@@ -402,7 +403,7 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP, WIDE>::WARPS * ElemCf
           const bool bad = ex.w == kPaNan || sA[0].nan || sA[1].nan || sA[2].nan;   // NaN everywhere
 #pragma unroll
           for (int a = 0; a < D; ++a) {
-            key[a] = max(key[a], bad ? 32000 : fx_point_key(pt[a]));
+            key[a] = max(key[a], bad ? kFxNan : fx_point_key(pt[a]));
             s_kq[warp][a * QP + q] = (short)(pt[a].zero() ? -16000 : pt[a].E);
           }
           continue;

@@ -530,6 +530,15 @@ struct FxPoint {
   }
   __device__ __forceinline__ bool zero() const { return (hi | lo) == 0; }
 };
+// Elements whose x - x_0 has a largest component within 2^-kFx303X and
+// 2^kFx303X (and v within 2^-kFx303V and 2^kFx303V) take this stage, the others
+// the FP64 one. At a point |T| can be 2^57 smaller than the element's, and det T
+// 2^58 smaller than |T|^3: with |T| within 2^-101 and 2^46, tau lies within
+// 2^-361 and 2^138, so cA and ct, the gradient's scalars, within 2^-100 and
+// 2^400. Those of dP can leave the range at such a point where v is large, as
+// they do in FP64: results are then NaN (dP's E below).
+constexpr int kFx303X = 40, kFx303V = 610;
+constexpr int kFxNan = 32000;   // E of a point whose results are not finite
 template <int ST, bool GRAD, bool HESS>
 __device__ __forceinline__ bool fx_point303(fx_t* T, fx_t* V, int kT, int kV, double s, FxPoint& pg, FxPoint& ph,
                                             double& mu, double& tau) {
@@ -603,6 +612,7 @@ __device__ __forceinline__ bool fx_point303(fx_t* T, fx_t* V, int kT, int kV, do
     const double bT = c1t * d, bC = fma(c1t, t, ctt * d);
     const int kD = kT + kV + 60 - 1023;
     const int E = max(max(ex(cA) + kV, ex(bT) + kT), max(ex(bC) + kC, ex(ct) + kD));
+    const bool finite = max(ex(bT), ex(bC)) < 2047;
     const Limbs hV = fx_split(fx_from_f64(cA, E - kV, 6)), hT = fx_split(fx_from_f64(bT, E - kT, 6));
     const Limbs hC = fx_split(fx_from_f64(bC, E - kC, 6)), hD = fx_split(fx_from_f64(ct, E - kD, 6));
     ph = {E};
@@ -620,6 +630,7 @@ __device__ __forceinline__ bool fx_point303(fx_t* T, fx_t* V, int kT, int kV, do
       V[i * ST] = y;
       ph.add(y);
     }
+    if (!finite) ph = {kFxNan, 1u << 30};
   }
   return ok;
 }
@@ -688,8 +699,8 @@ __device__ __forceinline__ void fx_stored_product(fx_t* A, const double* h, shor
   }
 }
 
-// The key whose maximum over the points gives the element's exponent (L), and
-// the exponent field of the largest magnitude (as fx_group_exp's) from it. Not
+// The key whose maximum over the points gives the element's exponent (L; with
+// kFxNan one that fx_scale takes for not finite), and the exponent field of the largest magnitude (as fx_group_exp's) from it. Not
 // below kFxKeyMin, whose field is fx_floor's 64: what lies below (fields that
 // are zero, products that underflow) becomes zero, and the exponent field of a
 // result cannot leave its range.

@@ -63,3 +63,55 @@ def test_gradient_of_the_ideal_mesh(order, nq):
     assert ctx.hess_apply(xd, xd).abs().max() <= tol
     ctx.linearize(xd)
     assert ctx.hess_apply_pa(xd).abs().max() <= tol
+
+
+@pytest.mark.parametrize("order,nq", [(1, 2), (2, 4), (3, 5), (4, 6)])
+@pytest.mark.parametrize("k", [-330, -250, -150, -100, -43, -42, -41, -38, -37, 37, 38, 41, 42, 43, 100, 150, 250, 330])
+def test_meshes_of_any_size(order, nq, k):
+    """x times 2^k, both sides of the sizes the fixed-point stage of mu303 takes:
+    mu is scale invariant, so F stays, det A takes 2^(3k), the gradient 2^-k and
+    the Hessian action 2^-2k. (The Hessian's tau^(-8/3) |T|^2 leaves the FP64
+    range by itself above |k| = 160.) 1e-11, as between two ways to compute it."""
+    import torch
+    from paper_1807_09807_gb300 import tmop as tm
+    m = _mesh(3, order, nq, 303)
+    ctx = tm.Context.from_mesh(m)
+    ctx.set_deterministic(True)
+    x = torch.tensor(m.x, device="cuda")
+    v = torch.tensor(np.random.default_rng(2).standard_normal(m.x.shape), device="cuda")
+    s = 2.0 ** k
+    F, g, y = ctx.energy(x), ctx.gradient(x), ctx.hess_apply(x, v)
+
+    def near(a, b):
+        return bool((a - b).norm() <= 1e-11 * b.norm())
+
+    Fs = ctx.energy(x * s)
+    assert Fs[0] == F[0] and abs(Fs[1] - F[1]) <= 1e-11 * F[1] and abs(Fs[2] / s / s / s - F[2]) <= 1e-11 * F[2]
+    assert near(ctx.gradient(x * s) * s, g)
+    ge, Fe, md = ctx.energy_gradient(x * s)
+    assert near(ge * s, g) and abs(Fe.item() - F[1]) <= 1e-11 * F[1] and md.item() == Fs[2]
+    if abs(k) > 150:
+        return
+    assert near(ctx.hess_apply(x * s, v) * s * s, y)
+    gh, yh = ctx.gradient_hess_apply(x * s, v)
+    assert near(gh * s, g) and near(yh * s * s, y)
+    ctx.linearize(x * s)
+    assert near(ctx.hess_apply_pa(v) * s * s, y)
+
+
+@pytest.mark.parametrize("order,nq", [(1, 2), (2, 4), (3, 5), (4, 6)])
+@pytest.mark.parametrize("kx", [-39, 0, 39])
+@pytest.mark.parametrize("kv", [-880, -616, -606, 602, 612, 850])
+def test_directions_of_any_size(order, nq, kx, kv):
+    """v times 2^kv at sizes of x near the ends of that range, on both sides of
+    the sizes of v the stage takes. (The terms of dP go as |v| |x|^-4.)"""
+    import torch
+    from paper_1807_09807_gb300 import tmop as tm
+    m = _mesh(3, order, nq, 303)
+    ctx = tm.Context.from_mesh(m)
+    ctx.set_deterministic(True)
+    x = torch.tensor(m.x, device="cuda")
+    v = torch.tensor(np.random.default_rng(2).standard_normal(m.x.shape), device="cuda")
+    y = ctx.hess_apply(x, v)
+    z = ctx.hess_apply(x * 2.0 ** kx, v * 2.0 ** kv) * 2.0 ** -kv * 2.0 ** (2 * kx)
+    assert (z - y).norm() <= 1e-11 * y.norm()
