@@ -23,6 +23,8 @@ constexpr int kThreads = 256;
 
 static int g_sms = 0;
 
+constexpr size_t kOneEach = 304;   // blocks, see red_grid
+
 int red_grid(size_t n) {
   if (g_sms == 0) {
     int dev = 0;
@@ -34,11 +36,14 @@ int red_grid(size_t n) {
   // stream 4 to 8 vectors, and more loads in flight keep HBM busier. A grid
   // of at least one block per SM is a whole number of blocks per SM, so every
   // SM streams the same share.
-  // Below that one value per thread: a pass over few values is bound by the
-  // latency of one thread's chain and by the FP64 pipe of the SMs it runs on
-  // (18 818 unknowns, plain MINRES: 24.9 us per iteration with four values
-  // per thread, 21.8 us with one).
-  size_t want = (n + kThreads - 1) / kThreads;
+  // Four values per thread, but one where that leaves fewer than kOneEach
+  // blocks: a pass over few values is bound by the latency of one thread's
+  // chain and by the FP64 pipe of the SMs it runs on (18 818 unknowns, plain
+  // MINRES: 24.9 us per iteration with four values per thread, 21.8 us with
+  // one), a pass over many by the blocks that have to be counted (FP32, 321 602
+  // unknowns: 46.4 us with one value per thread in 1216 blocks, 36.9 so).
+  size_t want = (n + kThreads * 4 - 1) / (kThreads * 4), one = (n + kThreads - 1) / kThreads;
+  if (want < kOneEach) want = one < kOneEach ? one : kOneEach;
   size_t cap = (size_t)g_sms * 8;
   if (cap > (size_t)kMaxRedBlocks) cap = kMaxRedBlocks;
   if (want > cap) want = cap;
@@ -194,16 +199,20 @@ __global__ void k_minres_init(const double* __restrict__ b, T* v, T* vprev, T* A
 }
 
 // st[KS_ALPHA] = a . b over T vectors: each thread sums its elements in T
-// (FP32 vectors: ~30 elements per thread at full occupancy), the blocks in FP64
-template <class T>
+// (FP32 vectors: ~30 elements per thread at full occupancy), the blocks in FP64.
+// LAST: the last block adds up the partials (else k_sum_final does).
+template <class T, bool LAST>
 __global__ void k_dot_alpha(const T* __restrict__ a, const T* __restrict__ b, size_t n, double* __restrict__ part,
                             double* st) {
   T s = T(0);
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
     s = fma(a[i], b[i], s);
-  double sum;
-  if (last_block_sum(block_sum((double)s), part, gridDim.x, st + KS_COUNTER, &sum) && threadIdx.x == 0)
-    st[KS_ALPHA] = sum;
+  double sum = block_sum((double)s);
+  if constexpr (LAST) {
+    if (last_block_sum(sum, part, gridDim.x, st + KS_COUNTER, &sum) && threadIdx.x == 0) st[KS_ALPHA] = sum;
+  } else {
+    if (threadIdx.x == 0) part[blockIdx.x] = sum;
+  }
 }
 
 __device__ void minres_scalars(double* st, double beta_next2);
@@ -358,7 +367,7 @@ __global__ void k_minres_vec_rot(const T* __restrict__ v, const T* __restrict__ 
 // on a copy of the state in shared memory; block 0 writes it back after the
 // barrier behind which all blocks have read it.
 namespace cg = cooperative_groups;
-constexpr size_t kLastBlockMax = 150000;   // unknowns of the Lanczos step with the scalar step in its last block
+constexpr size_t kLastBlockMax = 150000;   // unknowns up to which MINRES's reductions end in their last block
 constexpr int kClBlocks = 8, kClPer = 4;
 constexpr size_t kClMax = (size_t)256 * kClBlocks * kClPer;   // unknowns: kClPer per thread of the larger form
 
@@ -482,14 +491,17 @@ int minres_after_hv_rot(const T* v, T* vprev, T* Av, const T* w, T* wp, T* sol, 
   int g = red_grid(n);
   if (vdot) {  // alpha = v . (H v) from the product kernel's own partials
     k_sum_final<<<1, kThreads, 0, s>>>(vdot, vdot_np, st + KS_ALPHA);
+  } else if (n <= kLastBlockMax) {
+    k_dot_alpha<T, true><<<g, kThreads, 0, s>>>(v, Av, n, part, st);
   } else {
-    k_dot_alpha<T><<<g, kThreads, 0, s>>>(v, Av, n, part, st);
+    k_dot_alpha<T, false><<<g, kThreads, 0, s>>>(v, Av, n, part, st);
+    k_sum_final<<<1, kThreads, 0, s>>>(part, g, st + KS_ALPHA);
   }
-  // The last block's scalar step saves a launch, but every block then waits for
-  // its own stores before it counts itself: FP32 74 498 unknowns 22.6 us per
-  // iteration against 24.7 with both reductions in kernels of their own, but
-  // 296 450 unknowns 41.5 against 41.1 with this one in its own, FP64 55.9
-  // against 54.2
+  // A reduction that ends in its last block saves a launch, but every block then
+  // waits for its own stores before it counts itself: FP32 74 498 unknowns 22.6
+  // us per iteration against 24.7 with both in kernels of their own, but 296 450
+  // unknowns 33.0 against 32.2 with the dot product in its own; the scalar step
+  // in its own there: FP64 54.2 against 55.9
   if (n <= kLastBlockMax) {
     k_lanczos<T, true><<<g, kThreads, 0, s>>>(Av, v, vprev, st, n, part);
   } else {
