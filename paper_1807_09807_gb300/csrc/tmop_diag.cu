@@ -130,6 +130,22 @@ __global__ void __launch_bounds__(kDiagWarps * 32) diag_kernel(const DiagParams 
   // compact records (3D): entries b = 0..2 of row a of the response to E_ac
   __shared__ float whh[kDiagWarps][DIM == 3 ? 3 * QP : 1];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  // FP64 3D: the entries are packed (tmop_fixed.cuh), (h 2^30 + l) 2^(E + 2 s_a -
+  // 57); the exponents of the lane's points are loaded once, an entry's values
+  // while the one before is contracted, and both are joined by integer
+  // operations, as this kernel is bound by the FP64 pipe (32^3 order-3 hexes:
+  // 1.77 ms from plain doubles, 2.50 with a conversion and ldexp, 1.62 so; 8^3
+  // order 1: 27.3, 31.9, 25.6 us)
+  constexpr bool PACKED = DIM == 3 && sizeof(R) == 8;
+  constexpr int NPL = (QP + 31) / 32;
+  short4 ex[PACKED ? NPL : 1];
+  double hv[PACKED ? NPL : 1];
+  auto fetch = [&](const R* He, int a, int b, int c) {   // H[(a,b),(a,c)] of the lane's points
+    const int rr = a * DIM + b, s = rr * DD - rr * (rr - 1) / 2 + c - b;
+#pragma unroll
+    for (int k = 0; k < NPL; ++k)
+      if (lane + 32 * k < QP) hv[k] = __ldg(He + (size_t)s * QP + lane + 32 * k);
+  };
   for (int t = threadIdx.x; t < Q1 * N; t += blockDim.x) {
     const double b = p.B[t], g = p.G[t];
     tab[0][t] = A(b * b);
@@ -146,6 +162,12 @@ __global__ void __launch_bounds__(kDiagWarps * 32) diag_kernel(const DiagParams 
     const int e = p.elist ? __ldg(p.elist + ei) : ei;
     nodes.element(e, NDOF);
     const R* He = H + (size_t)e * p.pa_stride;
+    if constexpr (PACKED) {
+#pragma unroll
+      for (int k = 0; k < NPL; ++k)
+        if (lane + 32 * k < QP) ex[k] = __ldg(p.pa_exp + (size_t)e * QP + lane + 32 * k);
+      fetch(He, 0, 0, 0);
+    }
     for (int a = 0; a < DIM; ++a) {
       for (int t = lane; t < NDOF; t += 32) Y[t] = A(0);
       __syncwarp();
@@ -167,20 +189,23 @@ __global__ void __launch_bounds__(kDiagWarps * 32) diag_kernel(const DiagParams 
           if (DIM == 3 && p.compact) {
             for (int q = lane; q < QP; q += 32) r[q] = m * (A)hh[b * QP + q];
           } else {
-            // packed index of (row a*DIM+b, column a*DIM+c), row <= column
-            const int rr = a * DIM + b, cc = a * DIM + c;
-            const int s = rr * DD - rr * (rr - 1) / 2 + (cc - rr);
-            for (int q = lane; q < QP; q += 32) {
-              if constexpr (DIM == 3 && sizeof(R) == 8) {   // packed: (h 2^30 + l) 2^(E + 2 s_a - 57)
-                const short4 ex = __ldg(p.pa_exp + (size_t)e * QP + q);
-                const double v = He[(size_t)s * QP + q];
-                const long long i = ((long long)__double2hiint(v) << 30) + __double2loint(v);
-                const int sa = a == 0 ? ex.x : (a == 1 ? ex.y : ex.z);
-                r[q] = ex.w == kPaNan ? __longlong_as_double(0x7ff8000000000000LL)
-                                      : ldexp(m * (double)i, ex.w == kPaZero ? 0 : ex.w + 2 * sa - 57);
-              } else {
-                r[q] = m * (A)He[(size_t)s * QP + q];
+            if constexpr (PACKED) {
+#pragma unroll
+              for (int k = 0; k < NPL; ++k) {
+                const int q = lane + 32 * k;
+                if (q >= QP) break;
+                const int sa = a == 0 ? ex[k].x : (a == 1 ? ex[k].y : ex[k].z);
+                const FxScale sc = {1023 - 57 + ex[k].w + 2 * sa + (b != c), ex[k].w == kPaNan ? 0x7ff80000u : 0u};
+                r[q] = fx_to_f64(((long long)__double2hiint(hv[k]) << 30) + __double2loint(hv[k]), sc);
               }
+              if (b < c) fetch(He, a, b + 1, c);
+              else if (c + 1 < DIM) fetch(He, a, 0, c + 1);
+              else if (a + 1 < DIM) fetch(He, a + 1, 0, 0);
+            } else {
+              // packed index of (row a*DIM+b, column a*DIM+c), row <= column
+              const int rr = a * DIM + b, cc = a * DIM + c;
+              const int s = rr * DD - rr * (rr - 1) / 2 + (cc - rr);
+              for (int q = lane; q < QP; q += 32) r[q] = m * (A)He[(size_t)s * QP + q];
             }
           }
           __syncwarp();
