@@ -483,8 +483,7 @@ int linearize(tmop_ctx* c, const double* x, cudaStream_t s) {
     const size_t stride = (size_t)pa_stride_for(c->dim, c->Q, elt);
     CUDA_TRY(cudaMalloc(&c->d_pa, (size_t)elt * stride * (size_t)c->nelem));
   }
-  const bool pack = c->dim == 3 && c->precision == TMOP_FP64;   // for the fixed-point product
-  if (pack && !c->d_pa_exp) {
+  if (c->dim == 3 && c->precision == TMOP_FP64 && !c->d_pa_exp) {
     CUDA_TRY(cudaMalloc(&c->d_pa_exp, sizeof(short4) * (size_t)c->Q * (size_t)c->nelem));
     c->base.pa_exp = c->d_pa_exp;
   }
@@ -494,8 +493,6 @@ int linearize(tmop_ctx* c, const double* x, cudaStream_t s) {
   c->pa_valid = false;
   int rc = launch_op(c, OP_LINEARIZE, x, nullptr, nullptr, nullptr, s);
   if (rc) return rc;
-  if (pack && pa_pack(static_cast<double*>(c->d_pa), c->base.pa_stride, c->d_pa_exp, c->nelem, c->Q, s) != 0)
-    return TMOP_ERR_CUDA;
   c->pa_valid = true;
   return TMOP_OK;
 }

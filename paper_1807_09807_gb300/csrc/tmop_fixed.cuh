@@ -658,13 +658,58 @@ __device__ __forceinline__ void fx_group_max(int* key, int* s, int bar) {
 }
 
 // ---------------------------------------------------------------- stored Hessians
-// The FP64 3D stored Hessians are packed for the fixed-point product by
-// pa_pack (tmop_pa_pack.cu): the 45 entries H_(r,c) of a point, r = 3 a + b, as
+// The FP64 3D stored Hessians are packed for the fixed-point product by the
+// linearisation (fx_pack_point): the 45 entries H_(r,c) of a point, r = 3 a + b, as
 //   H_(r,c) = (h 2^30 + l) 2^(E + s_a + s_c - 57),  |h| <= 2^27, 0 <= l < 2^30,
 // (h, l) in the place of the double's high and low word, and {s_0, s_1, s_2, E}
 // beside them; s_a is half the exponent of block (a, a), so that directions
 // along which elements are long or short keep their digits.
+// (The least of their digits are not missed: an error of 2^-57 of a block's
+// largest entry stays below what FP64 rounding of dA, relative to the largest
+// nodal value of v, does through that entry. On elements of aspect 1 to 1000, in
+// rows or columns, the product's error from it is 1e-17 to 7e-15 where FP64
+// arithmetic has 1e-16 to 1e-12.)
 constexpr int kPaNan = 32767, kPaZero = -20000;   // E of a point with a non-finite entry, of one without any
+
+// Packs the 45 entries h of a point to H[i st], their exponents to *ex; ok: the
+// point's T has a Hessian (else zeros).
+__device__ __forceinline__ void fx_pack_point(const double (&h)[45], bool ok, double* H, int st, short4* ex) {
+  // largest entries of the blocks: their high words, then exponents (|entry| < 2^m)
+  unsigned w[3][3] = {};
+#pragma unroll
+  for (int r = 0; r < 9; ++r)
+#pragma unroll
+    for (int c = r; c < 9; ++c)
+      w[r / 3][c / 3] = max(w[r / 3][c / 3], fx_mag(h[r * 9 - r * (r - 1) / 2 + c - r]));
+  int m[3][3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a)
+#pragma unroll
+    for (int c = a; c < 3; ++c) m[a][c] = (int)(w[a][c] >> 20) - 1022;
+  const int top = max(max(max(m[0][0], m[1][1]), max(m[2][2], m[0][1])), max(m[0][2], m[1][2]));
+  // half the exponents of the diagonal blocks, or one for all where they do
+  // not bound the others (an indefinite point can have a small one)
+  int s[3] = {m[0][0] >> 1, m[1][1] >> 1, m[2][2] >> 1};
+  const bool even = m[0][1] > s[0] + s[1] + 8 || m[0][2] > s[0] + s[2] + 8 || m[1][2] > s[1] + s[2] + 8 ||
+                    min(m[0][0], min(m[1][1], m[2][2])) < -900;
+  if (even) s[0] = s[1] = s[2] = top >> 1;
+  int E = -100000;
+#pragma unroll
+  for (int a = 0; a < 3; ++a)
+#pragma unroll
+    for (int c = a; c < 3; ++c) E = max(E, m[a][c] - s[a] - s[c]);
+  const bool zero = !ok || top < -900;            // (nothing above 2^-900)
+  const int base = zero ? 4096 : E + 1022;        // (zero: everything is shifted out)
+#pragma unroll
+  for (int r = 0; r < 9; ++r)
+#pragma unroll
+    for (int c = r; c < 9; ++c) {
+      const int i = r * 9 - r * (r - 1) / 2 + c - r;
+      const Limbs l = fx_split(fx_from_f64(h[i], base + s[r / 3] + s[c / 3], 4));
+      H[(size_t)i * st] = __hiloint2double(l.h, l.l);
+    }
+  *ex = make_short4((short)s[0], (short)s[1], (short)s[2], (short)(zero ? kPaZero : (top >= 1025 ? kPaNan : E)));
+}
 
 // y = H dA at one point: h the packed entries, ex their exponents; A: dA in
 // fixed point at stride ST (rows' scales kb), shifted up by what the point has

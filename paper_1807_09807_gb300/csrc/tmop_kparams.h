@@ -57,7 +57,7 @@ struct KParams {
   double* part_F;                 // [grid] energy partials
   double* part_min;               // [grid] min det A partials
   double* elem_min;               // [nelem] per-element min det A, or null
-  const short4* pa_exp;           // FP64 3D: exponents of the packed Hessians, [nelem][Q] (tmop_fixed.cuh)
+  short4* pa_exp;                 // FP64 3D: exponents of the packed Hessians, [nelem][Q] (tmop_fixed.cuh)
   void* pa;                       // [nelem][pa_stride] packed Hessians [DD(DD+1)/2][Q] (float or double)
   double* vdot;                   // product from compact records: per-warp partials of v . (H v), or null
   // Deterministic sums: when elist is set, the launch runs only the ecount
@@ -117,9 +117,6 @@ bool rule_gl(int q, double* x, double* w);
 bool rule_gll(int q, double* x, double* w);
 void lagrange_bary(int n, const double* z, double s, double* phi, double* dphi);
 bool inv_h(int d, const double* W, double* Wi, double* detW);
-// Packs the FP64 3D stored Hessians for the fixed-point product, in place, and
-// writes their exponents (tmop_pa_pack.cu).
-int pa_pack(double* pa, int stride, short4* ex, int nelem, int Q, void* stream);
 bool fx_tables(int dim, int n, int q, const double* B, const double* G, FxTab* T);
 
 }  // namespace tmop

@@ -115,3 +115,23 @@ def test_directions_of_any_size(order, nq, kx, kv):
     y = ctx.hess_apply(x, v)
     z = ctx.hess_apply(x * 2.0 ** kx, v * 2.0 ** kv) * 2.0 ** -kv * 2.0 ** (2 * kx)
     assert (z - y).norm() <= 1e-11 * y.norm()
+
+
+@pytest.mark.parametrize("order,nq,metric", [(1, 2, 303), (2, 4, 302), (3, 5, 303), (3, 4, 98)])
+@pytest.mark.parametrize("target", ["unit", "scaled"])   # closed forms, nine directions
+def test_stored_product_of_a_mesh_with_inverted_points(order, nq, metric, target):
+    """Points with det T <= 0 have no Hessian: zeros, packed with the others'.
+    The recomputed action skips them; 1e-10 of the largest value, as the points
+    beside them have det T small."""
+    import torch
+    from paper_1807_09807_gb300 import tmop as tm
+    m = _mesh(3, order, nq, metric)
+    n = int(np.flatnonzero(m.fixed[0] == 0)[0])
+    m.x[0, n] += 2.0
+    ctx = tm.Context.from_mesh(m, target_scale=0.5 if target == "scaled" else None)
+    x = torch.tensor(m.x, device="cuda")
+    assert ctx.energy(x)[0] != tm.OK
+    v = torch.tensor(np.random.default_rng(2).standard_normal(m.x.shape), device="cuda")
+    ctx.linearize(x)
+    y, z = ctx.hess_apply_pa(v), ctx.hess_apply(x, v)
+    assert z.isfinite().all() and (y - z).abs().max() <= 1e-10 * z.abs().max()
