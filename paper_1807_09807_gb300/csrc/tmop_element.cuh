@@ -94,7 +94,7 @@ struct ElemCfg {
 // Second term of a composite metric at one point: T2 = A W2^-1 and, for a
 // direction dA, dT2 = dA W2^-1 (Section 4.2, eq. (4.1)).
 template <int D, class R>
-__device__ __forceinline__ void times_w2(const KParams& p, const R* M, R* out) {
+__device__ __forceinline__ void times_w2(const KBase& p, const R* M, R* out) {
 #pragma unroll
   for (int a = 0; a < D; ++a)
 #pragma unroll
@@ -145,7 +145,7 @@ __device__ __forceinline__ bool metric_dP(int id, const R* T, const R* dT, R* S)
 template <int D, int N, int Q1, class R, int OP, bool WIDE>
 __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP, WIDE>::WARPS * ElemCfg<D, N, Q1, R, OP, WIDE>::GT,
                                   ElemCfg<D, N, Q1, R, OP, WIDE>::MINB)
-    elem_kernel(const KParams p) {
+    elem_kernel(const typename KArg<R>::type p) {
   using Cfg = ElemCfg<D, N, Q1, R, OP, WIDE>;
   constexpr int NDOF = Shape<D, N, Q1>::NDOF, QP = Shape<D, N, Q1>::QP, DD = D * D;
   constexpr int WARPS = Cfg::WARPS, GT = Cfg::GT;   // elements per block, threads per element
@@ -587,7 +587,7 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP, WIDE>::WARPS * ElemCf
           else H[(size_t)i * QP] = ok ? v : R(0);
         };
         MetricLin<D, R> L;
-        const bool lin = p.metric != 302 && !metric_dual<R>(p.metric);
+        const bool lin = sizeof(R) == 4 ? !metric_dual<R>(p.metric) : p.metric != 302;
         if (lin) ok = L.init(p.metric, T);
         if constexpr (D == 3 && sizeof(R) == 8) {
           if (!lin && p.wkind == WK_IDENTITY && !p.metric2) {

@@ -277,7 +277,7 @@ __device__ __forceinline__ void pac_adj(const float2 (&tBG)[Q1 * N], float* P0, 
 // issue and leaves the FP64 pipe mostly idle, so one F2F beats the ~20
 // integer instructions of f64_to_f32.
 template <int N, int NT, bool IO32>
-__device__ __forceinline__ void fetch_v(const KParams& p, const NodeMap<N>& m, int lane, float (&v)[NT][3],
+__device__ __forceinline__ void fetch_v(const KBase& p, const NodeMap<N>& m, int lane, float (&v)[NT][3],
                                         unsigned& fmask) {
   constexpr int NDOF = N * N * N;
   fmask = 0u;
@@ -360,7 +360,7 @@ __device__ __forceinline__ void pac_point(const float (&h)[kCompactRec], const f
 // IO32: v and y are the FP32 vectors p.v32, p.y32 (FP32 atomics into y).
 // For n = 4 the kernel is held to 128 registers, two blocks per SM (0: no bound).
 template <int N, int Q1, bool IDENT, bool IO32>
-__global__ void __launch_bounds__(kPacWarps * 32, N == 4 ? 2 : 0) pac_kernel(const KParams p) {
+__global__ void __launch_bounds__(kPacWarps * 32, N == 4 ? 2 : 0) pac_kernel(const KBase p) {
   using Cfg = PacCfg<N, Q1>;
   using L = typename Cfg::L;
   constexpr int NDOF = Cfg::NDOF, QP = Cfg::QP, NT = Cfg::NT, NPL = Cfg::NPL;
@@ -377,7 +377,7 @@ __global__ void __launch_bounds__(kPacWarps * 32, N == 4 ? 2 : 0) pac_kernel(con
   const float* rec = static_cast<const float*>(p.pa);
   const int stride = gridDim.x * kPacWarps;
   // elements ei = warp slot + k stride: all elements, or one colour's list
-  // (deterministic sums: one add per node and launch, see KParams)
+  // (deterministic sums: one add per node and launch, see KBase)
   const int ecount = p.elist ? p.ecount : p.nelem;
   auto elem = [&](int i) { return p.elist ? __ldg(p.elist + i) : i; };
   int ei = blockIdx.x * kPacWarps + warp;
@@ -494,7 +494,7 @@ struct PacrCfg {
 
 // x at the nodes this lane gathers, relative to the element's first node
 template <int N, int NT>
-__device__ __forceinline__ void fetch_x(const KParams& p, const NodeMap<N>& m, int lane, float (&xr)[NT][3]) {
+__device__ __forceinline__ void fetch_x(const KBase& p, const NodeMap<N>& m, int lane, float (&xr)[NT][3]) {
   constexpr int NDOF = N * N * N;
   const int g0 = m(0);
   double x0[3];
@@ -547,7 +547,7 @@ __device__ __forceinline__ void pacr_record(int metric, const float (&Wi)[9], co
 }
 
 template <int N, int Q1, bool IDENT, bool IO32>
-__global__ void __launch_bounds__(kPacrWarps * 32, N == 4 ? 2 : 1) pacr_kernel(const KParams p) {
+__global__ void __launch_bounds__(kPacrWarps * 32, N == 4 ? 2 : 1) pacr_kernel(const KBase p) {
   using Cfg = PacCfg<N, Q1>;
   using RC = PacrCfg<N, Q1>;
   using L = typename Cfg::L;
