@@ -185,6 +185,7 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP, WIDE>::WARPS * ElemCf
   constexpr int NKQ = (FXPA || (FX303 && OP != OP_ENERGY)) ? NKEY * QP : 1;
   __shared__ short s_kq[NKQ > 1 ? WARPS : 1][NKQ];   // exponents of the points' results
   __shared__ int s_key[NKQ > 1 ? WARPS : 1][GW * NKEY];
+  __shared__ unsigned s_thin[WARPS][GW];
   __shared__ unsigned s_mag[WARPS][GW * 2 * D];   // per warp and component: largest magnitudes of the group's warps
   R Wi[DD];
 #pragma unroll
@@ -300,11 +301,11 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP, WIDE>::WARPS * ElemCf
     if constexpr (FX) fx_group_exp<GT, Cfg::NC>(mag, em, s_mag[warp], bar);
     else __syncwarp();
     if constexpr (FX303) {
-      // one exponent for all components (at most 4 bits lost to one of them),
+      // one exponent for all components (at most 2 bits lost to one of them),
       // where the scalars stay inside the FP64 range (kFx303X)
       const int lo = min(em[0], min(em[1], em[2])), hi = max(em[0], max(em[1], em[2]));
       fx303 = p.metric == 303 && p.wkind == WK_IDENTITY && !p.metric2 &&
-              hi >= 1023 - kFx303X && hi <= 1023 + kFx303X && hi - lo <= 4;
+              hi >= 1023 - kFx303X && hi <= 1023 + kFx303X && hi - lo <= 2;
       if (fx303) em[0] = em[1] = em[2] = hi;
     }
     // ---- forward contraction: A (and dA) at every point
@@ -315,6 +316,7 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP, WIDE>::WARPS * ElemCf
       for (int f = 0;; ++f) {
         fwd3_fx<N, Q1, D, GT>(p.fx, em, P0, f == 0 ? P2 : P1, lane, bar);
         if (f) break;
+        if constexpr (FX303) fx303 = fx303 && !fx_thin<QP, GT>(reinterpret_cast<const fx_t*>(P2), s_thin[warp], lane, bar);
 #pragma unroll
         for (int c = 0; c < D; ++c) {
           mag[c] = 0;
@@ -354,8 +356,10 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP, WIDE>::WARPS * ElemCf
       if constexpr (FX) fwd2_fx<N, Q1, Cfg::NC, GT>(p.fx, em, P0, P1, lane, bar);
       else fwd2<N, Q1, Cfg::NC, R>(sB, sG, P0, P1, lane);
     } else {
-      if constexpr (FX) fwd3_fx<N, Q1, Cfg::NC, GT>(p.fx, em, P0, P1, lane, bar);
-      else fwd3_rb<N, Q1, Cfg::NC, R>(tB, tG, P0, P1, lane);
+      if constexpr (FX) {
+        fwd3_fx<N, Q1, Cfg::NC, GT>(p.fx, em, P0, P1, lane, bar);
+        if constexpr (FX303) fx303 = fx303 && !fx_thin<QP, GT>(reinterpret_cast<const fx_t*>(P1), s_thin[warp], lane, bar);
+      } else fwd3_rb<N, Q1, Cfg::NC, R>(tB, tG, P0, P1, lane);
     }
     R* Abuf = Cfg::SPLIT ? P2 : ((D == 2) ? P0 : P1);     // A: [D][D][QP]
     R* dAbuf = Cfg::SPLIT ? P1 : Abuf + DD * QP;         // dA (Hessian action)

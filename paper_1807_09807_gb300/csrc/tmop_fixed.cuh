@@ -498,12 +498,44 @@ __device__ __forceinline__ void adj2_fx(const FxTab& T, const int (&em)[NC], dou
 // is r times smaller than the element's largest one would lose r^2 of the
 // cofactors and r^3 of det T to that one's scale (order-3 hexes graded to r =
 // 100: det T to 5e-10).
+__device__ __forceinline__ unsigned fx_word(fx_t y) { return (unsigned)((int)(y >> 32) ^ ((int)(y >> 32) >> 31)); }
 template <int ST>
 __device__ __forceinline__ int fx_room(const fx_t* T) {
   unsigned top = 0;   // (the same leading bit as the largest magnitude)
 #pragma unroll
-  for (int i = 0; i < 9; ++i) top |= (unsigned)((int)(T[i * ST] >> 32) ^ ((int)(T[i * ST] >> 32) >> 31));
+  for (int i = 0; i < 9; ++i) top |= fx_word(T[i * ST]);
   return max(__clz((int)top) - 5, 0);
+}
+
+// Whether T at one of the group's points has a row or a column more than about
+// four times smaller than its largest entry, which sends the element to the
+// FP64 stage: products of the small entries of an element long in one direction
+// (aspect r) lose r^2 to the scale of the long ones, where FP64 loses r to the
+// map (order-3 hexes of aspect 1000: gradient to 2e-11 in fixed point, 4e-13 in
+// FP64). The test takes 2 % of the gradient's time. s: a word per warp of the
+// group, rewritten only after a later barrier of the group.
+template <int ST, int GT>
+__device__ __forceinline__ bool fx_thin(const fx_t* T, unsigned* s, int lane, int bar) {
+  bool thin = false;
+  for (int q = lane; q < ST; q += GT) {
+    unsigned w[6] = {};   // rows, columns
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+      const unsigned m = fx_word(T[i * ST + q]);
+      w[i / 3] |= m;
+      w[3 + i % 3] |= m;
+    }
+    const unsigned least = min(min(min(w[0], w[1]), min(w[2], w[3])), min(w[4], w[5]));
+    thin |= least < (w[0] | w[1] | w[2]) >> 2;
+  }
+  thin = __any_sync(group_mask<GT>(), thin);
+  if constexpr (GT > 32) {
+    if ((threadIdx.x & 31) == 0) s[(threadIdx.x >> 5) % (GT / 32)] = thin;
+    group_sync<GT>(bar);
+#pragma unroll
+    for (int w = 0; w < GT / 32; ++w) thin |= s[w] != 0;
+  }
+  return thin;
 }
 
 // mu303 at one point in fixed point (W = I): s P (GRAD, in place of T) and s dP
