@@ -165,7 +165,7 @@ int tmop_gradient_hess_apply(tmop_ctx* ctx, const double* x, const double* v, do
  * (dim^2 (dim^2 + 1) / 2 values per point, FP64 under TMOP_FP64 and FP32
  * under the FP32 forms) in the context (allocated on first use:
  * nelem * Q * 45 * 8 bytes for order-k hexes in FP64, and 8 bytes per point
- * of exponents: a 3D FP64 context keeps each value as a signed 60-bit integer
+ * of exponents: a 3D FP64 context keeps each value as a signed 58-bit integer
  * in two 32-bit limbs, scaled by powers of two of its point). A 3D FP32 context
  * whose metric is written in |T|^2 and det T (1, 14, 303), with a constant
  * target and no second term, stores instead 14 values per point from which

@@ -243,10 +243,11 @@ void launch_dst(const R* A, const R* B, R* C, int M, int N, int Kd, int batch, s
   k_dst<R, T, P, KC, KS><<<g, (T / P) * (T / P) * KS, 0, s>>>(A, B, C, M, N, Kd, batch, sAb, lda, sBb, ldb, sCb, ldc);
 }
 
-// The tile by the number of 64 x 64 tiles. With 60 or more of them (47^3
-// coarse vertices: 104 to 141) the 64 tile's fewer loads per multiply-add
-// win: two-level FP32 Newton on 48^3 order-3 hexes 89.6 ms against 92.3 ms
-// with 32 tiles. A small coarse grid leaves one or two 64 tiles, i.e. one or
+// The tile by the number of 64 x 64 tiles. With 60 or more of them the 64
+// tile's fewer loads per multiply-add win in FP32: us per two-level MINRES
+// iteration on 320^2, 380^2 and 440^2 order-1 quads (50, 72, 98 tiles) 14.5,
+// 17.6, 21.0 with 64 tiles, 14.7, 22.6, 31.5 with 8 (FP64: 133, 160, 189
+// against 54, 85, 126). A small coarse grid leaves one or two 64 tiles, i.e. one or
 // two of 152 SMs, whose FP64 pipe (2 operations per clock) then bounds the
 // transform: 63^2 vertices, FP64, 71 us. 8 tiles (128 blocks) of four thread
 // groups take 2.4 us, and one iteration of the two-level FP64 solve on 64^2

@@ -1,4 +1,4 @@
-// Fused TMOP element kernel: one warp per element.
+// Fused TMOP element kernel: one group of threads (16, 32 or 64) per element.
 //
 //   gather  x (and v) of the element's n^d nodes into shared memory
 //   forward A(q) = sum_i x_i grad phi_i(q)            (eq. (2.2), sum factorised)
@@ -59,10 +59,8 @@ struct ElemCfg {
   // blocks per SM as shared memory holds: the contractions run on the integer
   // pipes beside the FP64 pipe, and with one warp per element only 2-3 warps
   // per scheduler hide their latency (48^3 order-3 hexes, gradient + Hessian
-  // action: 8.30 ms with one warp, 6.87 ms with two, 5.53 ms with one copy of
-  // the forward map's code for x and v, which took the misses of the
-  // instruction cache down). In 2D a stage has 6 to 24 lines, one per thread:
-  // on meshes that fill the chip (WIDE) half a warp per element leaves fewer
+  // action: 8.30 ms with one warp, 6.87 with two). In 2D a stage has 6 to 24 lines, one per thread:
+  // on meshes that fill the chip (WIDE, use_wide) half a warp per element leaves fewer
   // of them idle (150 x 117 order-4 quads, 6^2 points, gradient + Hessian
   // action: 266 us with a warp, 195 us with half, 197 us with a quarter); on
   // small ones, where an element's latency counts, a warp is faster (8^2
@@ -78,11 +76,11 @@ struct ElemCfg {
   static constexpr int FIT = 200 * 1024 / PER_WARP;
   static constexpr int WARPS = GT == 64 ? 1 : (TWO ? 6 : (FIT >= 8 ? 8 : (FIT < 1 ? 1 : FIT)));
   // Blocks per SM that bound the registers (0: no bound): 6 (168 registers)
-  // for the kernels that hold T and dT, 7 or 8 (128) for the others. 48^3
-  // order-3 hexes (5 points per axis), gradient + Hessian action: 4.61 ms with
-  // 8 (spills), 3.83 with 6, 3.70 with 5; 32^3 order 2 (4 points) 0.54-0.59
-  // with 6; 24^3, stored-Hessian product 227 us with 8, 242 with 10; energy +
-  // gradient 232 us with 9, 227 with 7.
+  // for the kernels that hold T and dT, 7 or 8 (128) for the others; 5 for the
+  // one-pass kernel at 5 points per axis, where 6 spills. 48^3 order-3 hexes (5
+  // points per axis), gradient + Hessian action: 4.61 ms with 8, 3.83 with 6,
+  // 3.70 with 5; 24^3, stored-Hessian product 227 us with 8, 242 with 10; energy
+  // + gradient 232 us with 9, 227 with 7.
   static constexpr int WANT = HV ? (OP == OP_GRAD_HESS && Q1 == 5 ? 5 : 6) : (OP == OP_HESS_PA ? 8 : 7);
   static constexpr int MINB = GT == 64 ? (FIT >= WANT ? WANT : FIT) : (TWO ? 2 : 0);
   // after the 1D tables: the product weight w_q0 w_q1 (w_q2) of every point
@@ -1036,10 +1034,12 @@ int prepare_elem_impl(int nelem, int* grid) {
   return 0;
 }
 
-// The WIDE form where it exists and every SM has a full block (8 elements).
+// The WIDE form where it exists and every one of GB300's 152 SMs has a full
+// block of 8 elements (a constant, so that prepare and launch agree).
+constexpr int kWideElements = 152 * 8;
 template <int D, int N, int Q1, class R, int OP>
 bool use_wide(int nelem) {
-  return ElemCfg<D, N, Q1, R, OP>::HAS_WIDE && nelem >= 1216;
+  return ElemCfg<D, N, Q1, R, OP>::HAS_WIDE && nelem >= kWideElements;
 }
 
 template <int D, int N, int Q1, class R, int OP>

@@ -40,8 +40,7 @@ struct Grid2 {
   }
 };
 
-// one warp per patch
-// One warp per element, the order a template parameter (the digits of a
+// One warp per element (its patch), the order a template parameter (the digits of a
 // feature's index then cost no run-time division) and the uniform patch's
 // positions in a table: GB300's FP64 pipe (2 operations per SM and clock, the
 // conversions among them) bounds this kernel, and the feature itself takes two
