@@ -183,7 +183,6 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP, WIDE>::WARPS * ElemCf
   constexpr int NKQ = (FXPA || (FX303 && OP != OP_ENERGY)) ? NKEY * QP : 1;
   __shared__ short s_kq[NKQ > 1 ? WARPS : 1][NKQ];   // exponents of the points' results
   __shared__ int s_key[NKQ > 1 ? WARPS : 1][GW * NKEY];
-  __shared__ unsigned s_thin[WARPS][GW];
   __shared__ unsigned s_mag[WARPS][GW * 2 * D];   // per warp and component: largest magnitudes of the group's warps
   R Wi[DD];
 #pragma unroll
@@ -314,7 +313,6 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP, WIDE>::WARPS * ElemCf
       for (int f = 0;; ++f) {
         fwd3_fx<N, Q1, D, GT>(p.fx, em, P0, f == 0 ? P2 : P1, lane, bar);
         if (f) break;
-        if constexpr (FX303) fx303 = fx303 && !fx_thin<QP, GT>(reinterpret_cast<const fx_t*>(P2), s_thin[warp], lane, bar);
 #pragma unroll
         for (int c = 0; c < D; ++c) {
           mag[c] = 0;
@@ -354,10 +352,8 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP, WIDE>::WARPS * ElemCf
       if constexpr (FX) fwd2_fx<N, Q1, Cfg::NC, GT>(p.fx, em, P0, P1, lane, bar);
       else fwd2<N, Q1, Cfg::NC, R>(sB, sG, P0, P1, lane);
     } else {
-      if constexpr (FX) {
-        fwd3_fx<N, Q1, Cfg::NC, GT>(p.fx, em, P0, P1, lane, bar);
-        if constexpr (FX303) fx303 = fx303 && !fx_thin<QP, GT>(reinterpret_cast<const fx_t*>(P1), s_thin[warp], lane, bar);
-      } else fwd3_rb<N, Q1, Cfg::NC, R>(tB, tG, P0, P1, lane);
+      if constexpr (FX) fwd3_fx<N, Q1, Cfg::NC, GT>(p.fx, em, P0, P1, lane, bar);
+      else fwd3_rb<N, Q1, Cfg::NC, R>(tB, tG, P0, P1, lane);
     }
     R* Abuf = Cfg::SPLIT ? P2 : ((D == 2) ? P0 : P1);     // A: [D][D][QP]
     R* dAbuf = Cfg::SPLIT ? P1 : Abuf + DD * QP;         // dA (Hessian action)
@@ -385,6 +381,13 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP, WIDE>::WARPS * ElemCf
     // adjoint map takes (OP_GRAD_HESS: the gradient's, then the Hessian action's)
     unsigned rmag[FX ? 2 * D : 1] = {};
     constexpr int NS = DD * (DD + 1) / 2;
+    // the exponents of a point's results in fixed point (k: 0 the gradient's
+    // fields, NKEY - 1 the Hessian action's)
+    auto record = [&](int k, int q, const FxPoint& pt) {
+      key[k] = max(key[k], fx_point_key(pt));
+      s_kq[warp][k * QP + q] = (short)(pt.zero() ? -16000 : pt.E);
+    };
+    unsigned thin_pts = 0;   // the thread's points of a fixed-point element that took the FP64 stage
     for (int q = lane; q < QP; q += GT) {
       if constexpr (OP == OP_HESS_PA) {
         // y = H dA with the stored symmetric A-space Hessian (already scaled by w det W)
@@ -432,19 +435,25 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP, WIDE>::WARPS * ElemCf
         continue;
       }
       if constexpr (FX303) {
+        fx_t* Tq = reinterpret_cast<fx_t*>(Abuf) + q;
+        int up = 0;
+        bool thin = true;
         if (fx303) {
-          FxPoint pt[2];   // of the gradient's fields, of the Hessian action's
+          // (one choice per warp: a warp that took both stages would pay for both;
+          // the lanes of the last points alone)
+          const int n = QP - (q - (int)(threadIdx.x & 31));
+          thin = __any_sync(n < 32 ? (1u << n) - 1u : 0xffffffffu, fx_thin<QP>(Tq, up));
+          if (OP == OP_GRAD_HESS && thin) thin_pts |= 1u << (q / GT);
+        }
+        if (!thin) {
+          FxPoint pt[2];
           double mu, tau;
           const double s = sWq[q] * p.detW;
           const bool ok = fx_point303<QP, GRADLIKE || OP == OP_GRAD_HESS, Cfg::HV>(
-              reinterpret_cast<fx_t*>(Abuf) + q, reinterpret_cast<fx_t*>(dAbuf) + q, sA[0].kb, sV[0].kb, s, pt[0],
-              pt[NKEY - 1], mu, tau);
+              Tq, reinterpret_cast<fx_t*>(dAbuf) + q, up, sA[0].kb, sV[0].kb, s, pt[0], pt[NKEY - 1], mu, tau);
           if constexpr (OP != OP_ENERGY) {
 #pragma unroll
-            for (int k = 0; k < NKEY; ++k) {
-              key[k] = max(key[k], fx_point_key(pt[k]));
-              s_kq[warp][k * QP + q] = (short)(pt[k].zero() ? -16000 : pt[k].E);
-            }
+            for (int k = 0; k < NKEY; ++k) record(k, q, pt[k]);
           }
           if constexpr (EG || OP == OP_ENERGY) {
             emin = fmin(emin, tau);
@@ -871,7 +880,21 @@ __global__ void __launch_bounds__(ElemCfg<D, N, Q1, R, OP, WIDE>::WARPS * ElemCf
               }
           }
         }
+        if constexpr (FX303) {
+          if (fx303) record(0, q, fx_point_pack<QP>(Rbuf + q));
+        }
       }
+    }
+    if constexpr (FX303 && OP == OP_GRAD_HESS) {
+      // (after the loop, which then keeps its registers for the metrics: 32^3
+      // order-2 hexes with mu98 782 us with the packing inside, 765 so; for the
+      // other operations inside: 48^3 order-3 gradient 1.73 ms after it, 1.65 so)
+#pragma unroll 1
+      for (int q = lane; thin_pts; q += GT, thin_pts >>= 1)
+        if (thin_pts & 1u) {
+          record(0, q, fx_point_pack<QP>(Abuf + q));
+          record(NKEY - 1, q, fx_point_pack<QP>(dAbuf + q));
+        }
     }
     if constexpr (OP == OP_LINEARIZE || OP == OP_LINEARIZE_C) {
       group_sync<GT>(bar);

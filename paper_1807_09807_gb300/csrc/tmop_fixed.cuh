@@ -507,35 +507,26 @@ __device__ __forceinline__ int fx_room(const fx_t* T) {
   return max(__clz((int)top) - 5, 0);
 }
 
-// Whether T at one of the group's points has a row or a column more than about
-// four times smaller than its largest entry, which sends the element to the
-// FP64 stage: products of the small entries of an element long in one direction
-// (aspect r) lose r^2 to the scale of the long ones, where FP64 loses r to the
-// map (order-3 hexes of aspect 1000: gradient to 2e-11 in fixed point, 4e-13 in
-// FP64). The test takes 2 % of the gradient's time. s: a word per warp of the
-// group, rewritten only after a later barrier of the group.
-template <int ST, int GT>
-__device__ __forceinline__ bool fx_thin(const fx_t* T, unsigned* s, int lane, int bar) {
-  bool thin = false;
-  for (int q = lane; q < ST; q += GT) {
-    unsigned w[6] = {};   // rows, columns
+// Bits to shift a point's T up by (up), and whether it has a row or a column
+// more than about four times smaller than its largest entry, which sends the
+// point to the FP64 stage (fx_point_pack): products of the small entries of an
+// element long in one direction (aspect r) lose r^2 to the scale of the long
+// ones, where FP64 loses r to the map (order-3 hexes of aspect 1000: gradient to
+// 2e-11 in fixed point, 4e-13 in FP64). Point by point and not by the element:
+// 16^3 order-4 hexes with nodes moved by a tenth of their spacing, gradient +
+// Hessian action 328 us, 390 with the whole element in FP64, 291 without the test.
+template <int ST>
+__device__ __forceinline__ bool fx_thin(const fx_t* T, int& up) {
+  unsigned w[6] = {};   // rows, columns
 #pragma unroll
-    for (int i = 0; i < 9; ++i) {
-      const unsigned m = fx_word(T[i * ST + q]);
-      w[i / 3] |= m;
-      w[3 + i % 3] |= m;
-    }
-    const unsigned least = min(min(min(w[0], w[1]), min(w[2], w[3])), min(w[4], w[5]));
-    thin |= least < (w[0] | w[1] | w[2]) >> 2;
+  for (int i = 0; i < 9; ++i) {
+    const unsigned m = fx_word(T[i * ST]);
+    w[i / 3] |= m;
+    w[3 + i % 3] |= m;
   }
-  thin = __any_sync(group_mask<GT>(), thin);
-  if constexpr (GT > 32) {
-    if ((threadIdx.x & 31) == 0) s[(threadIdx.x >> 5) % (GT / 32)] = thin;
-    group_sync<GT>(bar);
-#pragma unroll
-    for (int w = 0; w < GT / 32; ++w) thin |= s[w] != 0;
-  }
-  return thin;
+  const unsigned top = w[0] | w[1] | w[2];
+  up = max(__clz((int)top) - 5, 0);
+  return min(min(min(w[0], w[1]), min(w[2], w[3])), min(w[4], w[5])) < top >> 2;
 }
 
 // mu303 at one point in fixed point (W = I): s P (GRAD, in place of T) and s dP
@@ -572,10 +563,10 @@ struct FxPoint {
 constexpr int kFx303X = 40, kFx303V = 610;
 constexpr int kFxNan = 32000;   // E of a point whose results are not finite
 template <int ST, bool GRAD, bool HESS>
-__device__ __forceinline__ bool fx_point303(fx_t* T, fx_t* V, int kT, int kV, double s, FxPoint& pg, FxPoint& ph,
-                                            double& mu, double& tau) {
+__device__ __forceinline__ bool fx_point303(fx_t* T, fx_t* V, int upT, int kT, int kV, double s, FxPoint& pg,
+                                            FxPoint& ph, double& mu, double& tau) {
   Limbs a[9], c[9], v[HESS ? 9 : 1];
-  const int upT = fx_room<ST>(T), upV = HESS ? fx_room<ST>(V) : 0;
+  const int upV = HESS ? fx_room<ST>(V) : 0;
   kT -= upT;
   kV -= upV;
   const int kC = 2 * kT + 60 - 1023;
@@ -665,6 +656,25 @@ __device__ __forceinline__ bool fx_point303(fx_t* T, fx_t* V, int kT, int kV, do
     if (!finite) ph = {kFxNan, 1u << 30};
   }
   return ok;
+}
+
+// A point's nine results from the FP64 stage, in place: doubles to integers
+// below 2^59 under one exponent, as fx_point303 leaves them.
+template <int ST>
+__device__ __forceinline__ FxPoint fx_point_pack(double* R) {
+  unsigned m = 0;
+#pragma unroll
+  for (int i = 0; i < 9; ++i) m = max(m, fx_mag(R[i * ST]));
+  const int e = fx_floor(m >> 20);
+  FxPoint pt = {e + 2044 - 1022 - 59};
+#pragma unroll
+  for (int i = 0; i < 9; ++i) {
+    const fx_t y = fx_from_f64(R[i * ST], e, 6);
+    reinterpret_cast<fx_t*>(R)[i * ST] = y;
+    pt.add(y);
+  }
+  if (fx_nan(e)) pt = {kFxNan, 1u << 30};
+  return pt;
 }
 
 // Largest values of NK keys over the group, with a barrier (as fx_group_exp).
