@@ -686,8 +686,9 @@ def run_ours(args):
         if prec == tm.FP64:
             r["work"] = ("flops_per_launch: the plain sum-factorised contractions + the metric terms in FP64 (the "
                          "algorithmic work). The kernel runs the contractions (and mu303's pointwise terms with "
-                         "W = I) in 64-bit fixed point on the integer multiply-add units, to no larger an error, "
-                         "so frac against the FP64 peak can exceed 1; it is bound by instruction issue")
+                         "W = I and elements of moderate aspect) in 64-bit fixed point on the integer multiply-add "
+                         "units, so the FP64 peak is not its bound and frac can exceed 1: it is bound by "
+                         "instruction issue and latency (profiles/elem_kernel_gradhess_c4_fp64.md)")
         tr = traffic.get(f"{args.workload}:{args.precision}" + (":fused" if one_pass else ""))
         # only counters taken on the kernel sources as they are now
         if tr and tr.get("kernel_src_sha256") == kernel_src_hash():

@@ -12,7 +12,7 @@
 // largest value). The same holds for the products of matrix entries in the
 // pointwise stage of mu303 (fx_point303) where T's entries are of one size, of
 // which only the scalars stay in FP64. 48^3 order-3 hexes, gradient + Hessian
-// action: 11.13 ms with FP64 contractions, 5.53 ms with these, 3.81 ms with the
+// action: 11.13 ms with FP64 contractions, 5.53 ms with these, 3.82 ms with the
 // pointwise products too (FP64 instructions per element and warp 1490, 654, 98).
 //
 // Numbers: a value v of a component whose largest magnitude is below 2^E is
