@@ -492,13 +492,15 @@ __device__ __forceinline__ void adj2_fx(const FxTab& T, const int (&em)[NC], dou
   group_sync<GT>(bar);
 }
 
+// High word of a value's magnitude (of its complement for a negative one).
+__device__ __forceinline__ unsigned fx_word(fx_t y) { return (unsigned)((int)(y >> 32) ^ ((int)(y >> 32) >> 31)); }
+
 // Bits to shift the nine entries of a point up by: to |entries| < 2^59 by the
 // largest one, or none (< 2^59.4 by fx_tables). By the point's own largest
 // entry: products of entries have a fixed number of bits, so at a point whose T
 // is r times smaller than the element's largest one would lose r^2 of the
 // cofactors and r^3 of det T to that one's scale (order-3 hexes graded to r =
-// 100: det T to 5e-10).
-__device__ __forceinline__ unsigned fx_word(fx_t y) { return (unsigned)((int)(y >> 32) ^ ((int)(y >> 32) >> 31)); }
+// 100: det T to 1e-11).
 template <int ST>
 __device__ __forceinline__ int fx_room(const fx_t* T) {
   unsigned top = 0;   // (the same leading bit as the largest magnitude)
